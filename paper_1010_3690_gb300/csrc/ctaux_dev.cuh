@@ -272,26 +272,45 @@ __device__ __forceinline__ float g0_eval_f(const Chain<T>& c, int spin, float ti
 constexpr int kMaxChains = 2048;
 
 __device__ __forceinline__ void block_exclusive_scan(int* a, int n) {
-  // a[0..n] in shared memory; on return a[i] = sum_{k<i} a_k, a[n] = total
-  __shared__ int part[1024];
-  const int nt = blockDim.x, t = threadIdx.x;
+  // a[0..n] in shared memory; on return a[i] = sum_{k<i} a_k, a[n] = total.
+  // Every persistent kernel starts with it, so its latency is paid a dozen
+  // times per block: one chain needs no scan, more take warp shuffles (a
+  // serial pass over the threads' partial sums costs about 5 us per launch).
+  const int nt = blockDim.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
+  if (n == 1) {
+    if (t == 0) {
+      a[1] = a[0];
+      a[0] = 0;
+    }
+    __syncthreads();
+    return;
+  }
+  __shared__ int wsum[32];
   const int per = (n + nt - 1) / nt;
   const int lo = min(n, t * per), hi = min(n, lo + per);
   int sum = 0;
   for (int i = lo; i < hi; ++i) sum += a[i];
-  part[t] = sum;
+  int incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) wsum[w] = incl;
   __syncthreads();
-  if (t == 0) {
-    int run = 0;
-    for (int i = 0; i < nt; ++i) {
-      const int v = part[i];
-      part[i] = run;
-      run += v;
+  if (w == 0) {
+    const int own = lane < (nt >> 5) ? wsum[lane] : 0;
+    int x = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += v;
     }
-    a[n] = run;
+    wsum[lane] = x - own;
+    if (lane == 31) a[n] = x;
   }
   __syncthreads();
-  int run = part[t];
+  int run = wsum[w] + incl - sum;
   for (int i = lo; i < hi; ++i) {
     const int v = a[i];
     a[i] = run;
