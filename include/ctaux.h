@@ -119,12 +119,12 @@ typedef struct {
                                          measurement is launched as one CUDA graph, captured
                                          on a private stream at first use; direct launches
                                          while profiling is on, or if capture fails */
-  int refresh_df64;                   /* mixed form: 1 = the periodic from-scratch recomputation
-                                         eliminates in double-float arithmetic (two float32,
-                                         about 48 significand bits) on the float32 pipe, which
-                                         GB300 runs 64x faster than float64; 0 = float64.  The
-                                         matrix N^{-1} is built in float64 either way, and the
-                                         near-tie fallback always eliminates in float64 */
+  int refresh_df64;                   /* mixed form: accepted for either value, without effect.  Every
+                                         from-scratch recomputation eliminates in float64
+                                         accuracy on the tensor cores (sliced float16 products),
+                                         which is faster than the double-float elimination that
+                                         1 used to select; the near-tie fallback eliminates on
+                                         the float64 pipe */
   int meas_bin_size;                  /* measurements per bin of the binned error of
                                          ctaux_measure_G; 0 = 16 */
   int n_matsubara;                    /* 0 = off; 1..64: every measurement also evaluates

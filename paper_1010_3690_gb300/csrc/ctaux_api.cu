@@ -192,19 +192,10 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
     ls.tie_iters = P.tie_refine_iters == 0 ? 12 : std::max(0, P.tie_refine_iters);
   }
   std::vector<TcMaps> host_maps(mixed_tc ? 2 * ctx->chains.size() : 0);
-  ls.refresh_df64 = (sizeof(T) == 4 && P.refresh_df64) ? 1 : 0;
-  // refresh grid: every resident CTA, except when even a refresh of every chain
-  // at its capacity is small (at most 4096 trailing-update tiles of 32 x 32 per
-  // panel): then its ~35 grid barriers per panel, not its work, set its time,
-  // and one CTA per SM makes each barrier shorter (measured: 0.081 -> 0.059 ms
-  // per block for one 2x2x2 chain at n ~ 400; 22 % slower at n ~ 2100)
-  int nb = refresh_blocks_per_sm<T>(ls.refresh_df64 != 0);
-  long long cap_tiles = 0;
-  for (const auto& cp : ctx->chains) {
-    const long long tb = (cp.capacity + cp.k_max + 31) / 32;
-    cap_tiles += 2 * tb * tb;
-  }
-  ls.refresh_grid = (cap_tiles <= 4096 ? 1 : std::max(1, nb)) * ctx->sm_count;
+  // from-scratch recomputation: launch shapes for all chains and for one
+  CUDA_TRY(ctx, inv_configure(2, max_ld, ctx->sm_count, &ls.inv_one));
+  CUDA_TRY(ctx, inv_configure(items, max_ld, ctx->sm_count, &ls.inv_all));
+  std::vector<InvView> host_views(items);
 
   for (size_t ci = 0; ci < ctx->chains.size(); ++ci) {
     const ctaux_chain_params& cp = ctx->chains[ci];
@@ -319,6 +310,13 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
     c.used = dalloc<int8_t>(ctx, 2 * ld, &err);
     c.pcol = dalloc<int>(ctx, 2 * ld, &err);
     if (c.pcol) CUDA_TRY(ctx, cudaMemset(c.pcol, 0xFF, 2 * ld * sizeof(int)));
+    for (int spin = 0; spin < 2; ++spin) {
+      InvView& v = host_views[2 * ci + spin];
+      inv_layout(c.work + spin * refresh_work_one((int)ld), (int)ld, ls.inv_all.chunks, v);
+      v.perm = c.perm + spin * ld;
+      v.used = c.used + spin * ld;
+      v.pcol = c.pcol + spin * ld;
+    }
     c.pkeys = dalloc<unsigned long long>(ctx, 2 * ld, &err);
     c.work_drift = dalloc<double>(ctx, 3, &err);
     c.drift_limit = P.drift_limit;
@@ -360,6 +358,15 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
     d0.forced_t = -1;
     d0.guard_eff = c.tie_guard;
     CUDA_TRY(ctx, cudaMemcpy(c.dyn, &d0, sizeof(Dyn), cudaMemcpyHostToDevice));
+    for (int spin = 0; spin < 2; ++spin) host_views[2 * ci + spin].status = &c.dyn->status;
+  }
+  {
+    InvView* dv = dalloc<InvView>(ctx, items, &err);
+    ls.inv_orders = dalloc<int>(ctx, items, &err);
+    if (err != cudaSuccess)
+      return set_err(ctx, CTAUX_ENOMEM, "device allocation failed: %s", cudaGetErrorString(err));
+    CUDA_TRY(ctx, cudaMemcpy(dv, host_views.data(), items * sizeof(InvView), cudaMemcpyHostToDevice));
+    ls.inv_views = dv;
   }
   if (mixed_tc) {
     void* dm = nullptr;
@@ -421,9 +428,9 @@ ctaux_status read_dyn(ctaux_ctx* ctx, int chain, Dyn* out) {
 }
 
 template <typename T>
-ctaux_status do_refresh(ctaux_ctx* ctx, int only_chain, cudaStream_t st) {
+ctaux_status do_refresh(ctaux_ctx* ctx, int only_chain, int max_order, cudaStream_t st) {
   cudaError_t e = launch_refresh<T>(reinterpret_cast<Chain<T>*>(ctx->chains_dev), ctx->ls, only_chain,
-                                    st, ctx->timer);
+                                    max_order, st, ctx->timer);
   if (e != cudaSuccess) return set_err(ctx, CTAUX_ECUDA, "refresh launch: %s", cudaGetErrorString(e));
   return CTAUX_OK;
 }
@@ -519,7 +526,7 @@ ctaux_status do_sweeps(ctaux_ctx* ctx, int n_sweeps, int measure, cudaStream_t s
     if (e != cudaSuccess) return set_err(ctx, CTAUX_ECUDA, "block launch: %s", cudaGetErrorString(e));
     ctx->blocks_since_refresh += 1;
     if (ctx->params.refresh_every > 0 && ctx->blocks_since_refresh >= ctx->params.refresh_every) {
-      ctaux_status r = do_refresh<T>(ctx, -1, st);
+      ctaux_status r = do_refresh<T>(ctx, -1, ctx->max_ld, st);
       if (r != CTAUX_OK) return r;
       ctx->blocks_since_refresh = 0;
     }
@@ -737,8 +744,8 @@ ctaux_status ctaux_reset_measurements(ctaux_ctx* ctx) {
 ctaux_status ctaux_recompute(ctaux_ctx* ctx, double* drift_max_out) {
   if (!ctx) return CTAUX_EINVAL;
   FLUSH_PENDING(ctx);
-  ctaux_status r = is_mixed(ctx) ? do_refresh<float>(ctx, -1, ctx->last_stream)
-                                 : do_refresh<double>(ctx, -1, ctx->last_stream);
+  ctaux_status r = is_mixed(ctx) ? do_refresh<float>(ctx, -1, ctx->max_ld, ctx->last_stream)
+                                 : do_refresh<double>(ctx, -1, ctx->max_ld, ctx->last_stream);
   if (r != CTAUX_OK) return r;
   ctx->blocks_since_refresh = 0;
   r = ctaux_synchronize(ctx);
@@ -884,8 +891,8 @@ ctaux_status ctaux_set_config(ctaux_ctx* ctx, int chain, const double* tau, cons
   int sg = 1;
   d.sign = sg;
   CUDA_TRY(ctx, cudaMemcpy(dyn_of(ctx, chain), &d, sizeof(Dyn), cudaMemcpyHostToDevice));
-  ctaux_status r = is_mixed(ctx) ? do_refresh<float>(ctx, chain, ctx->last_stream)
-                                 : do_refresh<double>(ctx, chain, ctx->last_stream);
+  ctaux_status r = is_mixed(ctx) ? do_refresh<float>(ctx, chain, n, ctx->last_stream)
+                                 : do_refresh<double>(ctx, chain, n, ctx->last_stream);
   if (r != CTAUX_OK) return r;
   // the drift of this refresh compares N of the previous configuration with the
   // new one: it is not a drift of the chain

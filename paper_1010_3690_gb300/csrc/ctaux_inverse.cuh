@@ -1,0 +1,72 @@
+// Blocked Gauss-Jordan inversion in place, with partial pivoting, of many
+// matrices at once: the from-scratch recomputation of N and the inversion
+// entry point without allocation (kernels in ctaux_inverse.cu).
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace ctaux {
+
+// One matrix and its work area (device pointers).
+struct InvView {
+  double* X;            // the matrix, column-major, leading dimension ld
+  int ld;
+  int chunks;           // images per row block: 1, or 4 (panels of 128 columns in two levels)
+  unsigned char* As;    // slice images of the panel's columns: ceil(ld / 128) x chunks x oz::kImageA
+  unsigned char* Bs;    // slice images of the pivot rows: ceil(ld / 64) x chunks x oz::kImageB
+  int* ea;              // row exponents of the images
+  int* eb;
+  int* perm;            // pivot row of each column
+  int8_t* used;         // row already pivoted
+  int* pcol;            // column at which a row was pivoted, -1 if not yet
+  double* piv;          // pivots, in column order
+  int* status;          // DS_SINGULAR and DS_TIMEOUT bits
+};
+
+// Panels of 128 columns in two levels (see ctaux_inverse.cu) where the largest
+// leading dimension of a launch is at least this: the five extra launches per
+// 128 columns against three of four passes over the matrix.  One level against
+// two, ms per recomputation of one chain: 2.29 / 2.49 at order 700, 3.19 / 3.29
+// at 900, 4.44 / 4.46 at 1100, 6.51 / 6.23 at 1500, 10.9 / 9.6 at 2000 (leading
+// dimensions a quarter above the order).
+constexpr int kInvTwoLevel = 1408;
+inline int inv_chunks(int max_ld) { return max_ld >= kInvTwoLevel ? 4 : 1; }
+
+// Doubles of As, Bs, ea, eb and piv for a leading dimension (the matrix itself
+// comes first and takes ld^2 doubles).
+__host__ __device__ inline size_t inv_extra_doubles(int ld, int chunks = 4) {
+  const size_t lp = (size_t)((ld + 127) / 128 * 128);
+  return lp * (112 * (size_t)chunks + 2);   // 2 x 448 bytes of slices per chunk
+}
+__host__ __device__ inline void inv_layout(double* work, int ld, int chunks, InvView& v) {
+  const size_t lp = (size_t)((ld + 127) / 128 * 128), slices = lp * 448 * (size_t)chunks;
+  v.X = work;
+  v.ld = ld;
+  v.chunks = chunks;
+  unsigned char* p = reinterpret_cast<unsigned char*>(work + (size_t)ld * ld);
+  v.As = p;
+  v.Bs = p + slices;
+  v.ea = reinterpret_cast<int*>(p + 2 * slices);
+  v.eb = v.ea + lp;
+  v.piv = reinterpret_cast<double*>(v.eb + lp);
+}
+
+// Launch parameters of the inversion of up to `items` matrices of leading
+// dimension at most max_ld.
+struct InvShape {
+  int cluster;     // CTAs of a panel's cluster (16, 8 or 4)
+  int width;       // panel width (32; 16 or 8 where a panel would not fit)
+  int rows;        // panel rows per CTA at max_ld
+  int smem;        // dynamic shared memory of the panel kernel
+  int chunks;      // 4: two levels
+  int sm_count;
+};
+cudaError_t inv_configure(int items, int max_ld, int sm_count, InvShape* out);
+
+// Inverts the matrices views[0..items) of orders orders[0..items) (device; 0 =
+// leave out), none above max_order: afterwards inv[c][perm[j]] = X[perm[c]][j].
+// `used` must be zero and `pcol` -1 on entry.  Returns the kernels launched.
+int launch_inverse(const InvView* views, const int* orders, int items, int max_order,
+                   const InvShape& sh, cudaStream_t st, cudaError_t* err);
+
+}  // namespace ctaux

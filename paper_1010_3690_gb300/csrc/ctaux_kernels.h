@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "ctaux_dev.cuh"
+#include "ctaux_inverse.cuh"
 
 namespace ctaux {
 
@@ -89,13 +90,14 @@ struct LaunchShape {
   int persist_ctas;      // grid of the persistent batched kernels
   int tie_grid;          // cooperative grid of the near-tie refinement
   int tie_iters;         // most refinement iterations (0: every near tie takes the fallback)
-  int refresh_df64;      // float32 form: refresh elimination in double-float
   int prop_smem;
   int gamma_in_smem;
   int meas_lchunks;      // vertex chunks of the measurement evaluation
   int meas_cb_blocks;
   int meas_acc_blocks;   // one warp per (class, bin) output
-  int refresh_grid;
+  const InvView* inv_views;   // [chain][spin] matrices of the from-scratch recomputation (device)
+  int* inv_orders;            // [chain][spin] their orders, written by each recomputation
+  InvShape inv_all, inv_one;  // its launch shapes: every chain, one chain
   int use_tc;            // mixed form: flush on the tensor cores
   int tc_ctas;           // persistent grid of the tensor-core flush (one CTA per SM)
   int split_x_blocks;
@@ -170,9 +172,8 @@ template <typename T>
 cudaError_t configure_block_kernels(const LaunchShape& ls);
 template <typename T>
 int launch_gemm(Chain<T>* dchains, const LaunchShape& ls, int phase, cudaStream_t st);
-template <typename T>
-int refresh_blocks_per_sm(bool df);
 size_t refresh_work_doubles(int ld);
+size_t refresh_work_one(int ld);
 template <typename T>
 void launch_measure(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st, PhaseTimer* pt);
 // The measurement in two parts: the head (counters, G0 panels and the copy of
@@ -183,8 +184,8 @@ int launch_measure_head(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t s
 template <typename T>
 int launch_measure_tail(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st);
 template <typename T>
-cudaError_t launch_refresh(Chain<T>* dchains, const LaunchShape& ls, int only_chain,
-                           cudaStream_t st, PhaseTimer* pt, int filter = 0);
+cudaError_t launch_refresh(Chain<T>* dchains, const LaunchShape& ls, int only_chain, int max_order,
+                           cudaStream_t st, PhaseTimer* pt);   // max_order: no chain's order is above it
 // scratch: each chain's refresh work area (both spins)
 cudaError_t launch_tie_refine(Chain<float>* dchains, const LaunchShape& ls, cudaStream_t st);
 template <typename T>

@@ -1,80 +1,136 @@
-// From-scratch refresh kernels (bodies in ctaux_refresh.cuh): elimination in
-// float64, or in double-float on the float32 pipe (mixed form, optional).
-#include <type_traits>
-
+// From-scratch FP64 recomputation of N for every chain: build
+// N^{-1} = e^V - G0 (e^V - 1) (Eq. Nmatrix) of both spins from the
+// configuration, invert it (ctaux_inverse.cu), report the drift of the running
+// N and replace it.  Both precision forms eliminate in float64 accuracy on the
+// tensor cores, which is also the fastest form: the double-float elimination
+// that the mixed form offered as an option took 20 ms at n = 2085.
+#include "ctaux_inverse.cuh"
 #include "ctaux_refresh.cuh"
 
 namespace ctaux {
 
-template <typename T, typename E>
-__global__ void __launch_bounds__(256) k_refresh(Chain<T>* chains, int n_chains, int only_chain,
-                                                 int filter) {
-  refresh_body<T, E>(chains, n_chains, only_chain, filter);
+namespace {
+
+// Orders of the matrices (chain, spin) that take part: all chains, or one.
+template <typename T>
+__global__ void k_refresh_orders(const Chain<T>* chains, int n_chains, int only_chain, int* orders) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= 2 * n_chains) return;
+  const int ci = i >> 1;
+  const Dyn& d = *chains[ci].dyn;
+  const bool take = (only_chain < 0 || only_chain == ci) && !(d.status & ~DS_SINGULAR);
+  orders[i] = take ? d.n : 0;
 }
 
-// Small follow-up kernel: the stats of every refreshed chain.
+// N^{-1} into X, a column per CTA and unit.
 template <typename T>
-__global__ void k_refresh_finish(Chain<T>* chains, int n_chains, int only_chain, int filter) {
-  const int ci = (only_chain >= 0) ? only_chain : (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  if (ci >= n_chains) return;
-  if (only_chain >= 0 && (blockIdx.x | threadIdx.x)) return;
-  refresh_finish_one(chains[ci], filter);
-}
-
-template <typename T>
-cudaError_t launch_refresh(Chain<T>* dchains, const LaunchShape& ls, int only_chain,
-                           cudaStream_t st, PhaseTimer* pt, int filter) {
-  pt->begin(6, st);
-  int nch = ls.n_chains;
-  cudaError_t e = cudaSuccess;
-  void* args[] = {&dchains, &nch, &only_chain, &filter};
-  // double-float elimination only for the float32 form's own refreshes; the
-  // near-tie fallback (filter 1) keeps float64, whose N it also stores
-  const void* fn = (const void*)k_refresh<T, double>;
-  size_t dyn = 0;
-  if constexpr (std::is_same<T, float>::value)
-    if (ls.refresh_df64 && filter == 0) {
-      fn = (const void*)k_refresh<T, df64>;
-      dyn = refresh_dyn_smem<df64>();
+__global__ void __launch_bounds__(256) k_refresh_build(const Chain<T>* chains, const InvView* views,
+                                                       const int* orders, int items) {
+  __shared__ int off[2 * kMaxChains + 1];
+  for (int i = threadIdx.x; i < items; i += blockDim.x) off[i] = orders[i];
+  __syncthreads();
+  block_exclusive_scan(off, items);
+  const int total = off[items];
+  for (int u = blockIdx.x; u < total; u += gridDim.x) {
+    const int it = find_chain(off, items, u), j = u - off[it], m = orders[it], spin = it & 1;
+    const Chain<T>& c = chains[it >> 1];
+    const InvView& v = views[it];
+    const int buf = c.dyn->buf;
+    const double evj = c.ev[spin][c.s[buf][j] + 2], tj = c.tau[buf][j];
+    const int sj = c.site[buf][j];
+    if (threadIdx.x == 0) {
+      v.used[j] = 0;
+      v.pcol[j] = -1;
     }
-  e = cudaLaunchCooperativeKernel(fn, dim3(ls.refresh_grid), dim3(256), args, dyn, st);
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+      double x = -g0_eval(c, spin, c.tau[buf][i], c.site[buf][i], tj, sj) * (evj - 1.0);
+      if (i == j) x += evj;
+      v.X[(size_t)j * v.ld + i] = x;
+    }
+  }
+}
+
+// The inverse into N, with the drift; the pivot flags cleared for the next user.
+template <typename T>
+__global__ void __launch_bounds__(256) k_refresh_store(const Chain<T>* chains, const InvView* views,
+                                                       const int* orders, int items) {
+  __shared__ int off[2 * kMaxChains + 1];
+  __shared__ double red[3][8];
+  for (int i = threadIdx.x; i < items; i += blockDim.x) {
+    const bool ok = !(chains[i >> 1].dyn->status & ~DS_SINGULAR);   // no wait gave up
+    off[i] = ok ? orders[i] : 0;
+  }
+  __syncthreads();
+  block_exclusive_scan(off, items);
+  const int total = off[items];
+  for (int u = blockIdx.x; u < total; u += gridDim.x) {
+    const int it = find_chain(off, items, u), j = u - off[it];
+    const InvView& v = views[it];
+    if (threadIdx.x == 0) {
+      v.used[j] = 0;
+      v.pcol[j] = -1;
+    }
+    refresh_store_column(chains[it >> 1], it & 1, j, orders[it], v.X, (double*)nullptr, red);
+  }
+}
+
+// Log-determinants (sum of log|pivot|, in a fixed order) and the stats of
+// every refreshed chain, one CTA per chain.
+template <typename T>
+__global__ void __launch_bounds__(256) k_refresh_finish(const Chain<T>* chains, const InvView* views,
+                                                        const int* orders, int only_chain) {
+  const int ci = only_chain >= 0 ? only_chain : (int)blockIdx.x;
+  const Chain<T>& c = chains[ci];
+  if (c.dyn->status & ~DS_SINGULAR) return;
+  __shared__ double part[8];
+  for (int spin = 0; spin < 2; ++spin) {
+    const double* piv = views[2 * ci + spin].piv;
+    const int m = orders[2 * ci + spin];
+    double s = 0.0;
+    for (int k = threadIdx.x; k < m; k += blockDim.x) s += log(fabs(piv[k]));
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int w = 0; w < 8; ++w) t += part[w];
+      c.work_logdet[spin] = t;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) refresh_finish_one(c);
+}
+
+}  // namespace
+
+template <typename T>
+cudaError_t launch_refresh(Chain<T>* dchains, const LaunchShape& ls, int only_chain, int max_order,
+                           cudaStream_t st, PhaseTimer* pt) {
+  pt->begin(6, st);
+  const int items = 2 * ls.n_chains, nch = ls.n_chains;
+  k_refresh_orders<T><<<(items + 127) / 128, 128, 0, st>>>(dchains, nch, only_chain, ls.inv_orders);
+  // one chain: only its two matrices
+  const int first = only_chain >= 0 ? 2 * only_chain : 0, count = only_chain >= 0 ? 2 : items;
+  const InvView* views = ls.inv_views + first;
+  const int* orders = ls.inv_orders + first;
+  const Chain<T>* chains = dchains + first / 2;
+  k_refresh_build<T><<<ls.persist_ctas, 256, 0, st>>>(chains, views, orders, count);
+  cudaError_t e = cudaSuccess;
+  const int n = launch_inverse(views, orders, count, max_order, only_chain >= 0 ? ls.inv_one : ls.inv_all, st, &e);
   if (e == cudaSuccess) {
-    if (only_chain >= 0)
-      k_refresh_finish<T><<<1, 1, 0, st>>>(dchains, nch, only_chain, filter);
-    else
-      k_refresh_finish<T><<<(nch + 127) / 128, 128, 0, st>>>(dchains, nch, -1, filter);
+    k_refresh_store<T><<<ls.persist_ctas, 256, 0, st>>>(chains, views, orders, count);
+    k_refresh_finish<T><<<only_chain >= 0 ? 1 : nch, 256, 0, st>>>(dchains, ls.inv_views, ls.inv_orders, only_chain);
     e = cudaGetLastError();
   }
-  pt->end(6, st, 2);
+  pt->end(6, st, 4 + n);
   return e;
 }
 
-template <typename T>
-int refresh_blocks_per_sm(bool df) {
-  // with the double-float option the grid must be co-resident for either
-  // element type (the near-tie fallback keeps float64)
-  int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_refresh<T, double>, 256, 0);
-  if constexpr (std::is_same<T, float>::value) {
-    if (df) {
-      int nb2 = 0;
-      cudaFuncSetAttribute(k_refresh<T, df64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           refresh_dyn_smem<df64>());
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb2, k_refresh<T, df64>, 256,
-                                                    refresh_dyn_smem<df64>());
-      nb = nb < nb2 ? nb : nb2;
-    }
-  }
-  return nb;
-}
-
-template cudaError_t launch_refresh<double>(Chain<double>*, const LaunchShape&, int, cudaStream_t,
-                                            PhaseTimer*, int);
-template cudaError_t launch_refresh<float>(Chain<float>*, const LaunchShape&, int, cudaStream_t,
-                                           PhaseTimer*, int);
+template cudaError_t launch_refresh<double>(Chain<double>*, const LaunchShape&, int, int, cudaStream_t,
+                                            PhaseTimer*);
+template cudaError_t launch_refresh<float>(Chain<float>*, const LaunchShape&, int, int, cudaStream_t,
+                                           PhaseTimer*);
 size_t refresh_work_doubles(int ld) { return 2 * refresh_work_per_spin(ld); }
-
-template int refresh_blocks_per_sm<double>(bool);
-template int refresh_blocks_per_sm<float>(bool);
+size_t refresh_work_one(int ld) { return refresh_work_per_spin(ld); }
 
 }  // namespace ctaux

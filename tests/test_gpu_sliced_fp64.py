@@ -1,0 +1,43 @@
+"""Float64 products on the float16 tensor cores (sliced operands) at their edges.
+
+The tolerance is the one of the float64 parity tests (1e-10 of the matrix
+scale): a sliced product's error is below that of a chain of float64
+multiply-adds, and the oracle's N comes from a dense float64 inverse.
+"""
+import numpy as np
+import pytest
+
+from parity import oracle_for
+from workloads import configs
+
+pytestmark = pytest.mark.gpu
+
+pk = pytest.importorskip("paper_1010_3690_gb300")
+
+
+def _check_N(ctx, chains, cfgs):
+    for i, (ch, cfg) in enumerate(zip(chains, cfgs)):
+        oc = oracle_for(ch)
+        oc.set_config(cfg["tau"], cfg["site"], cfg["s"], cfg["birth"], cfg["t"])
+        st = ctx.stats(i)
+        for spin in (0, 1):
+            No = oc.N(spin)
+            np.testing.assert_allclose(ctx.get_N(i, spin), No, rtol=1e-10, atol=1e-10 * np.abs(No).max())
+            assert st["logdet"][spin] == pytest.approx(oc.slogdet(spin, oc.tau, oc.site, oc.s)[1],
+                                                       rel=1e-11, abs=1e-9)
+
+
+@pytest.mark.parametrize("orders,capacity", [
+    ((1, 33, 127, 128), 1500),        # panels in two levels (leading dimension >= 1408), 8 matrices
+    ((129, 160, 257, 1030, 96), 1500),  # the same, clusters of 8 CTAs
+    ((31, 64, 300) + (17,) * 127, 320),  # one level, clusters of 4 CTAs
+])
+def test_recomputation_of_uneven_chains_together(orders, capacity):
+    base = configs.cube8(K=256.0, k_max=32, capacity=capacity)
+    chains = [configs.dataclasses.replace(base, chain_id=i) for i in range(len(orders))]
+    cfgs = [configs.synthetic_configuration(c, n, seed=100 + i) for i, (c, n) in enumerate(zip(chains, orders))]
+    with pk.Context(chains) as ctx:
+        for i, cfg in enumerate(cfgs):
+            ctx.set_config(i, **cfg)
+        ctx.recompute()   # every chain in one set of launches
+        _check_N(ctx, chains[:5], cfgs[:5])
