@@ -33,6 +33,7 @@ struct ctaux_ctx {
   int blocks_since_refresh = 0;
   std::string err;
   int max_ld = 0;
+  std::vector<SlicedStrip> strips;   // of ls.sliced
   // CUDA graphs of one block (with its near-tie launch), of one measurement,
   // and of one block with the previous block's measurement beside it (on the
   // side stream), captured on first use on a private stream, with their
@@ -98,6 +99,110 @@ template <>
 std::vector<Chain<double>>& host_chains<double>(ctaux_ctx* ctx) { return ctx->hc64; }
 template <>
 std::vector<Chain<float>>& host_chains<float>(ctaux_ctx* ctx) { return ctx->hc32; }
+
+// Buffers and work list of the sliced prep and flush products (float64 form)
+// for the chains whose capacity calls for them, in one allocation made last.
+// They are an option: where they would take more than a quarter of the memory
+// that is left, the products stay on the float64 pipe.
+ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
+  LaunchShape& ls = ctx->ls;
+  const int nch = (int)hc.size();
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    const size_t o = at;
+    at += (bytes + 1023) / 1024 * 1024;
+    return o;
+  };
+  std::vector<SlicedView> views(2 * nch);
+  std::vector<SlicedJob> jobs;
+  std::vector<std::vector<size_t>> offs(2 * nch);
+  size_t img = 0, exps = 0, pool = 0, pool_exp = 0;
+  for (int ci = 0; ci < nch; ++ci) {
+    const Chain<double>& c = hc[ci];
+    if (c.cap_m < kSlicedMinOrder) continue;
+    const size_t pl = (c.cap_m + 127) / 128, rows = pl * 128, kr = round_up(c.k_max, 64), yc = round_up(c.k_max, 32) / 32;
+    const size_t partials = sliced_partials(c.cap_m, c.k_max), tiles = pl * ((c.k_max + 63) / 64);
+    for (int spin = 0; spin < 2; ++spin) {
+      std::vector<size_t>& o = offs[2 * ci + spin];
+      for (int pr = 0; pr < 2; ++pr) {
+        o.push_back(take(kr / 64 * pl * 4 * kSlicedImageB));
+        o.push_back(take(kr * pl * sizeof(int)));
+        o.push_back(take(partials * 8192 * sizeof(double)));
+        o.push_back(take(tiles * 16 * sizeof(int)));
+      }
+      o.push_back(take(pl * yc * kSlicedImageA));
+      o.push_back(take(pl * 2 * yc * kSlicedImageB));
+      o.push_back(take(rows * 2 * sizeof(int)));
+      o.push_back(take(rows * 2 * sizeof(int)));
+      views[2 * ci + spin].pl = (int)pl;
+      views[2 * ci + spin].yc = (int)yc;
+      for (int pr = 0; pr < 2; ++pr) {
+        const size_t ib = pl * pl * 4 * kSlicedImageA;
+        if (ctx->strips.empty() || img + ib > kSlicedPool) {   // a new strip
+          ctx->strips.push_back(SlicedStrip{(int)jobs.size(), 0});
+          img = exps = 0;
+        }
+        jobs.push_back(SlicedJob{ci, spin, pr, 0, img, exps});
+        ctx->strips.back().count += 1;
+        img += ib;
+        exps += rows * pl;
+        pool = std::max(pool, img);
+        pool_exp = std::max(pool_exp, exps);
+      }
+    }
+  }
+  ls.any_sliced = 0;
+  ls.any_plain = 1;
+  if (jobs.empty()) return CTAUX_OK;
+  const size_t o_views = take(views.size() * sizeof(SlicedView)), o_jobs = take(jobs.size() * sizeof(SlicedJob)),
+               o_exp = take(pool_exp * sizeof(int)), o_pool = take(pool);
+  size_t free_b = 0, total_b = 0;
+  CUDA_TRY(ctx, cudaMemGetInfo(&free_b, &total_b));
+  void* mem = nullptr;
+  if (at > free_b / 4 || cudaMalloc(&mem, at) != cudaSuccess) {
+    cudaGetLastError();
+    return CTAUX_OK;
+  }
+  ctx->allocations.push_back(mem);
+  unsigned char* base = reinterpret_cast<unsigned char*>(mem);
+  CUDA_TRY(ctx, cudaMemset(mem, 0, o_pool));   // the tickets start at zero
+  int plain = 0;
+  for (int ci = 0; ci < nch; ++ci) {
+    if (offs[2 * ci].empty()) {
+      plain = 1;
+      continue;
+    }
+    hc[ci].sliced = 1;
+    for (int spin = 0; spin < 2; ++spin) {
+      SlicedView& v = views[2 * ci + spin];
+      const std::vector<size_t>& o = offs[2 * ci + spin];
+      for (int pr = 0; pr < 2; ++pr) {
+        v.cs[pr] = base + o[4 * pr];
+        v.ce[pr] = reinterpret_cast<int*>(base + o[4 * pr + 1]);
+        v.part[pr] = reinterpret_cast<double*>(base + o[4 * pr + 2]);
+        v.ticket[pr] = reinterpret_cast<int*>(base + o[4 * pr + 3]);
+      }
+      v.ys = base + o[8];
+      v.xs = base + o[9];
+      v.ye = reinterpret_cast<int*>(base + o[10]);
+      v.xe = reinterpret_cast<int*>(base + o[11]);
+    }
+  }
+  CUDA_TRY(ctx, cudaMemcpy(base + o_views, views.data(), views.size() * sizeof(SlicedView), cudaMemcpyHostToDevice));
+  CUDA_TRY(ctx, cudaMemcpy(base + o_jobs, jobs.data(), jobs.size() * sizeof(SlicedJob), cudaMemcpyHostToDevice));
+  SlicedPlan& p = ls.sliced;
+  p.views = reinterpret_cast<const SlicedView*>(base + o_views);
+  p.jobs = reinterpret_cast<const SlicedJob*>(base + o_jobs);
+  p.pool = base + o_pool;
+  p.pool_exp = reinterpret_cast<int*>(base + o_exp);
+  p.strips = ctx->strips.data();
+  p.n_strips = (int)ctx->strips.size();
+  for (const SlicedStrip& s : ctx->strips) p.max_jobs = std::max(p.max_jobs, s.count);
+  ls.any_sliced = 1;
+  ls.any_plain = plain;
+  CUDA_TRY(ctx, configure_sliced(nch, p.max_jobs));
+  return CTAUX_OK;
+}
 
 template <typename T>
 ctaux_status build_chains(ctaux_ctx* ctx) {
@@ -375,6 +480,11 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
     CUDA_TRY(ctx, cudaMemcpy(dm, host_maps.data(), host_maps.size() * sizeof(TcMaps),
                              cudaMemcpyHostToDevice));
     ctx->tc_maps_dev = reinterpret_cast<TcMaps*>(dm);
+  }
+  ls.any_plain = 1;
+  if constexpr (sizeof(T) == 8) {
+    const ctaux_status bs = build_sliced(ctx, hc);
+    if (bs != CTAUX_OK) return bs;
   }
   void* dc = nullptr;
   CUDA_TRY(ctx, cudaMalloc(&dc, hc.size() * sizeof(Chain<T>)));
@@ -1153,8 +1263,9 @@ ctaux_status ctaux_autotune_tiles(ctaux_ctx* ctx, int n_blocks, int8_t* table_ou
   // work counter that measure them (0 prep, 1 flush, 2 measurement)
   std::vector<std::pair<int, int>> prods;
   if (!(mixed && ctx->ls.prep_tc))
-    for (int ph : {PH_RTILDE, PH_GCOL_OLD, PH_GCOL_NEW}) prods.push_back({ph, 0});
-  if (!(mixed && ctx->ls.use_tc)) prods.push_back({PH_FLUSH, 1});
+    for (int ph : {PH_RTILDE, PH_GCOL_OLD, PH_GCOL_NEW})
+      if (ctx->ls.any_plain || ph == PH_GCOL_NEW) prods.push_back({ph, 0});
+  if (!(mixed && ctx->ls.use_tc) && ctx->ls.any_plain) prods.push_back({PH_FLUSH, 1});
   prods.push_back({PH_MEAS, 2});
   const int timer_phase[3] = {1, 3, 5};
   // groups: (octave of the current order, octave of k_max) slots of the table

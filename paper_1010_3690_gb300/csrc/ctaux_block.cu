@@ -351,7 +351,8 @@ __global__ void __launch_bounds__(256) k_gemm(Chain<T>* chains, int n_chains, in
   for (int ci = threadIdx.x; ci < n_chains; ci += blockDim.x) {
     int a, b, q, wd;
     const Chain<T>& c = chains[ci];
-    off[ci] = (chain_tile_var(c, *c.dyn, PHASE) == V)
+    const bool other = c.sliced && PHASE != PH_GCOL_NEW && PHASE != PH_MEAS;   // ctaux_sliced.cu
+    off[ci] = (!other && chain_tile_var(c, *c.dyn, PHASE) == V)
                   ? gemm_items<T, PHASE>(c, *c.dyn, kchunk, V, a, b, q, wd)
                   : 0;
   }
@@ -1457,8 +1458,13 @@ void launch_block(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st, Pha
     if constexpr (std::is_same<T, float>::value) launch_prep_tc(dchains, maps, ls, st);
     pt->end(1, st, 1 + launch_gemm<T>(dchains, ls, PH_GCOL_NEW, st));
   } else {
-    int nk = launch_gemm<T>(dchains, ls, PH_RTILDE, st);
-    nk += launch_gemm<T>(dchains, ls, PH_GCOL_OLD, st);
+    int nk = 0;
+    if (ls.any_plain) {
+      nk += launch_gemm<T>(dchains, ls, PH_RTILDE, st);
+      nk += launch_gemm<T>(dchains, ls, PH_GCOL_OLD, st);
+    }
+    if constexpr (std::is_same<T, double>::value)
+      if (ls.any_sliced) nk += launch_sliced_prep(dchains, ls, st);
     nk += launch_gemm<T>(dchains, ls, PH_GCOL_NEW, st);
     pt->end(1, st, nk);
   }
@@ -1502,7 +1508,10 @@ void launch_block(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st, Pha
       pt->end(4, st, 1);
     }
   } else {
-    pt->end(3, st, launch_gemm<T>(dchains, ls, PH_FLUSH, st));
+    int nk = ls.any_plain ? launch_gemm<T>(dchains, ls, PH_FLUSH, st) : 0;
+    if constexpr (std::is_same<T, double>::value)
+      if (ls.any_sliced) nk += launch_sliced_flush(dchains, ls, st);
+    pt->end(3, st, nk);
   }
   if (fork) cudaStreamWaitEvent(st, fork->ev_join, 0);   // the side work ends before the block does
   k_finish_block<T><<<(nch + 127) / 128, 128, 0, st>>>(dchains, nch);

@@ -121,6 +121,7 @@ struct Chain {
   T* Gcol[2];
   T* Ginv[2];                // Gamma^{-1}, row-major, row stride k_max + 1 (inverse form)
   T* Glu[2];                 // L (strictly lower) and U (upper) of Gamma, same layout (LU form)
+  int sliced;                // float64 form: prep and flush products on the tensor cores
   int gamma_lu;              // 1: Gamma kept as L U
   double* lam[2];
   int* P;

@@ -5,6 +5,7 @@
 
 #include "ctaux_dev.cuh"
 #include "ctaux_inverse.cuh"
+#include "ctaux_sliced.cuh"
 
 namespace ctaux {
 
@@ -106,6 +107,8 @@ struct LaunchShape {
   int prep_tc;           // mixed form: prep products on the tensor cores
   int gamma_lu;          // Gamma kept as L U (CTAUX_GAMMA_LU)
   int max_k;             // largest k_max of the context's chains
+  int any_sliced, any_plain;  // float64 form: chains with sliced prep and flush products, and without
+  SlicedPlan sliced;
   int tile_mask[PH_COUNT];  // tile variants in the context's table, per product (bit v)
 };
 
@@ -206,6 +209,11 @@ void launch_flush_tc(Chain<float>* dchains, const TcMaps* maps, const LaunchShap
 void launch_transpose_n(Chain<float>* dchains, const LaunchShape& ls, cudaStream_t st);
 cudaError_t encode_tc_maps(TcMaps* out, float* yh, float* yl, float* xh, float* xl, int rows,
                            int kp, float* n0, float* n1, int ld);
+cudaError_t configure_sliced(int n_chains, int max_jobs);
+// The prep products R~ and G_{old,new}, and the flush product, of the sliced
+// chains; return the kernels launched.
+int launch_sliced_prep(const Chain<double>* dchains, const LaunchShape& ls, cudaStream_t st);
+int launch_sliced_flush(const Chain<double>* dchains, const LaunchShape& ls, cudaStream_t st);
 void launch_philox_test(uint64_t seed, uint32_t chain, int64_t t0, int count, int purpose,
                         double* out, cudaStream_t st);
 

@@ -7,7 +7,7 @@ multiply-adds, and the oracle's N comes from a dense float64 inverse.
 import numpy as np
 import pytest
 
-from parity import oracle_for
+from parity import compare_traces, oracle_for
 from workloads import configs
 
 pytestmark = pytest.mark.gpu
@@ -41,3 +41,21 @@ def test_recomputation_of_uneven_chains_together(orders, capacity):
             ctx.set_config(i, **cfg)
         ctx.recompute()   # every chain in one set of launches
         _check_N(ctx, chains[:5], cfgs[:5])
+
+
+@pytest.mark.parametrize("n0,k", [(40, 256), (100, 32), (127, 64), (128, 64), (129, 160), (257, 256), (511, 24)])
+def test_sliced_products_of_a_block_at_tile_edges(n0, k):
+    """Prep (tiles of 128 rows x 64 insertions, parts of 128 of the inner index, split
+    over it) and flush (ranks up to 256, two parts) against the oracle's ratios and N."""
+    ch = configs.cube8(K=256.0, k_max=k, capacity=n0 + 2 * k + 64)
+    cfg = configs.synthetic_configuration(ch, n0, seed=n0)
+    oc = oracle_for(ch, p_insert=0.45, p_flip=0.1)
+    oc.set_config(cfg["tau"], cfg["site"], cfg["s"], cfg["birth"], cfg["t"])
+    with pk.Context([ch], trace_capacity=2 * k, refresh_every=0, p_insert=0.45, p_flip=0.1) as ctx:
+        ctx.set_config(0, **cfg)
+        ctx.sweep(2)
+        ctx.synchronize()
+        compare_traces(ctx.trace(0), oc.run(2 * k), 1e-10)
+        for spin in (0, 1):
+            No = oc.N(spin)
+            np.testing.assert_allclose(ctx.get_N(0, spin), No, rtol=1e-9, atol=1e-10 * np.abs(No).max())
