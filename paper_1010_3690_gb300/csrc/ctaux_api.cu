@@ -274,6 +274,9 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
   ls.gamma_lu = P.gamma_form == CTAUX_GAMMA_LU ? 1 : 0;
   ls.max_k = max_k;
   CUDA_TRY(ctx, configure_block_kernels<T>(ls));
+  int max_cap = 0;
+  for (const auto& cp : ctx->chains) max_cap = std::max(max_cap, cp.capacity + cp.k_max);
+  CUDA_TRY(ctx, configure_gamma_cluster<T>(ls, max_cap, ctx->sm_count));
   const bool mixed_tc = (sizeof(T) == 4) && P.mixed_flush_tc != 0;
   ls.use_tc = mixed_tc ? 1 : 0;
   int max_rows = 128;

@@ -1480,6 +1480,8 @@ void launch_block(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st, Pha
   if (ls.gamma_lu) {
     if (ls.gamma_in_smem) k_proposals_smem<T, true><<<nch, 256, ls.prop_smem, st>>>(dchains);
     else k_proposals<T, true><<<nch, 256, ls.prop_smem, st>>>(dchains);
+  } else if (ls.gamma_cluster) {
+    launch_gamma_cluster<T>(dchains, ls, st);
   } else {
     if (ls.gamma_in_smem) k_proposals_smem<T, false><<<nch, 256, ls.prop_smem, st>>>(dchains);
     else k_proposals<T, false><<<nch, 256, ls.prop_smem, st>>>(dchains);

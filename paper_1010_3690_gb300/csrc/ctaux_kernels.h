@@ -106,11 +106,20 @@ struct LaunchShape {
   int tc_wait_limit;     // polls of a tensor-core flush pipeline wait (0: 2^24)
   int prep_tc;           // mixed form: prep products on the tensor cores
   int gamma_lu;          // Gamma kept as L U (CTAUX_GAMMA_LU)
+  int gamma_cluster, gamma_cluster_smem;  // CTAs per chain of the proposals, 0: one CTA (ctaux_block.cu)
+  int max_cap;           // largest capacity + k_max of the chains
   int max_k;             // largest k_max of the context's chains
   int any_sliced, any_plain;  // float64 form: chains with sliced prep and flush products, and without
   SlicedPlan sliced;
   int tile_mask[PH_COUNT];  // tile variants in the context's table, per product (bit v)
 };
+
+// Row stride of a CTA's share of Gamma^{-1} in the cluster form: four lanes per
+// row read consecutive elements of a warp's eight rows without bank conflicts.
+__host__ __device__ inline int gamma_share_stride(int k, size_t element) {
+  const int unit = element == 8 ? 16 : 32;
+  return k <= 4 ? 4 : (k - 4 + unit - 1) / unit * unit + 4;
+}
 
 // CUDA-event timing of the sweep phases and kernel launch counts.  Phases:
 // 0 plan + G0 gather, 1 prep products, 2 proposals (Gamma growth), 3 flush
@@ -209,6 +218,11 @@ void launch_flush_tc(Chain<float>* dchains, const TcMaps* maps, const LaunchShap
 void launch_transpose_n(Chain<float>* dchains, const LaunchShape& ls, cudaStream_t st);
 cudaError_t encode_tc_maps(TcMaps* out, float* yh, float* yl, float* xh, float* xl, int rows,
                            int kp, float* n0, float* n1, int ld);
+// Proposals with Gamma^{-1} spread over a cluster (ctaux_gamma.cu).
+template <typename T>
+cudaError_t configure_gamma_cluster(LaunchShape& ls, int max_cap, int sm_count);
+template <typename T>
+cudaError_t launch_gamma_cluster(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st);
 cudaError_t configure_sliced(int n_chains, int max_jobs);
 // The prep products R~ and G_{old,new}, and the flush product, of the sliced
 // chains; return the kernels launched.
