@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(256) k_inv_cols(const InvView* views, const in
 // run while it adds to X on the float64 pipe.  Per tile: 34 x 2 MMAs of 48
 // clocks (128 x 64 x 16, bound by shared-memory reads of A and B) against 8192
 // float64 additions, 19 clocks per warp.  Rank 32 takes about 9 us per tile
-// (the epilogue's float64 additions and loads), rank 128 about 15 us.
+// (the epilogue's float64 additions and loads), rank 128 about 9 us.
 constexpr int kUpdStages = 2, kUpdThreads = 576;
 constexpr int kUpdCols = 16;   // columns of an epilogue warp
 constexpr int kUpdStageBytes = oz::kImageA + oz::kImageB;
@@ -514,29 +514,36 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
     // every copy issued lands before the CTA may exit
     for (uint32_t i = issued > kUpdStages ? issued - kUpdStages : 0; i < issued; ++i)
       mbar_wait(smem_u32(full + i % kUpdStages), (i / kUpdStages) & 1);
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {   // all lanes wait, one issues
     uint32_t q = 0, taken = 0;
-    for (int w = blockIdx.x; w < total && !err_s; w += gridDim.x, ++q) {
+    for (int w = blockIdx.x; w < total; w += gridDim.x, ++q) {
+      if (__any_sync(0xffffffffu, err_s != 0)) break;
       const UpdTile t = upd_tile(off, orders, items, w, g.j0);
       const int nc = WIDE ? (min(g.width, t.m - g.c0) + oz::kK - 1) / oz::kK : 1;
-      bool ok = q == 0 || mbar_wait(smem_u32(&accempty), (q - 1) & 1);
+      bool ok = __all_sync(0xffffffffu, q == 0 || mbar_wait(smem_u32(&accempty), (q - 1) & 1));
       for (int c = 0; c < nc && ok; ++c, ++taken) {
         const uint32_t s = taken % kUpdStages;
-        ok = mbar_wait(smem_u32(full + s), (taken / kUpdStages) & 1);
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(full + s), (taken / kUpdStages) & 1));
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t a = smem_u32(base + s * kUpdStageBytes);
-        oz::mma_images(tmem, a, a + oz::kImageA, c == 0);
-        mma_commit(smem_u32(empty + s));
+        if (oz::elect_one()) {
+          if (c == 0) oz::mma_images<true>(tmem, a, a + oz::kImageA);
+          else oz::mma_images<false>(tmem, a, a + oz::kImageA);
+          mma_commit(smem_u32(empty + s));
+        }
+        __syncwarp();
       }
       if (!ok) {
         err_s = 1;
-        atomicOr(views[t.it].status, DS_TIMEOUT);
+        if (lane == 0) atomicOr(views[t.it].status, DS_TIMEOUT);
         break;
       }
-      mma_commit(smem_u32(&accfull));
+      if (oz::elect_one()) mma_commit(smem_u32(&accfull));
+      __syncwarp();
     }
-    mma_commit(smem_u32(&drain));   // every MMA issued completes before the TMEM is freed
+    if (oz::elect_one()) mma_commit(smem_u32(&drain));   // every MMA issued completes before the TMEM is freed
+    __syncwarp();
     mbar_wait(smem_u32(&drain), 0);
   } else if (warp >= 2) {
     const int quarter = warp & 3, group = (warp - 2) >> 2;

@@ -101,29 +101,46 @@ __device__ __forceinline__ void store_chunk(unsigned char* dst, int image_rows, 
 // kind::f16 instruction descriptor: D float32, A and B float16, both K-major, M = 128, N = 64.
 constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 
-__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t acc) {
+// One thread of a converged warp (the same one every time).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+
+// Shared-memory descriptors of K-major tiles with 64-byte rows (tc::smem_desc):
+// the lower word holds the address, the upper one is constant.
+constexpr uint32_t kDescHigh = (512u >> 4) | (1u << 14) | (4u << 29);
+
+template <bool ACC>
+__device__ __forceinline__ void mma_f16(uint32_t tmem, uint32_t a_low, uint32_t b_low) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-      "l"(a), "l"(b), "r"(kIdesc), "r"(acc)
+      "{\n .reg .pred p;\n .reg .b64 da, db;\n mov.b64 da, {%1, %3};\n mov.b64 db, {%2, %3};\n"
+      " setp.ne.b32 p, %5, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n}\n" ::"r"(tmem),
+      "r"(a_low), "r"(b_low), "n"(kDescHigh), "n"(kIdesc), "n"(ACC ? 1 : 0)
       : "memory");
 }
 
 // All digit products of one pair of images into the eight group accumulators
-// (64 TMEM columns each), `first` clearing them.
-__device__ __forceinline__ void mma_images(uint32_t tmem, uint32_t a, uint32_t b, bool first) {
-#pragma unroll 1
+// (64 TMEM columns each), FIRST clearing them; by the elected thread of a
+// converged warp.  With addresses that are uniform in the warp and 32-bit
+// arithmetic an MMA issues every 48 clocks also beside busy epilogue warps; from
+// one thread in a divergent branch with 64-bit descriptors it took 75 there.
+template <bool FIRST>
+__device__ __forceinline__ void mma_images(uint32_t tmem, uint32_t a, uint32_t b) {
+  const uint32_t al = (a >> 4) | (1u << 16), bl = (b >> 4) | (1u << 16);
+#pragma unroll
   for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
     for (int i = 0; i < kSlices; ++i) {
-      const uint64_t da = tc::smem_desc(a + (uint32_t)(i * kRowsA * 64 + kk * 32));
 #pragma unroll
       for (int j = 0; j < kSlices; ++j) {
         const int g = i + j;
         if (g >= kGroups) continue;
-        // the first product of group g is digit 0 of A (g = 7: digit 1) with the last of B
-        const bool fresh = first && kk == 0 && i == (g == 7 ? 1 : 0);
-        mma_f16(tmem + 64 * g, da, tc::smem_desc(b + (uint32_t)(j * kRowsB * 64 + kk * 32)), fresh ? 0u : 1u);
+        const uint32_t x = al + (uint32_t)((i * kRowsA * 64 + kk * 32) >> 4), y = bl + (uint32_t)((j * kRowsB * 64 + kk * 32) >> 4);
+        // the first product of group g is digit 0 of A (g = 7: digit 1)
+        if (FIRST && kk == 0 && i == (g == 7 ? 1 : 0)) mma_f16<false>(tmem + 64 * g, x, y);
+        else mma_f16<true>(tmem + 64 * g, x, y);
       }
     }
   }

@@ -395,27 +395,34 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src) {
     // every copy issued lands before the CTA may exit
     for (uint32_t i = issued > kProdStages ? issued - kProdStages : 0; i < issued; ++i)
       mbar_wait(smem_u32(full + i % kProdStages), (i / kProdStages) & 1);
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {   // all lanes wait, one issues
     uint32_t q = 0, taken = 0;
     bool ok = true;
-    for (int w = blockIdx.x; w < total && ok && !err_s; w += gridDim.x) {
+    for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+      if (__any_sync(0xffffffffu, err_s != 0)) break;
       const ProdItem t = item(w);
       for (int c0 = 0; c0 < t.chunks && ok; c0 += 4, ++q) {
-        ok = q == 0 || mbar_wait(smem_u32(&accempty), (q - 1) & 1);
+        ok = __all_sync(0xffffffffu, q == 0 || mbar_wait(smem_u32(&accempty), (q - 1) & 1));
         for (int c = c0; c < min(t.chunks, c0 + 4) && ok; ++c, ++taken) {
           const uint32_t s = taken % kProdStages;
-          ok = mbar_wait(smem_u32(full + s), (taken / kProdStages) & 1);
+          ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(full + s), (taken / kProdStages) & 1));
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t a = smem_u32(base + s * kProdStageBytes);
-          oz::mma_images(tmem, a, a + oz::kImageA, c == c0);
-          mma_commit(smem_u32(empty + s));
+          if (oz::elect_one()) {
+            if (c == c0) oz::mma_images<true>(tmem, a, a + oz::kImageA);
+            else oz::mma_images<false>(tmem, a, a + oz::kImageA);
+            mma_commit(smem_u32(empty + s));
+          }
+          __syncwarp();
         }
-        if (ok) mma_commit(smem_u32(&accfull));
+        if (ok && oz::elect_one()) mma_commit(smem_u32(&accfull));
+        __syncwarp();
       }
-      if (!ok) fail(t.ci);
+      if (!ok && lane == 0) fail(t.ci);
     }
-    mma_commit(smem_u32(&drain));   // every MMA issued completes before the TMEM is freed
+    if (oz::elect_one()) mma_commit(smem_u32(&drain));   // every MMA issued completes before the TMEM is freed
+    __syncwarp();
     mbar_wait(smem_u32(&drain), 0);
   } else if (warp >= 2) {
     const int quarter = warp & 3, group = (warp - 2) >> 2, rl = quarter * 32 + lane, cl = group * kProdCols;
