@@ -301,8 +301,10 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
   }
   std::vector<TcMaps> host_maps(mixed_tc ? 2 * ctx->chains.size() : 0);
   // from-scratch recomputation: launch shapes for all chains and for one
-  CUDA_TRY(ctx, inv_configure(2, max_ld, ctx->sm_count, &ls.inv_one));
-  CUDA_TRY(ctx, inv_configure(items, max_ld, ctx->sm_count, &ls.inv_all));
+  std::vector<int> lds;
+  for (const auto& cp : ctx->chains) lds.insert(lds.end(), 2, round_up(cp.capacity + cp.k_max, 32));
+  CUDA_TRY(ctx, inv_configure({max_ld, max_ld}, ctx->sm_count, &ls.inv_one));
+  CUDA_TRY(ctx, inv_configure(lds, ctx->sm_count, &ls.inv_all));
   std::vector<InvView> host_views(items);
 
   for (size_t ci = 0; ci < ctx->chains.size(); ++ci) {

@@ -39,10 +39,8 @@ namespace ctaux {
 
 namespace {
 
-constexpr int kPanelThreads = 512;
 constexpr int kMaxWidth = oz::kK;
 constexpr int kMaxCluster = 16;
-constexpr int kPanelWarps = kPanelThreads / 32;
 
 // Pivot key: the upper 32 bits of the float64 pattern of a magnitude (sign 0,
 // the whole exponent, 20 significand bits) order like the magnitude for every
@@ -122,16 +120,24 @@ __device__ __forceinline__ void st_async(uint32_t addr, unsigned long long v, ui
 }
 
 // Column steps of panel [c0, c0 + width) of every matrix, one cluster per
-// matrix, rows dealt to the CTAs in contiguous runs.  Shared memory: the
-// CTA's panel rows [column][row], the multipliers of the last two steps, and
-// three generations of every CTA's candidate (key and row values): a CTA may
-// push step k + 2's while another still updates with step k's.
-// A step of a 32-column panel takes 1.3 us at order 431 (27 rows per CTA: the
-// chain of exchange 540 clocks, selection 250, reciprocal 500, new column and
-// key 600, candidate 400) and 2.3 us at 2000 (125 rows: 116 float64 warp
-// operations of 19 clocks).
-__global__ void __launch_bounds__(kPanelThreads, 1)
+// matrix, rows dealt to the CTAs in contiguous runs.  Step k makes column k its
+// multipliers F[:, k] (-X[i][k] / pivot, and 1 / pivot in the pivot row) and
+// updates only the columns to its right: with the pivot rows' multipliers
+// L[k][l] = F[R_k][l], l < k, every column of the matrix, the panel's own ones
+// included, follows as X'[:, j] = Z[:, j] + F y (k_inv_rows, k_inv_update).  F is
+// written as slices, zero in a pivot row before its own step.
+// Shared memory: the CTA's panel rows [column][row] and three generations of
+// every CTA's candidate (key and row values): a CTA may push step k + 2's while
+// another still updates with step k's.
+// A step's critical chain is about 2500 clocks (exchange 540, selection 250,
+// reciprocal 500, new column and key 600, candidate 400); beside it the update
+// takes 19 clocks of the float64 pipe per column and 32 rows of a CTA, which
+// bounds the step from about 200 rows per CTA on.  Keeping the update to the
+// columns on the right halves that part.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 512 ? 1 : 3)
 k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows_cap) {
+  constexpr int kWarps = THREADS / 32;
   const uint32_t rank = cluster_rank(), ncta = cluster_size();
   const int item = blockIdx.x / ncta;
   const int m = orders[item];
@@ -139,25 +145,24 @@ k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows
   const InvView v = views[item];
   const int bw = min(width, m - c0);
   const int per = (m + (int)ncta - 1) / (int)ncta;
-  const int r0 = min(m, (int)rank * per), nr = min(m, r0 + per) - r0;
+  const int r0 = min(m, (int)rank * per), nr = min(m, r0 + per) - r0, groups = (nr + 31) >> 5;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rs = rows_cap;   // row stride of a panel column
 
   extern __shared__ __align__(16) unsigned char panel_smem[];
   double* Ps = reinterpret_cast<double*>(panel_smem);          // [width][rs]
-  double* fs = Ps + (size_t)width * rs;                        // [2][rs] multipliers
-  double* crow = fs + 2 * rs;                                  // [3][kMaxCluster][kMaxWidth]
+  double* crow = Ps + (size_t)width * rs;                      // [3][kMaxCluster][kMaxWidth]
   unsigned long long* ckey = reinterpret_cast<unsigned long long*>(crow + 3 * kMaxCluster * kMaxWidth);
-  int8_t* us = reinterpret_cast<int8_t*>(ckey + 3 * kMaxCluster);   // [rs] pivoted rows
-  __shared__ uint32_t wmag[kPanelWarps], wrow[kPanelWarps];
+  int8_t* us = reinterpret_cast<int8_t*>(ckey + 3 * kMaxCluster);   // [rs] 0 free, 1 pivoted before, 2 + k in step k
+  __shared__ uint32_t wmag[kWarps], wrow[kWarps];
   __shared__ double cand_row[kMaxWidth];
   __shared__ uint64_t landed[3];   // candidates of a generation: one local arrival and their bytes
   __shared__ volatile int gave_up;
   const uint32_t bytes = ncta * (uint32_t)(sizeof(double) * kMaxWidth + sizeof(unsigned long long));
 
   for (int k = 0; k < bw; ++k)
-    for (int r = tid; r < nr; r += kPanelThreads) Ps[(size_t)k * rs + r] = v.X[(size_t)(c0 + k) * v.ld + r0 + r];
-  for (int r = tid; r < nr; r += kPanelThreads) us[r] = v.used[r0 + r];
+    for (int r = tid; r < nr; r += THREADS) Ps[(size_t)k * rs + r] = v.X[(size_t)(c0 + k) * v.ld + r0 + r];
+  for (int r = tid; r < nr; r += THREADS) us[r] = v.used[r0 + r];
   if (tid == 0) {
     gave_up = 0;
     for (int g = 0; g < 3; ++g) tc::mbar_init(tc::smem_u32(landed + g), 1);
@@ -169,47 +174,11 @@ k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows
   cluster_wait();
 
   PivotKey key{0u, 0u};
-  for (int r = tid; r < nr; r += kPanelThreads)
+  for (int r = tid; r < nr; r += THREADS)
     if (!us[r]) key_max(key, magnitude(Ps[r]), 0xffffffffu - (uint32_t)(r0 + r));
 
   int prl = -1;             // the previous pivot row, local (outside [0, nr) when another CTA's)
   const double* prow = nullptr;   // its values before the step
-  // The update of the columns by step k's pivot row, by warps w0, w0 + 1, ...:
-  // a column per warp, a row per lane.  The pivot row's own multiplier is the
-  // reciprocal pivot and its old value counts as zero: X[pr][j] / pivot comes
-  // from the same multiply-add.
-  auto step_columns = [&](int k, int skip, int w0) {
-    const double* f = fs + (k & 1) * rs;
-    const int groups = (nr + 31) >> 5;
-    for (int j = warp < w0 ? bw : warp - w0; j < bw; j += kPanelWarps - w0) {
-      if (j == k || j == skip || j == skip + 1) continue;
-      const double pj = prow[j];
-      double* Pj = Ps + (size_t)j * rs;
-      // groups of 32 rows, four at a time; branches, not predicates: a float64
-      // operation whose lanes are all masked holds the pipe as long as a real one
-      int g = 0;
-      for (; g + 4 <= groups; g += 4) {
-        double x[4], y[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int r = (g + q) * 32 + lane;
-          x[q] = r < nr && r != prl ? Pj[r] : 0.0;
-          y[q] = r < nr ? f[r] : 0.0;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) x[q] = fma(y[q], pj, x[q]);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if ((g + q) * 32 + lane < nr) Pj[(g + q) * 32 + lane] = x[q];
-      }
-#pragma unroll 1
-      for (; g < groups; ++g) {
-        const int r = g * 32 + lane;
-        const double x = fma(r < nr ? f[r] : 0.0, pj, r < nr && r != prl ? Pj[r] : 0.0);
-        if (r < nr) Pj[r] = x;
-      }
-    }
-  };
 
   for (int k = 0; k < bw; ++k) {
     // ---- the CTA's candidate
@@ -221,36 +190,66 @@ k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows
     __syncthreads();
     const int gen = k % 3;
     const uint32_t bar = tc::smem_u32(landed + gen);
+    const double* f = k > 0 ? Ps + (size_t)(k - 1) * rs : Ps;   // the previous step's multipliers
     PivotKey cand{0u, 0u};
-    double x = 0.0;
     if (warp == 0) {
-      if (lane < kPanelWarps) cand = PivotKey{wmag[lane], wrow[lane]};
+      double x = 0.0;
+      if (lane < kWarps) cand = PivotKey{wmag[lane], wrow[lane]};
       cand = warp_key_max(cand);
-      if (cand.row && lane < bw) {   // otherwise no row is left here
+      if (cand.row && lane < bw && lane >= k) {   // otherwise no row is left here
         const int lr = (int)(0xffffffffu - cand.row) - r0;
         x = Ps[(size_t)lane * rs + lr];
-        if (k > 0 && lane != k && lane != k - 1) x = fma(fs[((k - 1) & 1) * rs + lr], prow[lane], x);
+        if (k > 0 && lane != k) x = fma(f[lr], prow[lane], x);
       }
       cand_row[lane] = x;
       if (lane == 0) tc::mbar_expect_tx(bar, bytes);
     }
     __syncthreads();   // the candidate row is read before the update below changes it
     const uint32_t slot = (uint32_t)(gen * kMaxCluster + (int)rank);
-    if (warp < (int)ncta)   // the row to every CTA, a warp each
-      st_async(map_rank(tc::smem_u32(crow + slot * kMaxWidth + lane), (uint32_t)warp),
-               (unsigned long long)__double_as_longlong(cand_row[lane]), map_rank(bar, (uint32_t)warp));
+    for (uint32_t w = (uint32_t)warp; w < ncta; w += kWarps)   // the row to every CTA, a warp each
+      st_async(map_rank(tc::smem_u32(crow + slot * kMaxWidth + lane), w),
+               (unsigned long long)__double_as_longlong(cand_row[lane]), map_rank(bar, w));
     if (warp == 0 && lane < (int)ncta)   // its key, a lane each
       st_async(map_rank(tc::smem_u32(ckey + slot), (uint32_t)lane),
                ((unsigned long long)cand.mag << 32) | cand.row, map_rank(bar, (uint32_t)lane));
-    // ---- the previous step's update of the other columns, while the candidates travel
+    // ---- the previous step's update of the columns to its right, while the
+    // candidates travel.  In the pivot row the multiplier is the reciprocal
+    // pivot and the old value counts as zero: X[pr][j] / pivot comes from the
+    // same multiply-add.
     if (k > 0) {
       if (k + 1 < bw) {   // column k + 1 by the threads that own its rows in this step
         const double pn = prow[k + 1];
-        const double* f = fs + ((k - 1) & 1) * rs;
         double* Pn = Ps + (size_t)(k + 1) * rs;
-        for (int r = tid; r < nr; r += kPanelThreads) Pn[r] = fma(f[r], pn, r == prl ? 0.0 : Pn[r]);
+        for (int r = tid; r < nr; r += THREADS) Pn[r] = fma(f[r], pn, r == prl ? 0.0 : Pn[r]);
       }
-      step_columns(k - 1, k, 1);   // warp 0 goes on to wait
+      // the others a column per warp, a row per lane; warp 0 goes on to wait
+      for (int j = warp == 0 ? bw : k + 1 + warp; j < bw; j += kWarps - 1) {
+        const double pj = prow[j];
+        double* Pj = Ps + (size_t)j * rs;
+        // groups of 32 rows, four at a time; branches, not predicates: a float64
+        // operation whose lanes are all masked holds the pipe as long as a real one
+        int g = 0;
+        for (; g + 4 <= groups; g += 4) {
+          double x[4], y[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int r = (g + q) * 32 + lane;
+            x[q] = r < nr && r != prl ? Pj[r] : 0.0;
+            y[q] = r < nr ? f[r] : 0.0;
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) x[q] = fma(y[q], pj, x[q]);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if ((g + q) * 32 + lane < nr) Pj[(g + q) * 32 + lane] = x[q];
+        }
+#pragma unroll 1
+        for (; g < groups; ++g) {
+          const int r = g * 32 + lane;
+          const double x = fma(r < nr ? f[r] : 0.0, pj, r < nr && r != prl ? Pj[r] : 0.0);
+          if (r < nr) Pj[r] = x;
+        }
+      }
     }
     if (!__all_sync(0xffffffffu, tc::mbar_wait(bar, (uint32_t)(k / 3) & 1, gave_up ? 1u : tc::kWaitLimit))) {
       if (lane == 0) {   // the remaining steps run without waiting and without pivots
@@ -280,17 +279,15 @@ k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows
       v.piv[c0 + k] = piv;
       if (!(fabs(piv) > 0.0) || !isfinite(piv)) atomicOr(v.status, DS_SINGULAR);
     }
-    double* f = fs + (k & 1) * rs;
     key = PivotKey{0u, 0u};
     const double ipiv = warp * 32 < nr ? reciprocal(prow[k]) : 0.0;   // warps that own rows
     const bool next = k + 1 < bw;
     const double pn = next ? prow[k + 1] : 0.0;
-    for (int r = tid; r < nr; r += kPanelThreads) {
+    for (int r = tid; r < nr; r += THREADS) {
       const bool piv_row = r == prl;
       const double fr = (piv_row ? 1.0 : -Ps[(size_t)k * rs + r]) * ipiv;
-      f[r] = fr;
       Ps[(size_t)k * rs + r] = fr;
-      if (piv_row) us[r] = 1;
+      if (piv_row) us[r] = (int8_t)(2 + k);
       if (next) {
         const double xn = fma(fr, pn, piv_row ? 0.0 : Ps[(size_t)(k + 1) * rs + r]);
         Ps[(size_t)(k + 1) * rs + r] = xn;
@@ -299,18 +296,17 @@ k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows
     }
   }
   __syncthreads();
-  step_columns(bw - 1, bw - 1, 0);
-  __syncthreads();
   cluster_arrive();   // no CTA exits while another may still store to it
-  // ---- P' back into X, and its slices
-  for (int k = 0; k < bw; ++k)
-    for (int r = tid; r < nr; r += kPanelThreads) v.X[(size_t)(c0 + k) * v.ld + r0 + r] = Ps[(size_t)k * rs + r];
-  // four threads per row, 8 columns (one 16-byte chunk of every slice) each
-  for (int e = tid; e < ((nr + 31) & ~31) * 4; e += kPanelThreads) {
+  // ---- L, and the slices of F: four threads per row, 8 columns (one 16-byte
+  // chunk of every slice) each
+  for (int e = tid; e < ((nr + 31) & ~31) * 4; e += THREADS) {
     const int r = (e >> 7) * 32 + lane, ch = (e >> 5) & 3;
     if (r >= nr) continue;
+    const int step = (int)us[r] - 2;   // of a pivot row of this panel
+    if (step >= 0)
+      for (int k = ch * 8; k < min(step, ch * 8 + 8); ++k) v.L[step * kMaxWidth + k] = Ps[(size_t)k * rs + r];
     int mx = 0;
-    for (int k = 0; k < bw; ++k)
+    for (int k = max(step, 0); k < bw; ++k)
       mx = max(mx, oz::exp_field((uint32_t)__double2hiint(Ps[(size_t)k * rs + r])));
     const int row = r0 + r;
     unsigned char* img = v.As + (size_t)(row >> 7) * v.chunks * oz::kImageA + oz::chunk_offset(row & 127, ch);
@@ -318,7 +314,7 @@ k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
       const int k = ch * 8 + t;
-      y[t] = oz::biased_digits(k < bw ? Ps[(size_t)k * rs + r] : 0.0, mx);
+      y[t] = oz::biased_digits(k < bw && k >= step ? Ps[(size_t)k * rs + r] : 0.0, mx);
     }
     oz::store_chunk(img, oz::kRowsA, y);
     if (ch == 0) v.ea[row] = oz::row_exponent(mx);
@@ -327,13 +323,16 @@ k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows
   cluster_wait();
 }
 
-// A product's columns: [j0, j1) without the panel [c0, c0 + width).
+// A product's columns: [j0, j1), of rank 32 with the panel [c0, c0 + width)
+// itself, of rank 128 without it (its columns are final then).
 struct InvRange {
   int c0, width, j0, j1;
 };
 
 // The pivot rows of the panel, in the columns of the range, as slice images: a
-// warp per column, up to four pivot rows per lane.
+// warp per column, a lane per pivot row.  Rank 32: y_k, the column at pivot row k
+// just before step k, y_k = X[R_k][j] + sum_{l<k} L[k][l] y_l; the panel's own
+// column c0 + k starts from the unit vector e_k.
 __global__ void __launch_bounds__(256) k_inv_rows(const InvView* views, const int* orders, int items,
                                                   InvRange g) {
   __shared__ int off[2 * kMaxChains + 1];
@@ -344,21 +343,38 @@ __global__ void __launch_bounds__(256) k_inv_rows(const InvView* views, const in
   __syncthreads();
   block_exclusive_scan(off, items);
   const int total = off[items], lane = threadIdx.x & 31;
+  const bool wide = g.width > oz::kK;
   for (int u = blockIdx.x; u < total; u += gridDim.x) {
     const int it = find_chain(off, items, u);
     const InvView& v = views[it];
     const int m = orders[it], bw = min(g.width, m - g.c0);
     const int j = g.j0 + (u - off[it]) * 8 + (threadIdx.x >> 5);
-    if (j >= min(m, g.j1) || (j >= g.c0 && j < g.c0 + bw)) continue;   // the whole warp
+    const bool own = j >= g.c0 && j < g.c0 + bw;
+    if (j >= min(m, g.j1) || (wide && own)) continue;   // the whole warp
     const int nc = (bw + oz::kK - 1) / oz::kK;
     double x[4];
     int mx = 0;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const int k = c * oz::kK + lane;
-      x[c] = k < bw ? v.X[(size_t)j * v.ld + v.perm[g.c0 + k]] : 0.0;
-      mx = max(mx, oz::exp_field((uint32_t)__double2hiint(x[c])));
+      x[c] = k >= bw ? 0.0 : own ? (j == g.c0 + k ? 1.0 : 0.0) : v.X[(size_t)j * v.ld + v.perm[g.c0 + k]];
     }
+    if (!wide) {
+      // forward substitution, a lane per row; eight multipliers in flight
+      for (int l0 = 0; l0 < bw - 1; l0 += 8) {
+        double lk[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) lk[t] = lane < bw && l0 + t < lane ? v.L[lane * kMaxWidth + l0 + t] : 0.0;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          if (l0 + t >= bw - 1) break;
+          const double yl = __shfl_sync(0xffffffffu, x[0], l0 + t);
+          x[0] = fma(lk[t], yl, x[0]);
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) mx = max(mx, oz::exp_field((uint32_t)__double2hiint(x[c])));
     mx = __reduce_max_sync(0xffffffffu, mx);
     unsigned char* img = v.Bs + (size_t)(j >> 6) * v.chunks * oz::kImageB +
                          oz::chunk_offset(j & 63, lane >> 3) + (lane & 7) * 2;
@@ -415,7 +431,8 @@ __global__ void __launch_bounds__(256) k_inv_cols(const InvView* views, const in
   }
 }
 
-// X'[:, J] = Z[:, J] + P' X[R, J] in 128 x 64 tiles: one persistent CTA per
+// X'[:, J] = Z[:, J] + F Y (rank 32; Z = 0 in the panel's own columns) or
+// Z[:, J] + P' X[R, J] (rank 128) in 128 x 64 tiles: one persistent CTA per
 // SM, warp 0 bulk copies (two stages of one image pair each), warp 1 the 68
 // MMAs of a tile into the eight group accumulators (all 512 TMEM columns),
 // warps 2-17 the epilogue (TMEM lane quarter w % 4, 16 columns each), which empties
@@ -449,8 +466,8 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
   __shared__ int off[2 * kMaxChains + 1];
   for (int i = threadIdx.x; i < items; i += blockDim.x) {
     const int m = orders[i];
-    const int cols = min(m, g.j1) - g.j0;   // more than the panel alone
-    off[i] = m > g.c0 && cols > min(g.width, m - g.c0) ? ((m + 127) / 128) * ((cols + 63) / 64) : 0;
+    const int cols = min(m, g.j1) - g.j0;
+    off[i] = m > g.c0 && !(WIDE && cols <= min(g.width, m - g.c0)) ? ((m + 127) / 128) * ((cols + 63) / 64) : 0;
   }
   __syncthreads();
   block_exclusive_scan(off, items);
@@ -596,7 +613,7 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
 #pragma unroll
       for (int e = 0; e < kUpdCols; ++e) {
         const int j = jb + e;
-        if (row_ok && j < je && !(j >= g.c0 && j < cn))
+        if (row_ok && j < je && !(WIDE && j >= g.c0 && j < cn))
           Xi[(size_t)e * ld] = z[e] + oz::scaled_double(S[e], ea + eb[e]);
       }
     }
@@ -610,58 +627,65 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
 constexpr int upd_smem() { return kUpdStages * kUpdStageBytes + 1024; }
 
 int panel_smem_bytes(int width, int rows) {
-  return (int)(sizeof(double) * ((size_t)(width + 2) * rows + 3 * kMaxCluster * kMaxWidth) +
+  return (int)(sizeof(double) * ((size_t)width * rows + 3 * kMaxCluster * kMaxWidth) +
                sizeof(unsigned long long) * 3 * kMaxCluster + (size_t)((rows + 15) & ~15));
 }
 
 }  // namespace
 
-cudaError_t inv_configure(int items, int max_ld, int sm_count, InvShape* out) {
+// Cluster size per panel, from the matrices that can still reach it: 16 CTAs for
+// a few (a GPC holds one such cluster; order 431 alone: 1.23 ms, against 1.35 with
+// 8 and 1.48 with 4; order 2000: 8.3, 9.8, 13.2), 8 in batches (192 matrices of up
+// to order 1084: 13.0 ms, 14.3 with 4; larger clusters pay where a batch's last,
+// largest matrices are left), 4 beyond 256 matrices, whose rows fill the float64
+// pipes of all SMs anyway.
+cudaError_t inv_configure(const std::vector<int>& lds, int sm_count, InvShape* out) {
   InvShape s{};
-  s.chunks = inv_chunks(max_ld);
   s.sm_count = sm_count;
-  // a cluster of 16 (one GPC holds one or two) for a few matrices; smaller
-  // clusters where more matrices than that run side by side
-  s.cluster = items <= 8 ? 16 : items <= 256 ? 8 : 4;
-  s.rows = (max_ld + s.cluster - 1) / s.cluster;
-  s.width = kMaxWidth;
-  while (s.width > 4 && panel_smem_bytes(s.width, s.rows) > 220 * 1024) s.width /= 2;
-  if (panel_smem_bytes(s.width, s.rows) > 220 * 1024) {   // very large orders in large batches
-    s.cluster = 16;
-    s.rows = (max_ld + 15) / 16;
-    s.width = kMaxWidth;
-    while (s.width > 4 && panel_smem_bytes(s.width, s.rows) > 220 * 1024) s.width /= 2;
-  }
-  s.smem = panel_smem_bytes(s.width, s.rows);
-  cudaError_t e = cudaFuncSetAttribute(k_inv_panel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_inv_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_inv_update<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, upd_smem());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_inv_update<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, upd_smem());
-  if (e == cudaSuccess && s.cluster == 16) {
+  int max_ld = 1;
+  for (int ld : lds) max_ld = ld > max_ld ? ld : max_ld;
+  s.chunks = inv_chunks(max_ld);
+  auto attrs = [&](auto* fn, int bytes) {
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return e;
+  };
+  const int most = 220 * 1024;
+  cudaError_t e = cudaFuncSetAttribute(k_inv_panel<512>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) e = attrs(k_inv_panel<512>, most);
+  if (e == cudaSuccess) e = attrs(k_inv_panel<256>, most);
+  if (e == cudaSuccess) e = attrs(k_inv_update<false>, upd_smem());
+  if (e == cudaSuccess) e = attrs(k_inv_update<true>, upd_smem());
+  if (e != cudaSuccess) return e;
+  auto smem_of = [&](int cluster) { return panel_smem_bytes(s.width, (max_ld + cluster - 1) / cluster); };
+  // 16 CTAs need a GPC with that many free SMs
+  int largest = 16;
+  {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(16);
-    cfg.blockDim = dim3(kPanelThreads);
-    cfg.dynamicSmemBytes = (size_t)s.smem;
+    cfg.blockDim = dim3(512);
+    cfg.dynamicSmemBytes = most;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeClusterDimension;
     at.val.clusterDim.x = 16;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    int fit = 0;
-    e = cudaOccupancyMaxActiveClusters(&fit, k_inv_panel, &cfg);
-    if (e == cudaSuccess && fit == 0) {   // no GPC with 16 free SMs: the portable size
-      s.cluster = 8;
-      s.rows = (max_ld + 7) / 8;
-      while (s.width > 4 && panel_smem_bytes(s.width, s.rows) > 220 * 1024) s.width /= 2;
-      s.smem = panel_smem_bytes(s.width, s.rows);
-    }
+    int n = 0;
+    e = cudaOccupancyMaxActiveClusters(&n, k_inv_panel<512>, &cfg);
+    if (e != cudaSuccess) return e;
+    if (n == 0) largest = 8;
+  }
+  s.width = kMaxWidth;
+  while (s.width > 4 && smem_of(largest) > most) s.width /= 2;
+  for (int c0 = 0; c0 < max_ld; c0 += s.width) {
+    int active = 0;
+    for (int ld : lds) active += ld > c0;
+    int cl = active <= 8 ? largest : active <= 256 ? 8 : 4;
+    while (cl < largest && smem_of(cl) > most) cl *= 2;
+    s.panels.push_back(InvPanel{cl, cl == 16 ? 512 : 256, (max_ld + cl - 1) / cl, smem_of(cl)});
   }
   *out = s;
-  return e;
+  return cudaSuccess;
 }
 
 int launch_inverse(const InvView* views, const int* orders, int items, int max_order,
@@ -682,25 +706,29 @@ int launch_inverse(const InvView* views, const int* orders, int items, int max_o
   const int outer = sh.chunks == 4 ? 128 : sh.width;
   for (int o0 = 0; o0 < max_order; o0 += outer) {
     for (int c0 = o0; c0 < o0 + outer && c0 < max_order; c0 += sh.width) {
+      const InvPanel& pn = sh.panels[c0 / sh.width];
       cudaLaunchConfig_t cfg{};
-      cfg.gridDim = dim3((unsigned)(items * sh.cluster));
-      cfg.blockDim = dim3(kPanelThreads);
-      cfg.dynamicSmemBytes = (size_t)sh.smem;
+      cfg.gridDim = dim3((unsigned)(items * pn.cluster));
+      cfg.blockDim = dim3((unsigned)pn.threads);
+      cfg.dynamicSmemBytes = (size_t)pn.smem;
       cfg.stream = st;
       cudaLaunchAttribute at{};
       at.id = cudaLaunchAttributeClusterDimension;
-      at.val.clusterDim.x = (unsigned)sh.cluster;
+      at.val.clusterDim.x = (unsigned)pn.cluster;
       at.val.clusterDim.y = at.val.clusterDim.z = 1;
       cfg.attrs = &at;
       cfg.numAttrs = 1;
-      const cudaError_t e = cudaLaunchKernelEx(&cfg, k_inv_panel, views, orders, c0, sh.width, sh.rows);
+      const cudaError_t e =
+          pn.threads == 512 ? cudaLaunchKernelEx(&cfg, k_inv_panel<512>, views, orders, c0, sh.width, pn.rows)
+                            : cudaLaunchKernelEx(&cfg, k_inv_panel<256>, views, orders, c0, sh.width, pn.rows);
       n += 1;
       if (e != cudaSuccess) {
         *err = e;
         return n;
       }
-      if (outer > sh.width && max_order > o0 + sh.width) update(c0, sh.width, o0, o0 + outer);
+      update(c0, sh.width, outer > sh.width ? o0 : 0, outer > sh.width ? o0 + outer : max_order);
     }
+    if (outer == sh.width) continue;
     if (max_order <= outer) continue;   // no columns outside the panel
     if (sh.chunks == 4) {
       k_inv_cols<<<grid(items * ((max_order + 15) / 16), 8 * sms), 256, 0, st>>>(views, orders, items, o0);

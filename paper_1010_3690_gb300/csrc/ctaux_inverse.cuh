@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 namespace ctaux {
 
 // One matrix and its work area (device pointers).
@@ -20,6 +22,7 @@ struct InvView {
   int8_t* used;         // row already pivoted
   int* pcol;            // column at which a row was pivoted, -1 if not yet
   double* piv;          // pivots, in column order
+  double* L;            // [32][32] multipliers of the current panel's pivot rows
   int* status;          // DS_SINGULAR and DS_TIMEOUT bits
 };
 
@@ -36,7 +39,7 @@ inline int inv_chunks(int max_ld) { return max_ld >= kInvTwoLevel ? 4 : 1; }
 // comes first and takes ld^2 doubles).
 __host__ __device__ inline size_t inv_extra_doubles(int ld, int chunks = 4) {
   const size_t lp = (size_t)((ld + 127) / 128 * 128);
-  return lp * (112 * (size_t)chunks + 2);   // 2 x 448 bytes of slices per chunk
+  return lp * (112 * (size_t)chunks + 2) + 1024;   // 2 x 448 bytes of slices per chunk; L
 }
 __host__ __device__ inline void inv_layout(double* work, int ld, int chunks, InvView& v) {
   const size_t lp = (size_t)((ld + 127) / 128 * 128), slices = lp * 448 * (size_t)chunks;
@@ -49,19 +52,24 @@ __host__ __device__ inline void inv_layout(double* work, int ld, int chunks, Inv
   v.ea = reinterpret_cast<int*>(p + 2 * slices);
   v.eb = v.ea + lp;
   v.piv = reinterpret_cast<double*>(v.eb + lp);
+  v.L = v.piv + lp;
 }
 
-// Launch parameters of the inversion of up to `items` matrices of leading
-// dimension at most max_ld.
-struct InvShape {
-  int cluster;     // CTAs of a panel's cluster (16, 8 or 4)
-  int width;       // panel width (32; 16 or 8 where a panel would not fit)
-  int rows;        // panel rows per CTA at max_ld
-  int smem;        // dynamic shared memory of the panel kernel
-  int chunks;      // 4: two levels
-  int sm_count;
+// Launch parameters of the inversion of a set of matrices.
+struct InvPanel {
+  int cluster;     // CTAs of a matrix's cluster (2 to 16)
+  int threads;     // of a CTA: 512 in clusters of 16, else 256
+  int rows;        // panel rows per CTA at the largest leading dimension
+  int smem;        // dynamic shared memory
 };
-cudaError_t inv_configure(int items, int max_ld, int sm_count, InvShape* out);
+struct InvShape {
+  int width;                     // panel width (32; 16 or 8 where a panel would not fit)
+  int chunks;                    // 4: two levels
+  int sm_count;
+  std::vector<InvPanel> panels;  // of each panel: fewer matrices reach the later ones
+};
+// lds: the leading dimension of every matrix.
+cudaError_t inv_configure(const std::vector<int>& lds, int sm_count, InvShape* out);
 
 // Inverts the matrices views[0..items) of orders orders[0..items) (device; 0 =
 // leave out), none above max_order: afterwards inv[c][perm[j]] = X[perm[c]][j].
