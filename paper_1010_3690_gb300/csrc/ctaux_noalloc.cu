@@ -1,116 +1,81 @@
-// ctaux_invert_noalloc: the FP64 Gauss-Jordan inversion of the from-scratch
-// recomputation, for callers that cannot allocate device memory.  Its scratch
-// (two ping-pong matrices, pivot keys, pivot flags, the pivot permutation and
-// the log-determinant accumulator) lives in one file-scope static device
-// array; nothing here calls cudaMalloc, cudaFree or an allocating library
-// routine.  Declared in include/ctaux.h.
-#include <cooperative_groups.h>
+// ctaux_invert_noalloc: the blocked Gauss-Jordan inversion of the from-scratch
+// recomputation (ctaux_inverse.cu), for callers that cannot allocate device
+// memory.  Its scratch (the matrix, the slices, pivots and flags) lives in one
+// file-scope static device array; nothing here calls cudaMalloc, cudaFree or an
+// allocating library routine.  Declared in include/ctaux.h.
 #include <cuda_runtime.h>
 
 #include <mutex>
 
 #include "../../include/ctaux.h"
-
-namespace cg = cooperative_groups;
+#include "ctaux_dev.cuh"
+#include "ctaux_inverse.cuh"
 
 namespace {
 
+using namespace ctaux;
+
 constexpr int kM = CTAUX_NOALLOC_MAX_M;
-constexpr size_t kWorkDoubles = (size_t)2 * kM * kM;
-constexpr size_t kScratchBytes = kWorkDoubles * sizeof(double)  // ping-pong matrices
-                                 + kM * sizeof(unsigned long long)  // pivot keys
-                                 + kM * sizeof(int)                 // pivot rows
-                                 + kM * sizeof(int)                 // pivot flags
-                                 + 2 * sizeof(double);              // log|det|, spare
-static_assert(kScratchBytes <= CTAUX_NOALLOC_SCRATCH_BYTES, "scratch size in the header");
+
+// Scratch layout, bytes: the work area of one matrix, then the pivot arrays,
+// the order and the view.
+constexpr size_t kWork = ((size_t)kM * kM + (size_t)kM * 114 + 1024) * sizeof(double);   // ld^2 + inv_extra_doubles(kM, 1)
+constexpr size_t kPerm = kWork, kPcol = kPerm + kM * sizeof(int), kUsed = kPcol + kM * sizeof(int),
+                 kStatus = kUsed + kM, kOrder = kStatus + 16, kView = kOrder + 16, kEnd = kView + sizeof(InvView);
+static_assert(kEnd <= CTAUX_NOALLOC_SCRATCH_BYTES, "scratch size in the header");
 
 // Shared by every call on a device; held by each device that loads the library.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[CTAUX_NOALLOC_SCRATCH_BYTES];
+static __device__ __align__(1024) unsigned char g_noalloc_scratch[CTAUX_NOALLOC_SCRATCH_BYTES];
 
-// Pivot key: the upper 32 bits of |v|'s float64 pattern (sign 0, the whole
-// exponent, 20 significand bits) order like |v| for every non-negative double,
-// so any normal entry, however small, beats an exact zero; ties within 2^-20
-// go to the lower row.
-__device__ __forceinline__ unsigned long long na_pivot_key(double v, int row) {
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(fabs(v));
-  return (bits & 0xffffffff00000000ull) | (unsigned long long)(0xffffffffu - (unsigned)row);
-}
-__device__ __forceinline__ int na_key_row(unsigned long long k) {
-  return (int)(0xffffffffu - (unsigned)(k & 0xffffffffull));
-}
-
-// Cooperative kernel: m Gauss-Jordan column steps with partial pivoting,
-// ping-pong between the two scratch matrices, grid barriers between steps
-// (the same arithmetic as the context's FP64 refresh).
-__global__ void __launch_bounds__(256) k_invert_noalloc(const double* __restrict__ A, int lda,
-                                                        double* __restrict__ Ainv, int ldi, int m,
-                                                        unsigned char* scratch, double* logdet_out) {
-  cg::grid_group grid = cg::this_grid();
-  double* W0 = reinterpret_cast<double*>(scratch);
-  double* W1 = W0 + (size_t)kM * kM;
-  unsigned long long* keys = reinterpret_cast<unsigned long long*>(W0 + kWorkDoubles);
-  int* perm = reinterpret_cast<int*>(keys + kM);
-  int* used = perm + kM;
-  double* acc = reinterpret_cast<double*>(used + kM);
-  const long gtid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long gthreads = (long)gridDim.x * blockDim.x;
-
-  // the previous call's keys, flags and log-determinant must not leak in
-  for (long e = gtid; e < kM; e += gthreads) {
-    keys[e] = 0ull;
-    used[e] = 0;
+// The matrix into the scratch, with the state the inversion starts from (the
+// previous call's must not leak in).
+__global__ void __launch_bounds__(256) k_noalloc_load(const double* __restrict__ A, int lda, int m, InvView v,
+                                                      unsigned char* scratch) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *reinterpret_cast<InvView*>(scratch + kView) = v;
+    *reinterpret_cast<int*>(scratch + kOrder) = m;
+    *v.status = 0;
   }
-  if (gtid == 0) acc[0] = 0.0;
-  grid.sync();
-
-  for (int j = blockIdx.x; j < m; j += gridDim.x)
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-      const double v = A[(size_t)j * lda + i];
-      W0[(size_t)j * kM + i] = v;
-      if (j == 0) atomicMax(keys, na_pivot_key(v, i));
+  for (int j = blockIdx.x; j < m; j += gridDim.x) {
+    if (threadIdx.x == 0) {
+      v.used[j] = 0;
+      v.pcol[j] = -1;
     }
-  grid.sync();
-
-  for (int col = 0; col < m; ++col) {
-    const double* X = (col & 1) ? W1 : W0;
-    double* Y = (col & 1) ? W0 : W1;
-    const int pr = na_key_row(keys[col]);
-    const double piv = X[(size_t)col * kM + pr];
-    if (gtid == 0) {
-      perm[col] = pr;
-      used[pr] = 1;
-      acc[0] += log(fabs(piv));
-    }
-    const double ipiv = 1.0 / piv;
-    for (int j = blockIdx.x; j < m; j += gridDim.x) {
-      const double xpj = X[(size_t)j * kM + pr] * ipiv;
-      const double* Xj = X + (size_t)j * kM;
-      const double* Xc = X + (size_t)col * kM;
-      double* Yj = Y + (size_t)j * kM;
-      for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        double v;
-        if (i == pr) v = (j == col) ? ipiv : xpj;
-        else if (j == col) v = -Xc[i] * ipiv;
-        else v = Xj[i] - Xc[i] * xpj;
-        Yj[i] = v;
-        if (j == col + 1 && i != pr && !used[i]) atomicMax(keys + col + 1, na_pivot_key(v, i));
-      }
-    }
-    grid.sync();
+    for (int i = threadIdx.x; i < m; i += blockDim.x) v.X[(size_t)j * v.ld + i] = A[(size_t)j * lda + i];
   }
+}
 
-  const double* X = (m & 1) ? W1 : W0;
-  for (int j = blockIdx.x; j < m; j += gridDim.x)
+// The inverse in the caller's order, and log|det| (the pivots' logarithms, in a
+// fixed order).  NaN where a bounded wait of the inversion gave up.
+__global__ void __launch_bounds__(256) k_noalloc_store(double* __restrict__ Ainv, int ldi, int m, InvView v,
+                                                       double* logdet) {
+  const double poison = (*v.status & ~DS_SINGULAR) ? nan("") : 0.0;
+  for (int j = blockIdx.x; j < m; j += gridDim.x) {
+    const int pj = v.perm[j];
     for (int c = threadIdx.x; c < m; c += blockDim.x)
-      Ainv[(size_t)perm[j] * ldi + c] = X[(size_t)j * kM + perm[c]];  // inv[c][perm[j]]
-  if (gtid == 0 && logdet_out) *logdet_out = acc[0];
+      Ainv[(size_t)pj * ldi + c] = v.X[(size_t)j * v.ld + v.perm[c]] + poison;   // inv[c][perm[j]]
+  }
+  if (blockIdx.x == 0 && logdet) {
+    __shared__ double part[8];
+    double s = 0.0;
+    for (int k = threadIdx.x; k < m; k += blockDim.x) s += log(fabs(v.piv[k]));
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int w = 0; w < 8; ++w) t += part[w];
+      *logdet = t + poison;
+    }
+  }
 }
 
 struct DeviceSetup {
   std::once_flag once;
   cudaError_t err = cudaSuccess;
   unsigned char* scratch = nullptr;  // device address of g_noalloc_scratch
-  int grid = 0;
+  int sms = 0;
+  InvShape shape;
 };
 constexpr int kMaxDevices = 64;
 DeviceSetup g_setup[kMaxDevices];
@@ -129,17 +94,24 @@ extern "C" ctaux_status ctaux_invert_noalloc(const double* d_a, int lda, double*
   // array is only a stand-in, so resolve its device address here
   std::call_once(s.once, [&s, dev]() {
     s.err = cudaGetSymbolAddress(reinterpret_cast<void**>(&s.scratch), g_noalloc_scratch);
-    int sms = 0, per_sm = 0;
-    if (s.err == cudaSuccess) s.err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (s.err == cudaSuccess)
-      s.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_invert_noalloc, 256, 0);
-    s.grid = (per_sm > 0 ? per_sm : 1) * sms;
+    if (s.err == cudaSuccess) s.err = cudaDeviceGetAttribute(&s.sms, cudaDevAttrMultiProcessorCount, dev);
+    if (s.err == cudaSuccess) s.err = inv_configure({kM}, s.sms, &s.shape);
   });
-  if (s.err != cudaSuccess || !s.scratch || s.grid < 1) return CTAUX_ECUDA;
-  unsigned char* scratch = s.scratch;
-  void* args[] = {(void*)&d_a, &lda, (void*)&d_inv, &ld_inv, &m, &scratch, (void*)&d_logdet};
-  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_invert_noalloc, dim3(s.grid),
-                                                    dim3(256), args, 0,
-                                                    reinterpret_cast<cudaStream_t>(cuda_stream));
+  if (s.err != cudaSuccess || !s.scratch) return CTAUX_ECUDA;
+  InvView v{};
+  inv_layout(reinterpret_cast<double*>(s.scratch), kM, 1, v);
+  v.perm = reinterpret_cast<int*>(s.scratch + kPerm);
+  v.pcol = reinterpret_cast<int*>(s.scratch + kPcol);
+  v.used = reinterpret_cast<int8_t*>(s.scratch + kUsed);
+  v.status = reinterpret_cast<int*>(s.scratch + kStatus);
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
+  k_noalloc_load<<<m, 256, 0, st>>>(d_a, lda, m, v, s.scratch);
+  cudaError_t e = cudaSuccess;
+  launch_inverse(reinterpret_cast<const InvView*>(s.scratch + kView), reinterpret_cast<const int*>(s.scratch + kOrder),
+                 1, m, s.shape, st, &e);
+  if (e == cudaSuccess) {
+    k_noalloc_store<<<m, 256, 0, st>>>(d_inv, ld_inv, m, v, d_logdet);
+    e = cudaGetLastError();
+  }
   return e == cudaSuccess ? CTAUX_OK : CTAUX_ECUDA;
 }
