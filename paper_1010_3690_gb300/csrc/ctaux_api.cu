@@ -316,6 +316,11 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
     c.gamma = std::acosh(1.0 + cp.beta * cp.U * (double)cp.n_c / (2.0 * cp.K));
     c.dtau = cp.beta / (double)(cp.n_tau - 1);
     c.inv_dtau = (double)(cp.n_tau - 1) / cp.beta;
+    // 46 fraction bits, fewer where the table is so long that positions would pass 2^62
+    c.fx_bits = 46;
+    while (((long long)(cp.n_tau - 1) >> (62 - c.fx_bits)) != 0) --c.fx_bits;
+    c.fx_scale = std::ldexp(c.inv_dtau, c.fx_bits);
+    c.fx_beta = (long long)(cp.n_tau - 1) << c.fx_bits;
     for (int spin = 0; spin < 2; ++spin) {
       const double sig = spin == 0 ? 1.0 : -1.0;
       for (int dd = -2; dd <= 2; ++dd) {
@@ -341,17 +346,30 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
     c.n_anchors = P.n_anchors;
     const size_t ld = c.ld, K = cp.k_max;
     const size_t tab = (size_t)2 * cp.n_classes * cp.n_tau;
-    double* g0 = dalloc<double>(ctx, tab, &err);
+    double2* g0 = dalloc<double2>(ctx, tab, &err);
+    float2* g0f = sizeof(T) == 4 ? dalloc<float2>(ctx, tab, &err) : nullptr;
     int* dxc = dalloc<int>(ctx, (size_t)cp.n_c * cp.n_c, &err);
     double* cw = dalloc<double>(ctx, cp.n_classes, &err);
     if (err != cudaSuccess) return set_err(ctx, CTAUX_ENOMEM, "device allocation failed: %s", cudaGetErrorString(err));
-    CUDA_TRY(ctx, cudaMemcpy(g0, cp.g0_table, tab * sizeof(double), cudaMemcpyHostToDevice));
+    std::vector<double2> pairs(tab);
+    std::vector<float2> pairs_f(g0f ? tab : 0);
+    for (size_t r = 0; r < tab; r += cp.n_tau) {
+      const double* t = cp.g0_table + r;
+      for (int i = 0; i < cp.n_tau; ++i) {
+        const int i1 = std::min(i + 1, cp.n_tau - 1);   // the last step is 0
+        pairs[r + i] = make_double2(t[i], i1 == i ? 0.0 : t[i1] - t[i]);
+        if (g0f) pairs_f[r + i] = make_float2((float)t[i], i1 == i ? 0.f : (float)t[i1] - (float)t[i]);
+      }
+    }
+    CUDA_TRY(ctx, cudaMemcpy(g0, pairs.data(), tab * sizeof(double2), cudaMemcpyHostToDevice));
+    if (g0f) CUDA_TRY(ctx, cudaMemcpy(g0f, pairs_f.data(), tab * sizeof(float2), cudaMemcpyHostToDevice));
     CUDA_TRY(ctx, cudaMemcpy(dxc, cp.dx_class, (size_t)cp.n_c * cp.n_c * sizeof(int), cudaMemcpyHostToDevice));
     std::vector<double> w(cp.n_classes, 0.0);
     for (int x = 0; x < cp.n_c; ++x) w[cp.dx_class[x * cp.n_c + 0]] += 1.0;
     for (int k = 0; k < cp.n_classes; ++k) w[k] = w[k] > 0 ? 1.0 / (w[k] * P.n_anchors) : 0.0;
     CUDA_TRY(ctx, cudaMemcpy(cw, w.data(), w.size() * sizeof(double), cudaMemcpyHostToDevice));
     c.g0 = g0;
+    c.g0f = g0f;
     c.dx_class = dxc;
     c.class_weight = cw;
     for (int b = 0; b < 2; ++b) {

@@ -74,8 +74,12 @@ __global__ void __launch_bounds__(256) k_plan(Chain<T>* chains) {
 //   B[l][a] = G0(old_l, new_a)                 (G_{:,new} = N_ext [B; G0(new,new)])
 //   Gcol[n + a][b] = G0(new_a, new_b)          (accumulated onto by the prep products)
 //   N_ext[:, n + a] = e_{n+a}                  (s=0 columns of N_ext are unit vectors)
+constexpr int kGatherNew = 4;   // new vertices per thread and old vertex: one conversion of its time
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_gather(Chain<T>* chains) {
+  __shared__ long long ft[kMaxK];
+  __shared__ int sa[kMaxK];
   const Chain<T>& c = chains[blockIdx.z];
   const Dyn& d = *c.dyn;
   if (d.status) return;
@@ -84,26 +88,56 @@ __global__ void __launch_bounds__(256) k_gather(Chain<T>* chains) {
   const double* tau = c.tau[buf];
   const int* site = c.site[buf];
   T* Nb = c.N[buf][spin];
-  const long nC = (long)k_ins * n, nB = nC, nG = (long)k_ins * k_ins, nI = (long)m * k_ins;
-  const long total = nC + nB + nG + nI;
+  // Up to two values per thread the launch takes the latency of one evaluation
+  // after another, and g0_eval is the shorter chain (14.1 against 15.9 us with
+  // k_plan at n = 415, k = 64); with more the FP64 pipe bounds the kernel, and
+  // the times are converted once for 2 kGatherNew values (0.27 against
+  // 0.135 ms for 96 chains of n = 415).
+  const long nC = (long)k_ins * n;
+  const bool single = nC <= (long)gridDim.x * blockDim.x;
+  if (!single) {
+    for (int a = threadIdx.x; a < k_ins; a += blockDim.x) {
+      ft[a] = tau_fix(c, tau[n + a]);
+      sa[a] = site[n + a];
+    }
+    __syncthreads();
+  }
+  const long nP = single ? 2 * nC : (long)((k_ins + kGatherNew - 1) / kGatherNew) * n;
+  const long nG = (long)k_ins * k_ins, nI = (long)m * k_ins;
+  const long total = nP + nG + nI;
   for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (long)gridDim.x * blockDim.x) {
-    if (e < nC) {
-      const int a = (int)(e / n), l = (int)(e % n);
-      const double ev = c.ev[spin][c.s0[l] + 2];
-      c.Cpan[spin][(long)a * ld + l] =
-          (T)(g0_eval(c, spin, tau[n + a], site[n + a], tau[l], site[l]) * (ev - 1.0));
-    } else if (e < nC + nB) {
-      const long f = e - nC;
+    if (e < nP && single) {
+      const bool row = e < nC;
+      const long f = row ? e : e - nC;
       const int a = (int)(f / n), l = (int)(f % n);
-      c.Bpan[spin][(long)a * ld + l] = (T)g0_eval(c, spin, tau[l], site[l], tau[n + a], site[n + a]);
-    } else if (e < nC + nB + nG) {
-      const long f = e - nC - nB;
+      const int i = row ? n + a : l, j = row ? l : n + a;
+      const double g = g0_eval(c, spin, tau[i], site[i], tau[j], site[j]);
+      if (row) c.Cpan[spin][(long)a * ld + l] = (T)(g * (c.ev[spin][c.s0[l] + 2] - 1.0));
+      else c.Bpan[spin][(long)a * ld + l] = (T)g;
+    } else if (e < nP) {
+      const int a0 = (int)(e / n) * kGatherNew, l = (int)(e % n);
+      const double em1 = c.ev[spin][c.s0[l] + 2] - 1.0;
+      const long long fl = tau_fix(c, tau[l]);
+      const int sl = site[l];
+#pragma unroll
+      for (int q = 0; q < kGatherNew; ++q) {
+        const int a = a0 + q;
+        if (a >= k_ins) break;
+        const long long dt = ft[a] - fl;
+        double ga, gl;
+        if (!g0_fixed(c, g0_row(c, spin, sa[a], sl), dt, ga)) ga = g0_eval(c, spin, tau[n + a], sa[a], tau[l], sl);
+        if (!g0_fixed(c, g0_row(c, spin, sl, sa[a]), -dt, gl)) gl = g0_eval(c, spin, tau[l], sl, tau[n + a], sa[a]);
+        c.Cpan[spin][(long)a * ld + l] = (T)(ga * em1);
+        c.Bpan[spin][(long)a * ld + l] = (T)gl;
+      }
+    } else if (e < nP + nG) {
+      const long f = e - nP;
       const int b = (int)(f / k_ins), a = (int)(f % k_ins);
       c.Gcol[spin][(long)b * ld + n + a] =
           (T)g0_eval(c, spin, tau[n + a], site[n + a], tau[n + b], site[n + b]);
     } else {
-      const long f = e - nC - nB - nG;
+      const long f = e - nP - nG;
       const int a = (int)(f / m), i = (int)(f % m);
       Nb[(long)(n + a) * ld + i] = (i == n + a) ? (T)1 : (T)0;
     }

@@ -106,7 +106,7 @@ struct Chain {
   int kp;                    // mixed form: k_max rounded up to 32 (split operand row length)
   double tie_guard;          // mixed form: relative guard band of the FP64 re-evaluation (0 = off)
   double* N64[2];            // mixed form: FP64 N of a tie refresh [spin], ld x ld
-  const double* g0;          // [2][n_classes][n_tau]
+  const double2* g0;         // [2][n_classes][n_tau] (value, step to the next value; last step 0)
   const int* dx_class;       // [n_c][n_c]
   const double* class_weight;  // [n_classes] 1/(n_anchors * #sites of the class)
   T* N[2][2];                // [buf][spin]
@@ -168,6 +168,10 @@ struct Chain {
   double* Gmeas;             // last measurement
   TraceRec* trace;
   Dyn* dyn;
+  const float2* g0f;         // mixed form: the same rounded to float32, steps of the rounded values
+  double fx_scale;           // imaginary time -> fixed-point table position (tau_fix)
+  long long fx_beta;         // position of beta
+  int fx_bits;               // fraction bits of a position
 };
 
 // ----------------------------------------------------------------- Philox
@@ -219,12 +223,12 @@ __device__ __forceinline__ int move_of(double u_move, double p_insert, double p_
 // ------------------------------------------------------- G0 interpolation
 // Linear interpolation of a table row at 0 <= x <= beta; explicit _rn
 // operations keep the arithmetic free of FMA contraction.
-__device__ __forceinline__ double interp_row(const double* row, int n_tau, double inv_dtau, double x) {
+__device__ __forceinline__ double interp_row(const double2* row, int n_tau, double inv_dtau, double x) {
   const double pos = x * inv_dtau;
   const int idx = min(max((int)floor(pos), 0), n_tau - 2);
   const double f = pos - (double)idx;
-  const double g0 = __ldg(row + idx), g1 = __ldg(row + idx + 1);
-  return fma(f, g1 - g0, g0);
+  const double2 g = __ldg(row + idx);
+  return fma(f, g.y, g.x);
 }
 
 // G0_sigma(x_i - x_j, tau_i - tau_j): antiperiodic in tau; equal times take
@@ -236,21 +240,52 @@ __device__ __forceinline__ double g0_eval(const Chain<T>& c, int spin, double ti
                                           int xj) {
   const double dt = ti - tj;
   const int cls = __ldg(c.dx_class + xi * c.n_c + xj);
-  const double* row = c.g0 + ((size_t)spin * c.n_classes + cls) * c.n_tau;
+  const double2* row = c.g0 + ((size_t)spin * c.n_classes + cls) * c.n_tau;
   const bool neg = dt < 0.0;
   const double v = interp_row(row, c.n_tau, c.inv_dtau, neg ? dt + c.beta : dt);
-  if (dt == 0.0) return -__ldg(row + c.n_tau - 1);
+  if (dt == 0.0) return -__ldg(&row[c.n_tau - 1].x);
   return neg ? -v : v;
+}
+
+// The same value for kernels that evaluate many pairs: the times become
+// fixed-point table positions once per vertex (tau_fix), and a pair then costs
+// integer operations and two FP64 operations (the fraction and the fma) in
+// place of eleven; the FP64 pipe issues a warp's operation in 19 cycles and
+// bounds these kernels.  A position carries fx_bits <= 46 fraction bits, more
+// than float64 holds at the upper end of the table (41 bits at 4096 points),
+// and rounds once, so positions are ordered as the times are.
+template <typename T>
+__device__ __forceinline__ long long tau_fix(const Chain<T>& c, double tau) {
+  const double hi = tau * c.fx_scale;
+  return __double2ll_rn(hi) + __double2ll_rn(fma(tau, c.fx_scale, -hi));
+}
+
+template <typename T>
+__device__ __forceinline__ const double2* g0_row(const Chain<T>& c, int spin, int xi, int xj) {
+  return c.g0 + ((size_t)spin * c.n_classes + __ldg(c.dx_class + xi * c.n_c + xj)) * c.n_tau;
+}
+
+// v = G0 at position difference d; false when the positions are equal or lie
+// the full period apart (the caller takes g0_eval, which compares the times).
+template <typename T>
+__device__ __forceinline__ bool g0_fixed(const Chain<T>& c, const double2* row, long long d, double& v) {
+  const long long p = d < 0 ? d + c.fx_beta : d;
+  if ((unsigned long long)(p - 1) >= (unsigned long long)(c.fx_beta - 1)) return false;
+  const unsigned long long frac = (unsigned long long)p << (64 - c.fx_bits);
+  const double f = __longlong_as_double((long long)(0x3FF0000000000000ull | (frac >> 12))) - 1.0;
+  const double2 g = __ldg(row + (p >> c.fx_bits));
+  v = __longlong_as_double(__double_as_longlong(fma(f, g.y, g.x)) ^ (d & (long long)0x8000000000000000ull));
+  return true;
 }
 
 // Same interpolation in float32 (the mixed form's measurement): table entries
 // rounded to float, position and weights in float.
-__device__ __forceinline__ float interp_row_f(const double* row, int n_tau, float inv_dtau, float x) {
+__device__ __forceinline__ float interp_row_f(const float2* row, int n_tau, float inv_dtau, float x) {
   const float pos = x * inv_dtau;
   const int idx = min(max((int)floorf(pos), 0), n_tau - 2);
   const float f = pos - (float)idx;
-  const float g0 = (float)__ldg(row + idx), g1 = (float)__ldg(row + idx + 1);
-  return fmaf(f, g1 - g0, g0);
+  const float2 g = __ldg(row + idx);
+  return fmaf(f, g.y, g.x);
 }
 
 template <typename T>
@@ -258,10 +293,10 @@ __device__ __forceinline__ float g0_eval_f(const Chain<T>& c, int spin, float ti
                                            int xj) {
   const float dt = ti - tj;
   const int cls = __ldg(c.dx_class + xi * c.n_c + xj);
-  const double* row = c.g0 + ((size_t)spin * c.n_classes + cls) * c.n_tau;
+  const float2* row = c.g0f + ((size_t)spin * c.n_classes + cls) * c.n_tau;
   const bool neg = dt < 0.f;
   const float v = interp_row_f(row, c.n_tau, (float)c.inv_dtau, neg ? dt + (float)c.beta : dt);
-  if (dt == 0.f) return -(float)__ldg(row + c.n_tau - 1);
+  if (dt == 0.f) return -__ldg(&row[c.n_tau - 1].x);
   return neg ? -v : v;
 }
 

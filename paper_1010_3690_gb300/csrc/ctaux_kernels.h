@@ -204,7 +204,7 @@ template <typename T>
 void launch_reset_measure(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st);
 template <typename T>
 void launch_matsubara(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st);
-void launch_g0_matsubara(const double* table, int n_classes, int n_tau, double beta, int n_freq,
+void launch_g0_matsubara(const double2* table, int n_classes, int n_tau, double beta, int n_freq,
                          double2* out, cudaStream_t st);
 int tc_smem_bytes();
 cudaError_t configure_prep_tc();

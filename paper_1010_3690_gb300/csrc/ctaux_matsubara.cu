@@ -43,19 +43,19 @@ __device__ __forceinline__ double mats_w(int f, double beta) {
 // interpolant g of the table row, integrated by parts (e^{i w beta} = -1):
 //   -(g(beta-) + g(0+)) / (i w) + sum_j s_j (e^{i w t_{j+1}} - e^{i w t_j}) / w^2,
 // s_j the slope of interval j.  One thread per (spin, class, f).
-__global__ void k_g0_matsubara(const double* table, int n_classes, int n_tau, double beta,
+__global__ void k_g0_matsubara(const double2* table, int n_classes, int n_tau, double beta,
                                int n_freq, double2* out) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= 2 * n_classes * n_freq) return;
   const int f = e % n_freq, row = e / n_freq;  // row = spin * n_classes + class
-  const double* g = table + (size_t)row * n_tau;
+  const double2* g = table + (size_t)row * n_tau;
   const double w = mats_w(f, beta), h = beta / (double)(n_tau - 1);
   double re = 0.0, im = 0.0;
   double c0 = 1.0, s0 = 0.0;
   for (int j = 0; j + 1 < n_tau; ++j) {
     double s1, c1;
     sincos(w * (double)(j + 1) * h, &s1, &c1);
-    const double slope = (g[j + 1] - g[j]) / h;
+    const double slope = g[j].y / h;
     re += slope * (c1 - c0);
     im += slope * (s1 - s0);
     c0 = c1;
@@ -65,7 +65,7 @@ __global__ void k_g0_matsubara(const double* table, int n_classes, int n_tau, do
   re *= iw2;
   im *= iw2;
   // -(g(beta-) + g(0+)) / (i w) = i (g(beta-) + g(0+)) / w
-  im += (g[n_tau - 1] + g[0]) / w;
+  im += (g[n_tau - 1].x + g[0].x) / w;
   out[e] = make_double2(re, im);
 }
 
@@ -312,7 +312,7 @@ void launch_matsubara(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st)
   k_mats_G<T, 1><<<ls.persist_ctas, 256, 0, st>>>(dchains, nch);
 }
 
-void launch_g0_matsubara(const double* table, int n_classes, int n_tau, double beta, int n_freq,
+void launch_g0_matsubara(const double2* table, int n_classes, int n_tau, double beta, int n_freq,
                          double2* out, cudaStream_t st) {
   const int total = 2 * n_classes * n_freq;
   k_g0_matsubara<<<(total + 127) / 128, 128, 0, st>>>(table, n_classes, n_tau, beta, n_freq, out);
