@@ -346,23 +346,16 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
     c.n_anchors = P.n_anchors;
     const size_t ld = c.ld, K = cp.k_max;
     const size_t tab = (size_t)2 * cp.n_classes * cp.n_tau;
-    double2* g0 = dalloc<double2>(ctx, tab, &err);
-    float2* g0f = sizeof(T) == 4 ? dalloc<float2>(ctx, tab, &err) : nullptr;
+    // pairs, then the plain table, whose place the float32 pairs take in the mixed form
+    double2* g0 = reinterpret_cast<double2*>(dalloc<double>(ctx, 3 * tab, &err));
+    double* g0_plain = reinterpret_cast<double*>(g0 + tab);
+    float2* g0f = sizeof(T) == 4 ? reinterpret_cast<float2*>(g0_plain) : nullptr;
     int* dxc = dalloc<int>(ctx, (size_t)cp.n_c * cp.n_c, &err);
     double* cw = dalloc<double>(ctx, cp.n_classes, &err);
     if (err != cudaSuccess) return set_err(ctx, CTAUX_ENOMEM, "device allocation failed: %s", cudaGetErrorString(err));
-    std::vector<double2> pairs(tab);
-    std::vector<float2> pairs_f(g0f ? tab : 0);
-    for (size_t r = 0; r < tab; r += cp.n_tau) {
-      const double* t = cp.g0_table + r;
-      for (int i = 0; i < cp.n_tau; ++i) {
-        const int i1 = std::min(i + 1, cp.n_tau - 1);   // the last step is 0
-        pairs[r + i] = make_double2(t[i], i1 == i ? 0.0 : t[i1] - t[i]);
-        if (g0f) pairs_f[r + i] = make_float2((float)t[i], i1 == i ? 0.f : (float)t[i1] - (float)t[i]);
-      }
-    }
-    CUDA_TRY(ctx, cudaMemcpy(g0, pairs.data(), tab * sizeof(double2), cudaMemcpyHostToDevice));
-    if (g0f) CUDA_TRY(ctx, cudaMemcpy(g0f, pairs_f.data(), tab * sizeof(float2), cudaMemcpyHostToDevice));
+    CUDA_TRY(ctx, cudaMemcpy(g0_plain, cp.g0_table, tab * sizeof(double), cudaMemcpyHostToDevice));
+    launch_g0_pairs(g0_plain, cp.n_tau, (long)tab, g0, g0f, nullptr);
+    CUDA_TRY(ctx, cudaGetLastError());
     CUDA_TRY(ctx, cudaMemcpy(dxc, cp.dx_class, (size_t)cp.n_c * cp.n_c * sizeof(int), cudaMemcpyHostToDevice));
     std::vector<double> w(cp.n_classes, 0.0);
     for (int x = 0; x < cp.n_c; ++x) w[cp.dx_class[x * cp.n_c + 0]] += 1.0;

@@ -1471,6 +1471,26 @@ void launch_philox_test(uint64_t seed, uint32_t chain, int64_t t0, int count, in
   k_philox_test<<<(count + 255) / 256, 256, 0, st>>>(seed, chain, t0, count, purpose, out);
 }
 
+// ------------------------------------------------------------ G0 tables
+__global__ void k_g0_pairs(const double* plain, int n_tau, long entries, double2* g0) {
+  const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= entries) return;
+  const double v = plain[e];
+  g0[e] = make_double2(v, e % n_tau == n_tau - 1 ? 0.0 : plain[e + 1] - v);
+}
+__global__ void k_g0_pairs_f(const double2* g0, int n_tau, long entries, float2* g0f) {
+  const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= entries) return;
+  const float v = (float)g0[e].x;
+  g0f[e] = make_float2(v, e % n_tau == n_tau - 1 ? 0.f : (float)g0[e + 1].x - v);
+}
+
+void launch_g0_pairs(const double* plain, int n_tau, long entries, double2* g0, float2* g0f, cudaStream_t st) {
+  const unsigned blocks = (unsigned)((entries + 255) / 256);
+  k_g0_pairs<<<blocks, 256, 0, st>>>(plain, n_tau, entries, g0);
+  if (g0f) k_g0_pairs_f<<<blocks, 256, 0, st>>>(g0, n_tau, entries, g0f);
+}
+
 // ----------------------------------------------------------- launchers
 template <typename T>
 int lu_inverse_smem(const LaunchShape& ls) {

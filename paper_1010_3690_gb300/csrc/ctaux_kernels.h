@@ -204,6 +204,9 @@ template <typename T>
 void launch_reset_measure(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st);
 template <typename T>
 void launch_matsubara(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st);
+// (value, step to the next value) of every table entry, the last step of a row 0;
+// the same in float32 into g0f, unless null (it may take the plain table's place).
+void launch_g0_pairs(const double* plain, int n_tau, long entries, double2* g0, float2* g0f, cudaStream_t st);
 void launch_g0_matsubara(const double2* table, int n_classes, int n_tau, double beta, int n_freq,
                          double2* out, cudaStream_t st);
 int tc_smem_bytes();

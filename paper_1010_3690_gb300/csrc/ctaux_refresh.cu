@@ -24,7 +24,7 @@ __global__ void k_refresh_orders(const Chain<T>* chains, int n_chains, int only_
 
 // N^{-1} into X: kBuildCols columns by kBuildRows rows per CTA and unit, so that
 // a thread's conversion of its row's time serves kBuildCols entries.
-// Bounded by the FP64 pipe and the table gathers: 2.46 -> 1.1 ms at n = 6760 (both spins).
+// Bounded by the FP64 pipe and the table gathers: 2.46 -> 0.82 ms at n = 6760 (both spins).
 constexpr int kBuildCols = 8, kBuildRows = 1024;
 
 template <typename T>
