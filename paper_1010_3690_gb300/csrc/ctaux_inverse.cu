@@ -439,8 +439,13 @@ __global__ void __launch_bounds__(256) k_inv_cols(const InvView* views, const in
 // the accumulators into 64-bit integers first, so that the next tile's MMAs
 // run while it adds to X on the float64 pipe.  Per tile: 34 x 2 MMAs of 48
 // clocks (128 x 64 x 16, bound by shared-memory reads of A and B) against 8192
-// float64 additions, 19 clocks per warp.  Rank 32 takes about 9 us per tile
-// (the epilogue's float64 additions and loads), rank 128 about 9 us.
+// float64 additions, 19 clocks per warp.  X's loads and additions hide behind
+// the next tile's MMAs once the tile has been sent for (834 -> 740 us per rank-128
+// product at order 6760, both spins); what is left open is the emptying of the
+// accumulators, bound by the conversions to integers (740 -> 660 us with four of
+// them per element in place of six; 590 with none, where shared memory, reads for
+// the MMAs and writes of the bulk copies, is the bound).  Releasing the accumulators
+// group by group took 694: its shorter loads wait more often.
 constexpr int kUpdStages = 2, kUpdThreads = 576;
 constexpr int kUpdCols = 16;   // columns of an epilogue warp
 constexpr int kUpdStageBytes = oz::kImageA + oz::kImageB;
@@ -576,6 +581,11 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
       const bool load = row_ok && !(pci >= g.c0 && pci < cn);   // pivot rows start from zero
       const int ea = row_ok ? v.ea[i] - (WIDE ? 54 : 56) : 0;
       double* Xi = v.X + (size_t)jb * ld + i;
+      {   // the warp's share of X towards L2 while the products run, a 128-byte line per lane
+        const int pi = t.i0 + quarter * 32 + (lane & 1) * 16, pj = jb + (lane >> 1);
+        if (pi < t.m && pj < je)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(v.X + (size_t)pj * ld + pi));
+      }
       if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&accfull), q & 1))) {
         if (lane == 0) {
           err_s = 1;
