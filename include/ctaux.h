@@ -324,12 +324,14 @@ ctaux_status ctaux_autotune_k(ctaux_ctx *ctx, const int *candidates, int n_candi
                               int n_blocks, int *k_out, double *rate_out);
 
 /* Tile shapes of the CUDA-core products (the prep products, the flush of the
- * FP64 form, the measurement product).  Each product has CTAUX_TILE_VARIANTS
+ * FP64 form).  Each product has CTAUX_TILE_VARIANTS
  * compiled output-tile shapes; a table of one byte per (product, octave of the
  * chain's current order n, octave of its k_max),
  *   index = (product * 16 + min(floor(log2 n), 15)) * 9 + min(floor(log2 k_max), 8),
- * products 0 R~, 1 G_{old,new}, 2 G_{new,new}, 3 flush, 4 measurement, picks the
- * shape each chain uses (the table is read on the device for every chain's
+ * products 0 R~, 1 G_{old,new}, 2 G_{new,new}, 3 flush (4, the measurement product,
+ * has one shape: its entries are kept and have no effect; nor have those of 0, 1
+ * and 3 for FP64 chains of capacity + k_max 256 and more, whose products run on
+ * the tensor cores), picks the shape each chain uses (the table is read on the device for every chain's
  * current order, so chains of different sizes in one launch use different
  * shapes).  A new context starts with all zeros (the default shapes).
  * ctaux_autotune_tiles times the variants on the context's own chains: per

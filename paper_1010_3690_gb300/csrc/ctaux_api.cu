@@ -228,15 +228,15 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
   ls.kchunk = (sizeof(T) == 8) ? 32 : 128;
   // split-K partial tiles per (chain, spin): the most any product of the chain
   // can use at its capacity, at most kMaxPartials (device rule in gemm_items)
-  std::vector<size_t> kpart_of(ctx->chains.size(), 1), kpart_meas_of(ctx->chains.size(), 1);
+  std::vector<size_t> kpart_of(ctx->chains.size(), 1);
   for (size_t ci = 0; ci < ctx->chains.size(); ++ci) {
     const ctaux_chain_params& cp = ctx->chains[ci];
     const long cap_m = cp.capacity + cp.k_max, k = cp.k_max;
     // output rows and columns of each product at capacity (setup_gemm)
-    const long rows[PH_COUNT] = {k, cap_m, k, cap_m, cap_m};
-    const long cols[PH_COUNT] = {cap_m, k, k, cap_m, P.n_anchors};
+    const long rows[PH_MEAS] = {k, cap_m, k, cap_m};
+    const long cols[PH_MEAS] = {cap_m, k, k, cap_m};
     size_t need = 1;  // elements
-    for (int ph = 0; ph < PH_COUNT; ++ph)
+    for (int ph = 0; ph < PH_MEAS; ++ph)
       for (int v = 0; v < kTileVariants; ++v) {
         const GemmTile tl = tile_variant(sizeof(T) == 8, ph, v);
         const long tiles = ((rows[ph] + tl.bm - 1) / tl.bm) * ((cols[ph] + tl.bn - 1) / tl.bn);
@@ -245,7 +245,6 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
         if (ks > 1) {
           const size_t el = (size_t)std::min<long>(kMaxPartials, tiles * ks) * tl.bm * tl.bn;
           need = std::max(need, el);
-          if (ph == PH_MEAS) kpart_meas_of[ci] = std::max(kpart_meas_of[ci], el);
         }
       }
     kpart_of[ci] = need;
@@ -389,8 +388,8 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
       c.Mpts[spin] = dalloc<double>(ctx, (size_t)ls.meas_lchunks * P.n_anchors * cp.n_c * P.n_tau_bins, &err);
       c.kpart[spin] = dalloc<T>(ctx, kpart_of[ci], &err);
       c.ticket[spin] = dalloc<int>(ctx, kMaxPartials, &err);
-      c.kpart_meas[spin] = dalloc<T>(ctx, kpart_meas_of[ci], &err);
-      c.ticket_meas[spin] = dalloc<int>(ctx, kMaxPartials, &err);
+      c.vpart[spin] = dalloc<T>(ctx, meas_v_partials(c.cap_m, P.n_anchors, sizeof(T) == 8), &err);
+      c.vticket[spin] = dalloc<int>(ctx, meas_v_tickets(c.cap_m, P.n_anchors), &err);
     }
     c.gamma_lu = P.gamma_form == CTAUX_GAMMA_LU ? 1 : 0;
     c.kp = round_up(cp.k_max, 32);
@@ -1282,14 +1281,13 @@ ctaux_status ctaux_autotune_tiles(ctaux_ctx* ctx, int n_blocks, int8_t* table_ou
   const int nch = (int)ctx->chains.size();
   const bool mixed = is_mixed(ctx);
   // products this context launches on the CUDA cores, with the phase timer and
-  // work counter that measure them (0 prep, 1 flush, 2 measurement)
+  // work counter that measure them (0 prep, 1 flush)
   std::vector<std::pair<int, int>> prods;
   if (!(mixed && ctx->ls.prep_tc))
     for (int ph : {PH_RTILDE, PH_GCOL_OLD, PH_GCOL_NEW})
       if (ctx->ls.any_plain || ph == PH_GCOL_NEW) prods.push_back({ph, 0});
   if (!(mixed && ctx->ls.use_tc) && ctx->ls.any_plain) prods.push_back({PH_FLUSH, 1});
-  prods.push_back({PH_MEAS, 2});
-  const int timer_phase[3] = {1, 3, 5};
+  const int timer_phase[2] = {1, 3};
   // groups: (octave of the current order, octave of k_max) slots of the table
   std::vector<int> slot_pop(kTileOct * kTileKOct, 0);
   for (int c = 0; c < nch; ++c) {
@@ -1315,17 +1313,16 @@ ctaux_status ctaux_autotune_tiles(ctaux_ctx* ctx, int n_blocks, int8_t* table_ou
   auto score = [&](int kind, double* out) -> ctaux_status {
     ctaux_status r = ctaux_set_tile_table(ctx, table.data());
     if (r != CTAUX_OK) return r;
-    if ((r = ctaux_sweep(ctx, 1, kind == 2, ctx->last_stream)) != CTAUX_OK) return r;  // untimed
+    if ((r = ctaux_sweep(ctx, 1, 0, ctx->last_stream)) != CTAUX_OK) return r;  // untimed
     if ((r = ctaux_synchronize(ctx)) != CTAUX_OK) return r;
     double ms0[PhaseTimer::kPhases], ms1[PhaseTimer::kPhases], w0[7], w1[7];
     ctaux_get_phase_times(ctx, ms0, nullptr);
     ctaux_get_work(ctx, &w0[0], &w0[1], &w0[2], &w0[3], &w0[4], &w0[5], &w0[6]);
-    if ((r = ctaux_sweep(ctx, n_blocks, kind == 2, ctx->last_stream)) != CTAUX_OK) return r;
+    if ((r = ctaux_sweep(ctx, n_blocks, 0, ctx->last_stream)) != CTAUX_OK) return r;
     if ((r = ctaux_synchronize(ctx)) != CTAUX_OK) return r;
     ctaux_get_phase_times(ctx, ms1, nullptr);
     ctaux_get_work(ctx, &w1[0], &w1[1], &w1[2], &w1[3], &w1[4], &w1[5], &w1[6]);
-    const int wi = kind == 0 ? 0 : kind == 1 ? 1 : 4;
-    const double work = w1[wi] - w0[wi];
+    const double work = w1[kind] - w0[kind];
     const double ms = ms1[timer_phase[kind]] - ms0[timer_phase[kind]];
     *out = work > 0.0 ? ms / work : ms;
     return CTAUX_OK;

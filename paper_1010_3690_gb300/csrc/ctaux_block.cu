@@ -198,19 +198,13 @@ __device__ __forceinline__ bool setup_gemm(const Chain<T>& c, const Dyn& d, int 
       g.Cin.p = c.Gcol[spin] + n; g.Cin.rs = 1; g.Cin.cs = ld; g.has_cin = true;
       g.out = c.Gcol[spin] + n; g.out_rs = 1; g.out_cs = ld;
       break;
-    case PH_FLUSH:  // N'[a,b] = N[S_a,S_b] - Y[a,:] N[P,S_b]
+    default:  // PH_FLUSH: N'[a,b] = N[S_a,S_b] - Y[a,:] N[P,S_b]
       g.M = d.flush_noop ? 0 : d.n_new; g.Nn = d.n_new; g.Kk = d.k_acc;
       g.alpha = -1.0;
       g.A.p = c.Y[spin]; g.A.rs = 1; g.A.cs = ld;
       g.B.p = Nb; g.B.rs = 1; g.B.cs = ld; g.B.ri = c.P; g.B.ci = c.S;
       g.Cin.p = Nb; g.Cin.rs = 1; g.Cin.cs = ld; g.Cin.ri = c.S; g.Cin.ci = c.S; g.has_cin = true;
       g.out = c.N[1 - d.buf][spin]; g.out_rs = 1; g.out_cs = ld;
-      break;
-    default:  // measurement: v_b = N g_b
-      g.M = n; g.Nn = c.n_anchors; g.Kk = n;
-      g.A.p = Nb; g.A.rs = 1; g.A.cs = ld;
-      g.B.p = c.Mg[spin]; g.B.rs = 1; g.B.cs = ld;
-      g.out = c.Mv[spin]; g.out_rs = 1; g.out_cs = ld;
       break;
   }
   return g.M > 0 && g.Nn > 0;
@@ -327,10 +321,8 @@ __device__ __forceinline__ void gemm_item(const Chain<T>& c, const Dyn& d, int l
     __syncthreads();
   }
   if (nslices > 1) {
-    // the measurement product has partial tiles and tickets of its own: it
-    // may run beside a block's products
-    T* part = (PHASE == PH_MEAS ? c.kpart_meas[spin] : c.kpart[spin]) + (size_t)tile * nslices * GBM * GBN;
-    int* tickets = PHASE == PH_MEAS ? c.ticket_meas[spin] : c.ticket[spin];
+    T* part = c.kpart[spin] + (size_t)tile * nslices * GBM * GBN;
+    int* tickets = c.ticket[spin];
 #pragma unroll
     for (int a = 0; a < TM; ++a)
 #pragma unroll
@@ -385,7 +377,7 @@ __global__ void __launch_bounds__(256) k_gemm(Chain<T>* chains, int n_chains, in
   for (int ci = threadIdx.x; ci < n_chains; ci += blockDim.x) {
     int a, b, q, wd;
     const Chain<T>& c = chains[ci];
-    const bool other = c.sliced && PHASE != PH_GCOL_NEW && PHASE != PH_MEAS;   // ctaux_sliced.cu
+    const bool other = c.sliced && PHASE != PH_GCOL_NEW;   // ctaux_sliced.cu
     off[ci] = (!other && chain_tile_var(c, *c.dyn, PHASE) == V)
                   ? gemm_items<T, PHASE>(c, *c.dyn, kchunk, V, a, b, q, wd)
                   : 0;
@@ -417,8 +409,7 @@ int launch_gemm(Chain<T>* dchains, const LaunchShape& ls, int phase, cudaStream_
     case PH_RTILDE: launch_gemm_variants<T, PH_RTILDE>(dchains, ls, st); break;
     case PH_GCOL_OLD: launch_gemm_variants<T, PH_GCOL_OLD>(dchains, ls, st); break;
     case PH_GCOL_NEW: launch_gemm_variants<T, PH_GCOL_NEW>(dchains, ls, st); break;
-    case PH_FLUSH: launch_gemm_variants<T, PH_FLUSH>(dchains, ls, st); break;
-    default: launch_gemm_variants<T, PH_MEAS>(dchains, ls, st); break;
+    default: launch_gemm_variants<T, PH_FLUSH>(dchains, ls, st); break;
   }
   return __builtin_popcount(ls.tile_mask[phase]);
 }
@@ -1585,8 +1576,6 @@ cudaError_t configure_block_kernels(const LaunchShape& ls) {
   return e;
 }
 
-template int launch_gemm<double>(Chain<double>*, const LaunchShape&, int, cudaStream_t);
-template int launch_gemm<float>(Chain<float>*, const LaunchShape&, int, cudaStream_t);
 template void launch_block<double>(Chain<double>*, const LaunchShape&, cudaStream_t, PhaseTimer*,
                                    const TcMaps*, const BlockFork*);
 template void launch_block<float>(Chain<float>*, const LaunchShape&, cudaStream_t, PhaseTimer*,

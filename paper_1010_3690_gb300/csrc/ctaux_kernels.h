@@ -19,6 +19,40 @@ constexpr int kMeasChunk = 16;      // the shortest chunk (sizes the partial-sum
 constexpr int kMeasChunkMax = 32;
 __host__ __device__ inline int meas_chunk(int n) { return n <= 1024 ? kMeasChunk : kMeasChunkMax; }
 
+// Measurement product v_b = N g_b (k_meas_v): items of kMeasRows rows, up to
+// kMeasAnchors anchors and one slice of the columns.  The slices are narrow
+// where an order alone has few row blocks (order 415: 7 blocks x 7 slices for
+// each spin in float64), wide where partial sums would cost more than they
+// spread: float32, which is bound by its reads of N, four times as wide (96
+// uneven mixed chains: 0.40 -> 0.346 ms per measurement).  One float64 chain of
+// order 415, whose measurement runs beside the next block, takes 64 rather than
+// 32 columns: twice the CTAs slowed that block by half a percent.  They depend on
+// the order and the anchors only, so a chain gives the same bits alone or in a
+// batch.
+constexpr int kMeasRows = 64, kMeasAnchors = 8;
+__host__ __device__ inline int meas_v_groups(int anchors) { return (anchors + kMeasAnchors - 1) / kMeasAnchors; }
+__host__ __device__ inline int meas_v_width(int n, int anchors, bool fp64) {
+  return (n <= 1024 ? 64 : n <= 4096 ? 128 : n <= 16384 ? 256 : 512) * meas_v_groups(anchors) *
+         (fp64 ? 1 : 4);
+}
+__host__ __device__ inline int meas_v_slices(int n, int anchors, bool fp64) {
+  const int w = meas_v_width(n, anchors, fp64);
+  return (n + w - 1) / w;
+}
+// partial sums [slice][anchor][row] and tickets [row block][anchor group] of a spin
+inline size_t meas_v_partials(int cap, int anchors, bool fp64) {
+  size_t most = 1;   // the largest order of each width
+  for (int n : {1024, 4096, 16384, cap}) {
+    const int m = n < cap ? n : cap, s = meas_v_slices(m, anchors, fp64);
+    const size_t need = s > 1 ? (size_t)s * anchors * m : 1;
+    most = need > most ? need : most;
+  }
+  return most;
+}
+inline size_t meas_v_tickets(int cap, int anchors) {
+  return (size_t)((cap + kMeasRows - 1) / kMeasRows) * meas_v_groups(anchors);
+}
+
 // tensor-core flush (mixed form): 128 x 128 output tiles, K chunks of 16 float32;
 // the gathered N[S_m][S_n] input of a tile is staged as 128 column segments of
 // kTcNsRows source rows
@@ -41,16 +75,15 @@ enum { PH_RTILDE = 0, PH_GCOL_OLD = 1, PH_GCOL_NEW = 2, PH_FLUSH = 3, PH_MEAS = 
 
 // Output tile of each product (rows x columns, per thread TM x TN; 256
 // threads).  float64 (FP64-pipe bound, so padding costs time): skinny where
-// one dimension is the number of insertions (R~: rows, G_{old,new}: columns)
-// or of anchors (measurement product), 32 x 32 otherwise.  float32 (the
-// faster pipe makes re-reads of N and per-item overheads matter more): 64 x 64,
-// and 128 x 8 for the measurement product.
+// one dimension is the number of insertions (R~: rows, G_{old,new}: columns),
+// 32 x 32 otherwise.  float32 (the faster pipe makes re-reads of N and per-item
+// overheads matter more): 64 x 64.  The measurement product has a kernel of its
+// own (k_meas_v), without variants.
 struct GemmTile {
   int bm, bn, tm, tn;
 };
 constexpr GemmTile gemm_tile(bool fp64, int phase) {
-  return phase == PH_MEAS ? GemmTile{128, 8, 4, 1}
-         : !fp64          ? GemmTile{64, 64, 4, 4}
+  return !fp64                  ? GemmTile{64, 64, 4, 4}
          : phase == PH_RTILDE   ? GemmTile{16, 64, 1, 4}
          : phase == PH_GCOL_OLD ? GemmTile{64, 16, 4, 1}
                                 : GemmTile{32, 32, 2, 2};
@@ -62,7 +95,6 @@ constexpr GemmTile gemm_tile(bool fp64, int phase) {
 constexpr int kTileVariants = 3;
 constexpr GemmTile tile_variant(bool fp64, int phase, int v) {
   return v == 0 ? gemm_tile(fp64, phase)
-         : phase == PH_MEAS ? (v == 1 ? GemmTile{64, 8, 2, 1} : GemmTile{256, 8, 8, 1})
          : !fp64 ? (v == 1 ? GemmTile{32, 32, 2, 2} : GemmTile{128, 64, 8, 4})
          : phase == PH_RTILDE   ? (v == 1 ? GemmTile{32, 32, 2, 2} : GemmTile{16, 128, 1, 8})
          : phase == PH_GCOL_OLD ? (v == 1 ? GemmTile{32, 32, 2, 2} : GemmTile{128, 16, 8, 1})
@@ -182,8 +214,6 @@ void launch_block(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st, Pha
                   const TcMaps* maps, const BlockFork* fork = nullptr);
 template <typename T>
 cudaError_t configure_block_kernels(const LaunchShape& ls);
-template <typename T>
-int launch_gemm(Chain<T>* dchains, const LaunchShape& ls, int phase, cudaStream_t st);
 size_t refresh_work_doubles(int ld);
 size_t refresh_work_one(int ld);
 template <typename T>

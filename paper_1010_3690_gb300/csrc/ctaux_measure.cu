@@ -8,9 +8,9 @@
 // antiperiodic sign.  G_sigma(class(x_a), bin) is the average over anchors
 // and over the sites of a class.
 //
-// Steps: gather g_b[m] = G0(m, b) (k_meas_gather), v_b = N g_b (batched GEMM,
-// split over K), evaluate every point (k_meas_eval), reduce per class in a
-// fixed order and accumulate sums and squares (k_meas_accumulate).
+// Steps: gather g_b[m] = G0(m, b) (k_meas_gather), v_b = N g_b (k_meas_v),
+// evaluate every point (k_meas_eval), reduce per class in a fixed order and
+// accumulate sums and squares (k_meas_accumulate).
 #include "ctaux_dev.cuh"
 #include "ctaux_kernels.h"
 
@@ -46,6 +46,136 @@ __global__ void __launch_bounds__(256) k_meas_gather(Chain<T>* chains) {
   }
 }
 
+// v_b = N g_b.  A thread owns two adjacent rows and reads them of every eighth
+// column of its item's slice, each entry of N once for all anchors of the group
+// (a compile-time count: a padded anchor would hold the FP64 pipe like a real
+// one); the eight warps' sums and then the slices' add up in a fixed order, the
+// slices by the last to arrive.  float64 is bound by the FP64 pipe (19 clocks per
+// warp operation), float32 by reading N.  Against the tiled product (8 columns
+// wide: half of it padding at 4 anchors) the whole measurement takes, ms, 2 chains
+// of order 6760 4.52 -> 2.61, one of 2085 0.322 -> 0.202, 40 of up to 542 0.374 ->
+// 0.305; float32, one of order 6760, 0.52 -> 0.41.
+template <typename T> struct Pair;
+template <> struct Pair<double> { using type = double2; };
+template <> struct Pair<float> { using type = float2; };
+
+template <typename T>
+__device__ __forceinline__ int meas_v_items(const Chain<T>& c, const Dyn& d) {
+  if (d.status) return 0;
+  return 2 * ((d.n + kMeasRows - 1) / kMeasRows) * meas_v_groups(c.n_anchors) * meas_v_slices(d.n, c.n_anchors, sizeof(T) == 8);
+}
+
+// One item with NA anchors; sh: the staged g [column][anchor], then the warps' sums.
+template <int NA, typename T>
+__device__ __forceinline__ void meas_v_item(const Chain<T>& c, const Dyn& d, int spin, int block, int group,
+                                            int slice, int slices, T* sh, int* s_last) {
+  const int n = d.n, ld = c.ld, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int kLoads = 64 / sizeof(T), kMeasStageCols = 8 * kLoads;   // columns of a warp and of g at a time
+  static_assert(kMeasStageCols <= 8 * kMeasRows, "g fits in the warps' sums");
+  const int width = meas_v_width(n, c.n_anchors, sizeof(T) == 8);
+  const int j0 = slice * width, j1 = min(n, j0 + width), b0 = group * kMeasAnchors;
+  const int i = block * kMeasRows + 2 * lane;   // i + 1 < ld (even)
+  using P2 = typename Pair<T>::type;
+  const T* rows = c.N[d.buf][spin] + i;
+  const T* gp = c.Mg[spin] + (size_t)b0 * ld;
+  T acc[2][NA];
+#pragma unroll
+  for (int b = 0; b < NA; ++b) acc[0][b] = acc[1][b] = (T)0;
+  for (int js = j0; js < j1; js += kMeasStageCols) {
+    const int w = min(kMeasStageCols, j1 - js);
+    __syncthreads();   // the previous readers are done
+    for (int e = threadIdx.x; e < NA * kMeasStageCols; e += blockDim.x) {
+      const int q = e % kMeasStageCols, b = e / kMeasStageCols;
+      sh[q * NA + b] = q < w ? gp[(size_t)b * ld + js + q] : (T)0;
+    }
+    P2 x[kLoads];
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int q = warp + 8 * u;
+      x[u].x = x[u].y = (T)0;
+      if (i < n && q < w) x[u] = *reinterpret_cast<const P2*>(rows + (size_t)(js + q) * ld);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      if (warp + 8 * u >= w) break;   // the whole warp
+#pragma unroll
+      for (int b = 0; b < NA; ++b) {
+        const T g = sh[(warp + 8 * u) * NA + b];
+        acc[0][b] = fma(x[u].x, g, acc[0][b]);
+        acc[1][b] = fma(x[u].y, g, acc[1][b]);
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int b = 0; b < NA; ++b) {
+    sh[(warp * NA + b) * kMeasRows + 2 * lane] = acc[0][b];
+    sh[(warp * NA + b) * kMeasRows + 2 * lane + 1] = acc[1][b];
+  }
+  __syncthreads();
+  T* out = c.Mv[spin] + (size_t)b0 * ld;
+  T* part = c.vpart[spin] + (size_t)b0 * n;   // + (slice * A + b) * n + row
+  for (int e = threadIdx.x; e < NA * kMeasRows; e += blockDim.x) {
+    const int r = e % kMeasRows, b = e / kMeasRows, row = block * kMeasRows + r;
+    if (row >= n) continue;
+    T s = (T)0;
+#pragma unroll
+    for (int v = 0; v < 8; ++v) s += sh[(v * NA + b) * kMeasRows + r];
+    if (slices == 1) out[(size_t)b * ld + row] = s;
+    else part[((size_t)slice * c.n_anchors + b) * n + row] = s;
+  }
+  if (slices == 1) return;
+  __threadfence();
+  __syncthreads();
+  int* ticket = c.vticket[spin] + block * meas_v_groups(c.n_anchors) + group;
+  if (threadIdx.x == 0) *s_last = atomicAdd(ticket, 1) == slices - 1;
+  __syncthreads();
+  if (!*s_last) return;
+  __threadfence();
+  for (int e = threadIdx.x; e < NA * kMeasRows; e += blockDim.x) {
+    const int r = e % kMeasRows, b = e / kMeasRows, row = block * kMeasRows + r;
+    if (row >= n) continue;
+    T s = (T)0;
+    for (int v = 0; v < slices; ++v) s += __ldcg(part + ((size_t)v * c.n_anchors + b) * n + row);
+    out[(size_t)b * ld + row] = s;
+  }
+  if (threadIdx.x == 0) *ticket = 0;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256, 3) k_meas_v(Chain<T>* chains, int n_chains) {
+  __shared__ int off[kMaxChains + 1];
+  __shared__ T sh[8 * kMeasAnchors * kMeasRows];
+  __shared__ int s_last;
+  for (int ci = threadIdx.x; ci < n_chains; ci += blockDim.x) off[ci] = meas_v_items(chains[ci], *chains[ci].dyn);
+  __syncthreads();
+  block_exclusive_scan(off, n_chains);
+  const int total = off[n_chains];
+  for (int w = blockIdx.x; w < total; w += gridDim.x) {
+    const int ci = find_chain(off, n_chains, w);
+    const Chain<T>& c = chains[ci];
+    const Dyn& d = *c.dyn;
+    const int slices = meas_v_slices(d.n, c.n_anchors, sizeof(T) == 8), groups = meas_v_groups(c.n_anchors);
+    int l = w - off[ci];
+    const int slice = l % slices;
+    l /= slices;
+    const int group = l % groups;
+    l /= groups;
+    const int blocks = (d.n + kMeasRows - 1) / kMeasRows, block = l % blocks, spin = l / blocks;
+    switch (min(kMeasAnchors, c.n_anchors - group * kMeasAnchors)) {
+      case 1: meas_v_item<1>(c, d, spin, block, group, slice, slices, sh, &s_last); break;
+      case 2: meas_v_item<2>(c, d, spin, block, group, slice, slices, sh, &s_last); break;
+      case 3: meas_v_item<3>(c, d, spin, block, group, slice, slices, sh, &s_last); break;
+      case 4: meas_v_item<4>(c, d, spin, block, group, slice, slices, sh, &s_last); break;
+      case 5: meas_v_item<5>(c, d, spin, block, group, slice, slices, sh, &s_last); break;
+      case 6: meas_v_item<6>(c, d, spin, block, group, slice, slices, sh, &s_last); break;
+      case 7: meas_v_item<7>(c, d, spin, block, group, slice, slices, sh, &s_last); break;
+      default: meas_v_item<8>(c, d, spin, block, group, slice, slices, sh, &s_last); break;
+    }
+  }
+}
+
 // Evaluation of the estimator, persistent over the (chain, spin, point block,
 // vertex chunk) items of all chains; partial sums over a chunk of meas_chunk(n)
 // vertices go to Mpts[spin][chunk][(anchor * N_c + site) * B + bin].
@@ -60,7 +190,7 @@ __global__ void __launch_bounds__(256) k_meas_gather(Chain<T>* chains) {
 //
 // The FP64 pipe bounds the shared form: 2 + A operations per (point, vertex)
 // with fixed-point positions (tau_fix) where the times as float64 took 11 + A.
-// The measurement of two 100-site chains of order 4500: 6.05 -> 4.52 ms, of 96
+// The measurement of two 100-site chains of order 6760: 6.05 -> 4.52 ms, of 96
 // float32 chains (table as (value, step) pairs of float32, no conversions):
 // 0.47 -> 0.355 ms.
 constexpr int kMaxSharedAnchors = 16;
@@ -313,11 +443,11 @@ int launch_measure_head(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t s
 template <typename T>
 int launch_measure_tail(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st) {
   const int nch = ls.n_chains;
-  const int ng = launch_gemm<T>(dchains, ls, PH_MEAS, st);
+  k_meas_v<T><<<ls.persist_ctas, 256, 0, st>>>(dchains, nch);
   k_meas_eval<T><<<ls.persist_ctas, 256, 0, st>>>(dchains, nch);
   k_meas_accumulate<T><<<dim3(ls.meas_acc_blocks, 2, nch), 256, 0, st>>>(dchains);
   if (ls.mats) launch_matsubara<T>(dchains, ls, st);
-  return 2 + ng + (ls.mats ? 5 : 0);
+  return 3 + (ls.mats ? 5 : 0);
 }
 
 template <typename T>
