@@ -134,6 +134,7 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
       o.push_back(take(pl * 2 * yc * kSlicedImageB));
       o.push_back(take(rows * 2 * sizeof(int)));
       o.push_back(take(rows * 2 * sizeof(int)));
+      o.push_back(take(c.k_max * sizeof(int)));
       views[2 * ci + spin].pl = (int)pl;
       views[2 * ci + spin].yc = (int)yc;
       for (int pr = 0; pr < 2; ++pr) {
@@ -151,8 +152,8 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
       }
     }
   }
-  ls.any_sliced = 0;
-  ls.any_plain = 1;
+  ls.any_sliced = ls.any_sliced_y = 0;
+  ls.any_plain = ls.any_plain_y = 1;
   if (jobs.empty()) return CTAUX_OK;
   const size_t o_views = take(views.size() * sizeof(SlicedView)), o_jobs = take(jobs.size() * sizeof(SlicedJob)),
                o_exp = take(pool_exp * sizeof(int)), o_pool = take(pool);
@@ -166,13 +167,15 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
   ctx->allocations.push_back(mem);
   unsigned char* base = reinterpret_cast<unsigned char*>(mem);
   CUDA_TRY(ctx, cudaMemset(mem, 0, o_pool));   // the tickets start at zero
-  int plain = 0;
+  int plain = 0, plain_y = 0;
   for (int ci = 0; ci < nch; ++ci) {
     if (offs[2 * ci].empty()) {
-      plain = 1;
+      plain = plain_y = 1;
       continue;
     }
     hc[ci].sliced = 1;
+    hc[ci].sliced_y = hc[ci].k_max >= kSlicedYMinK;
+    (hc[ci].sliced_y ? ls.any_sliced_y : plain_y) = 1;
     for (int spin = 0; spin < 2; ++spin) {
       SlicedView& v = views[2 * ci + spin];
       const std::vector<size_t>& o = offs[2 * ci + spin];
@@ -186,6 +189,7 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
       v.xs = base + o[9];
       v.ye = reinterpret_cast<int*>(base + o[10]);
       v.xe = reinterpret_cast<int*>(base + o[11]);
+      v.qe = reinterpret_cast<int*>(base + o[12]);
     }
   }
   CUDA_TRY(ctx, cudaMemcpy(base + o_views, views.data(), views.size() * sizeof(SlicedView), cudaMemcpyHostToDevice));
@@ -200,6 +204,7 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
   for (const SlicedStrip& s : ctx->strips) p.max_jobs = std::max(p.max_jobs, s.count);
   ls.any_sliced = 1;
   ls.any_plain = plain;
+  ls.any_plain_y = plain_y;
   CUDA_TRY(ctx, configure_sliced(nch, p.max_jobs));
   return CTAUX_OK;
 }
@@ -496,7 +501,7 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
                              cudaMemcpyHostToDevice));
     ctx->tc_maps_dev = reinterpret_cast<TcMaps*>(dm);
   }
-  ls.any_plain = 1;
+  ls.any_plain = ls.any_plain_y = 1;
   if constexpr (sizeof(T) == 8) {
     const ctaux_status bs = build_sliced(ctx, hc);
     if (bs != CTAUX_OK) return bs;

@@ -415,22 +415,6 @@ int launch_gemm(Chain<T>* dchains, const LaunchShape& ls, int phase, cudaStream_
 }
 
 // ------------------------------------------------------------ proposals
-// Interacting Green's function of the block start, G0int(i, j) = G^0_{ij}
-// (Sec. III C: "G^0 is the interacting Green's function at step k=0"):
-// old columns from N by G = (N e^V - 1)/(e^V - 1) (Eq. NfromG), new (s=0)
-// columns from the prep product G_{:,new} = N_ext G0_{:,new}.  Evaluated in
-// the arithmetic type A of the form (float64, or float32 in the mixed form).
-template <typename A, typename T>
-__device__ __forceinline__ A g_int(const Chain<T>& c, const T* Nb, const T* Gc, int n_old, int spin,
-                                   int i, int j) {
-  if (j < n_old) {
-    const int k = c.s0[j] + 2;
-    return ((A)Nb[(long)j * c.ld + i] * (A)c.ev[spin][k] - (i == j ? (A)1 : (A)0)) *
-           (A)c.inv_em1[spin][k];
-  }
-  return (A)Gc[(long)(j - n_old) * c.ld + i];
-}
-
 // Select the idx-th set bit of a bitmask (one warp).
 __device__ __forceinline__ int select_bit(const uint32_t* mask, int n_words, int idx, int lane) {
   int base = 0;
@@ -1334,8 +1318,9 @@ __device__ __forceinline__ void split_tf32_y(float x, float& hi, float& lo) {
 }
 
 template <typename T, bool SPLIT>
-__device__ __forceinline__ int flush_y_items(const Dyn& d) {
-  if (d.status || d.flush_noop || (!SPLIT && d.k_acc == 0)) return 0;
+__device__ __forceinline__ int flush_y_items(const Chain<T>& c) {
+  const Dyn& d = *c.dyn;
+  if (c.sliced_y || d.status || d.flush_noop || (!SPLIT && d.k_acc == 0)) return 0;
   return 2 * ((d.n_new + kYRows - 1) / kYRows);
 }
 
@@ -1347,7 +1332,7 @@ __global__ void __launch_bounds__(256) k_flush_y(Chain<T>* chains, int n_chains)
   __shared__ int Ps[kMaxK];
   __shared__ int Si[kYRows];
   for (int ci = threadIdx.x; ci < n_chains; ci += blockDim.x)
-    off[ci] = flush_y_items<T, SPLIT>(*chains[ci].dyn);
+    off[ci] = flush_y_items<T, SPLIT>(chains[ci]);
   __syncthreads();
   block_exclusive_scan(off, n_chains);
   const int total = off[n_chains];
@@ -1541,10 +1526,17 @@ void launch_block(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st, Pha
   if (tc) {
     if constexpr (std::is_same<T, float>::value)
       k_flush_y<float, true><<<ls.persist_ctas, 256, 0, st>>>(dchains, nch);
+    pt->end(4, st, 2);
   } else {
-    k_flush_y<T, false><<<ls.persist_ctas, 256, 0, st>>>(dchains, nch);
+    int nk = 1;
+    if (ls.any_plain_y) {
+      k_flush_y<T, false><<<ls.persist_ctas, 256, 0, st>>>(dchains, nch);
+      nk += 1;
+    }
+    if constexpr (std::is_same<T, double>::value)
+      if (ls.any_sliced_y) nk += launch_sliced_y(dchains, ls, st);
+    pt->end(4, st, nk);
   }
-  pt->end(4, st, 2);
   pt->begin(3, st);
   if (tc) {
     if constexpr (std::is_same<T, float>::value) launch_flush_tc(dchains, maps, ls, st);

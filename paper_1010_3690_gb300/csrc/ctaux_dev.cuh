@@ -172,6 +172,7 @@ struct Chain {
   double fx_scale;           // imaginary time -> fixed-point table position (tau_fix)
   long long fx_beta;         // position of beta
   int fx_bits;               // fraction bits of a position
+  int sliced_y;              // with `sliced`: the flush coefficients Y too
 };
 
 // ----------------------------------------------------------------- Philox
@@ -298,6 +299,22 @@ __device__ __forceinline__ float g0_eval_f(const Chain<T>& c, int spin, float ti
   const float v = interp_row_f(row, c.n_tau, (float)c.inv_dtau, neg ? dt + (float)c.beta : dt);
   if (dt == 0.f) return -__ldg(&row[c.n_tau - 1].x);
   return neg ? -v : v;
+}
+
+// Interacting Green's function of the block start, G0int(i, j) = G^0_{ij}
+// (Sec. III C: "G^0 is the interacting Green's function at step k=0"):
+// old columns from N by G = (N e^V - 1)/(e^V - 1) (Eq. NfromG), new (s=0)
+// columns from the prep product G_{:,new} = N_ext G0_{:,new}.  Evaluated in
+// the arithmetic type A of the form (float64, or float32 in the mixed form).
+template <typename A, typename T>
+__device__ __forceinline__ A g_int(const Chain<T>& c, const T* Nb, const T* Gc, int n_old, int spin,
+                                   int i, int j) {
+  if (j < n_old) {
+    const int k = c.s0[j] + 2;
+    return ((A)Nb[(long)j * c.ld + i] * (A)c.ev[spin][k] - (i == j ? (A)1 : (A)0)) *
+           (A)c.inv_em1[spin][k];
+  }
+  return (A)Gc[(long)(j - n_old) * c.ld + i];
 }
 
 // ------------------------------------------------------------ work lists

@@ -142,6 +142,7 @@ struct LaunchShape {
   int max_cap;           // largest capacity + k_max of the chains
   int max_k;             // largest k_max of the context's chains
   int any_sliced, any_plain;  // float64 form: chains with sliced prep and flush products, and without
+  int any_sliced_y, any_plain_y;  // the same for the flush coefficients
   SlicedPlan sliced;
   int tile_mask[PH_COUNT];  // tile variants in the context's table, per product (bit v)
 };
@@ -260,6 +261,7 @@ cudaError_t configure_sliced(int n_chains, int max_jobs);
 // The prep products R~ and G_{old,new}, and the flush product, of the sliced
 // chains; return the kernels launched.
 int launch_sliced_prep(const Chain<double>* dchains, const LaunchShape& ls, cudaStream_t st);
+int launch_sliced_y(const Chain<double>* dchains, const LaunchShape& ls, cudaStream_t st);
 int launch_sliced_flush(const Chain<double>* dchains, const LaunchShape& ls, cudaStream_t st);
 void launch_philox_test(uint64_t seed, uint32_t chain, int64_t t0, int count, int purpose,
                         double* out, cudaStream_t st);

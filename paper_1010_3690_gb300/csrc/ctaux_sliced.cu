@@ -2,12 +2,15 @@
 // (sliced operands, ctaux_oz.cuh):
 //   prep 0: R~^T[j][a] = sum_{l<n} N[l][j] C[a][l]      -> N_ext[n + a][j]
 //   prep 1: G[i][a]    = sum_{l<n} N[i][l] B[l][a]      -> Gcol[a][i]
+//   Y:      Y[a][r]    = sum_q (G - 1)[S_a][P_q] Gamma^{-1}[q][r]
 //   flush:  N'[a][b]   = N[S_a][S_b] + sum_q (-Y)[a][q] N[P_q][S_b]
 // On the float64 pipe (1/64 of the float32 rate) these were nine tenths of a
-// block at 100 sites (per block of two chains: prep 86 -> 8.0 ms with the third
-// product, flush 69 -> 3.6 ms; at the 6 x 6 cluster 2.8 -> 0.47 and 1.33 -> 0.13).
+// block at 100 sites (per block of two chains: prep 86 -> 7.6 ms with the third
+// product, Y 2.67 -> 0.25, flush 69 -> 2.6; at the 6 x 6 cluster 2.8 -> 0.46, 0.16 ->
+// 0.06 and 1.33 -> 0.10).  Relative error of N after 8 blocks without recomputation,
+// 6 x 6 cluster, sliced / on the float64 pipe: 2.4e-14 / 4.5e-14.
 // Bound by the MMAs (68 per chunk of 32, 48 clocks each: shared-memory reads at
-// N = 64) and, exposed between parts, by the 6 conversions per output of the
+// N = 64) and, exposed between parts, by the 4 conversions per output of the
 // eight accumulators that fill the TMEM.  The matrix side (N, N^T or Y) is the tensor cores' A
 // operand, 128 rows per tile; the insertions or surviving columns are B, 64
 // per tile.  Long inner dimensions are summed in parts of 128: within a part
@@ -75,15 +78,16 @@ struct Balance {
   __device__ __forceinline__ double of(int s) const { return s > 0 ? up : s < 0 ? down : 1.0; }
 };
 
-// Sixteen rows x 128 inner elements whose rows are strided (element (r, k) at
-// src[k ks + r]), times scale[k] (may be null), zero for k >= kn and r >= rn: staged in shared memory, then a
-// thread per row and 16-byte chunk.  256 threads.
+// Sixteen rows x 128 inner elements val(k, r), zero for k >= kn and r >= rn, into
+// images of ROWS rows: staged in shared memory, then a thread per row and 16-byte
+// chunk.  256 threads.
 struct StageRows {
   double xs[128][17];
   int mxs[16];
 };
-__device__ __forceinline__ void slice_strided(StageRows& st, const double* src, size_t ks, int rn, int kn, const double* scale,
-                                              unsigned char* img, int r_in_image, int* exps, int exp_stride) {
+template <int ROWS, class F>
+__device__ __forceinline__ void slice_rows(StageRows& st, int rn, int kn, F val, unsigned char* img, int r_in_image,
+                                           int* exps, int exp_stride) {
   const int r = threadIdx.x & 15, ch = threadIdx.x >> 4;
   __syncthreads();   // the previous unit's readers are done
   if (threadIdx.x < 16) st.mxs[r] = 0;
@@ -92,8 +96,7 @@ __device__ __forceinline__ void slice_strided(StageRows& st, const double* src, 
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const int k = ch + 16 * q;
-    double x = k < kn && r < rn ? src[(size_t)k * ks + r] : 0.0;
-    if (scale) x *= scale[k];
+    const double x = k < kn && r < rn ? val(k, r) : 0.0;
     st.xs[k][r] = x;
     mx = max(mx, oz::exp_field((uint32_t)__double2hiint(x)));
   }
@@ -104,7 +107,7 @@ __device__ __forceinline__ void slice_strided(StageRows& st, const double* src, 
     long long y[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) y[t] = oz::biased_digits(st.xs[ch * 8 + t][r], mx);
-    oz::store_chunk(img + (size_t)(ch >> 2) * oz::kImageA + oz::chunk_offset(r_in_image + r, ch & 3), oz::kRowsA, y);
+    oz::store_chunk(img + (size_t)(ch >> 2) * oz::kSlices * ROWS * 64 + oz::chunk_offset(r_in_image + r, ch & 3), ROWS, y);
   }
   if (r < rn && ch == 0) exps[(size_t)r * exp_stride] = oz::row_exponent(mx);
 }
@@ -180,9 +183,11 @@ __global__ void __launch_bounds__(256) k_slice_n(const Chain<double>* chains, co
         if (lane == 0) exps[(size_t)r * pl + p] = oz::row_exponent(mx);
       }
     } else {
-      for (int p = 0; p < parts; ++p)
-        slice_strided(st, N + (size_t)p * 128 * c.ld + r0, (size_t)c.ld, n - r0, n - p * 128, nullptr,
-                      img + (size_t)p * 4 * oz::kImageA, r0 & 127, exps + p, pl);
+      for (int p = 0; p < parts; ++p) {
+        const double* src = N + (size_t)p * 128 * c.ld + r0;
+        slice_rows<oz::kRowsA>(st, n - r0, n - p * 128, [&](int k, int r) { return src[(size_t)k * c.ld + r]; },
+                               img + (size_t)p * 4 * oz::kImageA, r0 & 127, exps + p, pl);
+      }
     }
   }
 }
@@ -213,8 +218,13 @@ __global__ void __launch_bounds__(256) k_slice_flush(const Chain<double>* chains
       __syncthreads();
       for (int q = threadIdx.x; q < kMaxK; q += blockDim.x) ys[q] = q < ka ? -bal.of(c.s0[c.P[q]]) : 0.0;
       for (int p = 0; p * 128 < ka; ++p)   // starts with a barrier
-        slice_strided(st, c.Y[spin] + (size_t)p * 128 * c.ld + r0, (size_t)c.ld, nn - r0, ka - p * 128, ys + p * 128,
-                      v.ys + ((size_t)(r0 >> 7) * v.yc + p * 4) * oz::kImageA, r0 & 127, v.ye + (size_t)r0 * 2 + p, 2);
+      {
+        const double* src = c.Y[spin] + (size_t)p * 128 * c.ld + r0;
+        slice_rows<oz::kRowsA>(st, nn - r0, ka - p * 128,
+                               [&](int k, int r) { return src[(size_t)k * c.ld + r] * ys[p * 128 + k]; },
+                               v.ys + ((size_t)(r0 >> 7) * v.yc + p * 4) * oz::kImageA, r0 & 127,
+                               v.ye + (size_t)r0 * 2 + p, 2);
+      }
     } else {
       const double* N = c.N[d.buf][spin];
       const Balance bal(c, spin, false);
@@ -233,6 +243,102 @@ __global__ void __launch_bounds__(256) k_slice_flush(const Chain<double>* chains
             store_four(v.xs + ((size_t)(r >> 6) * v.yc + p * 4) * oz::kImageB, oz::kRowsB, oz::kImageB, r & 63, lane, x, mx);
           if (lane == 0) v.xe[(size_t)r * 2 + p] = oz::row_exponent(mx);
         }
+      }
+    }
+  }
+}
+
+// Balance of Y's inner index: the columns of G - 1 and the rows of Gamma^{-1} carry
+// a slot's e^V inversely (a factor of 400 between the spins at K = 1; without a
+// balance N lost three digits there in a block), and Gamma^{-1} is graded where it is
+// nearly singular.  Column q is scaled by the power of two that brings its largest
+// element and that of row q to the same size.  A CTA per q.
+__global__ void __launch_bounds__(256) k_balance_y(const Chain<double>* chains, int n_chains, const SlicedView* views) {
+  __shared__ int off[kMaxChains + 1], most[2];
+  for (int ci = threadIdx.x; ci < n_chains; ci += blockDim.x)
+    off[ci] = chains[ci].sliced_y && flush_rows(chains[ci]) ? 2 * chains[ci].dyn->k_acc : 0;
+  __syncthreads();
+  block_exclusive_scan(off, n_chains);
+  const int total = off[n_chains];
+  for (int u = blockIdx.x; u < total; u += gridDim.x) {
+    const int ci = find_chain(off, n_chains, u);
+    const Chain<double>& c = chains[ci];
+    const Dyn& d = *c.dyn;
+    const int l = u - off[ci], spin = l & 1, q = l >> 1, nn = d.n_new, ka = d.k_acc;
+    if (threadIdx.x < 2) most[threadIdx.x] = 0;
+    __syncthreads();
+    const double *N = c.N[d.buf][spin], *Gc = c.Gcol[spin], *Gi = c.Ginv[spin] + (size_t)q * (c.k_max + 1);
+    const int j = c.P[q];
+    int mg = 0, mi = 0;
+#pragma unroll 4
+    for (int a = threadIdx.x; a < nn; a += blockDim.x) {
+      const int i = c.S[a];
+      mg = max(mg, oz::exp_field((uint32_t)__double2hiint(g_int<double>(c, N, Gc, d.n, spin, i, j) - (i == j ? 1.0 : 0.0))));
+    }
+    for (int r = threadIdx.x; r < ka; r += blockDim.x) mi = max(mi, oz::exp_field((uint32_t)__double2hiint(Gi[r])));
+    mg = __reduce_max_sync(0xffffffffu, mg);
+    mi = __reduce_max_sync(0xffffffffu, mi);
+    if ((threadIdx.x & 31) == 0) {
+      atomicMax(&most[0], mg);
+      atomicMax(&most[1], mi);
+    }
+    __syncthreads();
+    mg = most[0];
+    mi = most[1];
+    // zero, subnormal and non-finite rows and columns stay as they are
+    if (threadIdx.x == 0) views[2 * ci + spin].qe[q] = mg == 0 || mg == 0x7ff || mi == 0 || mi == 0x7ff ? 0 : (mi - mg) / 2;
+    __syncthreads();   // both read before the next unit clears them
+  }
+}
+
+// G - 1 at the surviving rows and touched columns (16 rows per CTA unit) and the
+// columns of Gamma^{-1} (16 per CTA unit) of every chain, in the images of -Y and
+// N[P, S], which follow once Y is there.
+__global__ void __launch_bounds__(256) k_slice_y(const Chain<double>* chains, int n_chains, const SlicedView* views) {
+  __shared__ int off[kMaxChains + 1];
+  __shared__ StageRows st;
+  __shared__ int ps[kMaxK], si[16];
+  __shared__ double bs[kMaxK];
+  for (int ci = threadIdx.x; ci < n_chains; ci += blockDim.x) {
+    const int nn = chains[ci].sliced_y ? flush_rows(chains[ci]) : 0;
+    off[ci] = nn ? 2 * ((nn + 15) / 16 + (chains[ci].dyn->k_acc + 15) / 16) : 0;
+  }
+  __syncthreads();
+  block_exclusive_scan(off, n_chains);
+  const int total = off[n_chains];
+  for (int u = blockIdx.x; u < total; u += gridDim.x) {
+    const int ci = find_chain(off, n_chains, u);
+    const Chain<double>& c = chains[ci];
+    const Dyn& d = *c.dyn;
+    const int l = u - off[ci], spin = l & 1, nn = d.n_new, ka = d.k_acc, rb = (nn + 15) / 16;
+    const bool rows = (l >> 1) < rb;
+    const int r0 = (rows ? l >> 1 : (l >> 1) - rb) * 16;
+    const SlicedView& v = views[2 * ci + spin];
+    __syncthreads();
+    for (int q = threadIdx.x; q < ka; q += blockDim.x) {
+      ps[q] = c.P[q];
+      // |qe| <= 1023: a power of two within the normal range, or next to it
+      bs[q] = __hiloint2double((1023 + max(-1022, min(1023, rows ? v.qe[q] : -v.qe[q]))) << 20, 0);
+    }
+    if (rows) {
+      if (threadIdx.x < 16) si[threadIdx.x] = r0 + threadIdx.x < nn ? c.S[r0 + threadIdx.x] : 0;
+    }
+    for (int p = 0; p * 128 < ka; ++p) {   // starts with a barrier
+      if (rows) {
+        const double *N = c.N[d.buf][spin], *Gc = c.Gcol[spin];
+        slice_rows<oz::kRowsA>(st, nn - r0, ka - p * 128,
+                               [&](int k, int r) {
+                                 const int i = si[r], j = ps[p * 128 + k];
+                                 return (g_int<double>(c, N, Gc, d.n, spin, i, j) - (i == j ? 1.0 : 0.0)) * bs[p * 128 + k];
+                               },
+                               v.ys + ((size_t)(r0 >> 7) * v.yc + p * 4) * oz::kImageA, r0 & 127,
+                               v.ye + (size_t)r0 * 2 + p, 2);
+      } else {
+        const double* Gi = c.Ginv[spin] + (size_t)p * 128 * (c.k_max + 1) + r0;
+        slice_rows<oz::kRowsB>(st, ka - r0, ka - p * 128,
+                               [&](int k, int r) { return Gi[(size_t)k * (c.k_max + 1) + r] * bs[p * 128 + k]; },
+                               v.xs + ((size_t)(r0 >> 6) * v.yc + p * 4) * oz::kImageB, r0 & 63,
+                               v.xe + (size_t)r0 * 2 + p, 2);
       }
     }
   }
@@ -322,6 +428,39 @@ struct FlushSrc {
     t.eb = v.xe + (size_t)t.n0 * 2;
     t.es_a = t.es_b = 2;
     t.prod = t.tile = t.slice = 0;
+    t.slices = 1;
+    return t;
+  }
+};
+
+struct YSrc {
+  const Chain<double>* chains;
+  const SlicedView* views;
+  int n;
+  __device__ __forceinline__ int count(int i) const {
+    const int nn = chains[i].sliced_y ? flush_rows(chains[i]) : 0;
+    return nn ? 2 * ((nn + 127) / 128) * ((chains[i].dyn->k_acc + 63) / 64) : 0;
+  }
+  __device__ __forceinline__ ProdItem item(int i, int l) const {
+    const Dyn& d = *chains[i].dyn;
+    ProdItem t;
+    t.ci = i;
+    t.M = d.n_new;
+    t.N = d.k_acc;
+    const int tm = (t.M + 127) / 128, tn = (t.N + 63) / 64;
+    t.spin = l / (tm * tn);
+    l -= t.spin * tm * tn;
+    const SlicedView& v = views[2 * i + t.spin];
+    t.m0 = (l / tn) * 128;
+    t.n0 = (l % tn) * 64;
+    t.chunks = (d.k_acc + oz::kK - 1) / oz::kK;
+    t.a = v.ys + (size_t)(t.m0 >> 7) * v.yc * oz::kImageA;
+    t.b = v.xs + (size_t)(t.n0 >> 6) * v.yc * oz::kImageB;
+    t.ea = v.ye + (size_t)t.m0 * 2;
+    t.eb = v.xe + (size_t)t.n0 * 2;
+    t.es_a = t.es_b = 2;
+    t.prod = 2;
+    t.tile = t.slice = 0;
     t.slices = 1;
     return t;
   }
@@ -509,7 +648,9 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src) {
         for (int e = 0; e < kProdCols; ++e)
           if (t.n0 + cl + e < t.N) out[(size_t)(t.n0 + cl + e) * ld] = z[e];
       } else {
-        double* out = t.prod == 0 ? c.N[d.buf][t.spin] + (size_t)i * ld + d.n : c.Gcol[t.spin] + i;
+        double* out = t.prod == 0   ? c.N[d.buf][t.spin] + (size_t)i * ld + d.n
+                      : t.prod == 1 ? c.Gcol[t.spin] + i
+                                    : c.Y[t.spin] + i;
         const size_t cs = t.prod == 0 ? 1 : (size_t)ld;
 #pragma unroll
         for (int e = 0; e < kProdCols; ++e)
@@ -531,6 +672,7 @@ cudaError_t configure_sliced(int n_chains, int max_jobs) {
   const cudaFuncAttribute dyn = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e = cudaFuncSetAttribute(k_sliced_product<PrepSrc, false>, dyn, prod_smem(max_jobs));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_slice_n, dyn, (int)sizeof(int) * (max_jobs + 1));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sliced_product<YSrc, false>, dyn, prod_smem(n_chains));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sliced_product<FlushSrc, true>, dyn, prod_smem(n_chains));
   return e;
 }
@@ -548,6 +690,14 @@ int launch_sliced_prep(const Chain<double>* dchains, const LaunchShape& ls, cuda
     k_sliced_product<PrepSrc, false><<<ls.tc_ctas, kProdThreads, prod_smem(sp.count), st>>>(src);
   }
   return n;
+}
+
+int launch_sliced_y(const Chain<double>* dchains, const LaunchShape& ls, cudaStream_t st) {
+  k_balance_y<<<ls.persist_ctas, 256, 0, st>>>(dchains, ls.n_chains, ls.sliced.views);
+  k_slice_y<<<ls.persist_ctas, 256, 0, st>>>(dchains, ls.n_chains, ls.sliced.views);
+  const YSrc src{dchains, ls.sliced.views, ls.n_chains};
+  k_sliced_product<YSrc, false><<<ls.tc_ctas, kProdThreads, prod_smem(ls.n_chains), st>>>(src);
+  return 3;
 }
 
 int launch_sliced_flush(const Chain<double>* dchains, const LaunchShape& ls, cudaStream_t st) {

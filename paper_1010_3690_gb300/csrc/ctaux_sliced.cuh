@@ -15,6 +15,7 @@ struct SlicedView {
   unsigned char* ys;      // -Y rows: [128 rows][chunk] images
   unsigned char* xs;      // N[P, S] columns: [64 rows][chunk] images
   int *ye, *xe;           // exponents, [row][2]
+  int* qe;                // balance of Y's inner index, exponents
   double* part[2];        // split-K partial tiles of the prep products (128 x 64)
   int* ticket[2];         // arrivals per tile and epilogue warp
   int pl;                 // parts of the inner dimension at the capacity
@@ -73,6 +74,11 @@ inline size_t sliced_partials(int cap, int k) {
 // 212 / 220 at 200, 435 / 410 at 300, 513 / 451 at 415; in batches the float64
 // pipe saturates, so that the line lies below the crossover of one chain.
 constexpr int kSlicedMinOrder = 256;
+// k_max from which a sliced chain's flush coefficients Y are a sliced product too:
+// us per block of the flush support, float64 pipe against sliced, 53 / 71 for 40
+// chains of k_max 32, 37.3 / 36.4 for one of 64 at order 415, 164 / 57 for one of 128
+// at order 2085, 2670 / 254 for two of 256 at order 6760.
+constexpr int kSlicedYMinK = 64;
 // Bytes of the strip pool, unless one job needs more.
 constexpr size_t kSlicedPool = (size_t)8 << 30;
 

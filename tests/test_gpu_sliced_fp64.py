@@ -59,3 +59,22 @@ def test_sliced_products_of_a_block_at_tile_edges(n0, k):
         for spin in (0, 1):
             No = oc.N(spin)
             np.testing.assert_allclose(ctx.get_N(0, spin), No, rtol=1e-9, atol=1e-10 * np.abs(No).max())
+
+
+@pytest.mark.parametrize("K,n0,k", [(1.0, 130, 64), (256.0, 200, 160), (16.0, 257, 256)])
+def test_sliced_flush_coefficients_in_the_lu_form(K, n0, k):
+    """Y = (G - 1) Gamma^{-1} with Gamma kept as L U, at weak and strong e^V."""
+    ch = configs.cube8(K=K, k_max=k, capacity=n0 + 2 * k + 64)
+    cfg = configs.synthetic_configuration(ch, n0, seed=n0)
+    oc = oracle_for(ch, p_insert=0.45, p_flip=0.1)
+    oc.set_config(cfg["tau"], cfg["site"], cfg["s"], cfg["birth"], cfg["t"])
+    with pk.Context([ch], trace_capacity=2 * k, refresh_every=0, p_insert=0.45, p_flip=0.1,
+                    gamma_form=pk.ctaux.CTAUX_GAMMA_LU) as ctx:
+        ctx.set_config(0, **cfg)
+        tol = max(1e-10, 64 * 2.0**-52 * max(np.linalg.cond(oc.N(spin)) for spin in (0, 1)))
+        ctx.sweep(2)
+        ctx.synchronize()
+        compare_traces(ctx.trace(0), oc.run(2 * k), tol)
+        for spin in (0, 1):
+            No = oc.N(spin)
+            np.testing.assert_allclose(ctx.get_N(0, spin), No, rtol=tol, atol=tol * np.abs(No).max())
