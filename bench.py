@@ -63,17 +63,10 @@ WORKLOADS = {
 }
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the
-# dominant kernel, per unit of work, from an ncu capture of the same kernel on a
-# smaller case (profiles/k_refresh_cube100_traffic.md).  The refresh reads and
-# writes its float64 work matrix X (8 m^2 bytes per spin, far above L2 at these
-# orders) once per 32-column panel, so its traffic grows as m^3: the capture at
-# m = 4000 (one chain, both spins, 66.1 GB) gives bytes per m^3, scaled to a
-# launch by the sum of m^3 over the chains it refreshes.  An entry is removed
-# when its kernel changes.
-DRAM_TRAFFIC = {
-    ("cube100", "fp64", "refresh"): (32925212672 + 33162264064) / 4000.0 ** 3,
-    ("cube100", "mixed_df64", "refresh"): (32591805952 + 33272619776) / 4000.0 ** 3,
-}
+# dominant kernel per unit of work (sum of m^3 over the chains), from an ncu
+# capture of the same kernel on a smaller case.  An entry is removed when its
+# kernel changes; the recomputation's went with the elimination it was taken of.
+DRAM_TRAFFIC = {}
 
 
 def workload(name, K=None, k_max=None, chain_id=0, n_chains=None):
@@ -414,8 +407,9 @@ def main():
     ap.add_argument("--warmup", type=int, default=5)
     ap.add_argument("--impl", choices=["ours", "reference"], default="ours")
     ap.add_argument("--precision", choices=["both", "fp64", "mixed", "mixed_df64"], default="both",
-                    help="both = fp64, mixed and mixed_df64 (the mixed form with its refresh "
-                         "eliminating in double-float on the float32 pipe)")
+                    help="both = fp64, mixed and mixed_df64 (the mixed form with the "
+                         "refresh_df64 parameter set, which has no effect any more: the refresh "
+                         "keeps float64 accuracy on the tensor cores in every form)")
     ap.add_argument("--workload", default="cube100", choices=sorted(WORKLOADS))
     ap.add_argument("--K", type=float, default=None)
     ap.add_argument("--k-max", dest="k_max", type=int, default=None)
@@ -708,12 +702,17 @@ def measure_form(args, pk, torch, dist, chains, meta, refresh, form, local, worl
     fp64_peak = peaks["bf16_tflops"] * NOMINAL["fp64"] / NOMINAL["bf16"]
     fp32_peak = 152 * 128 * 2 * 2.07e9 / 1e12     # 152 SMs x 128 FP32 lanes x FMA x 2.07 GHz
     tf32x3_peak = peaks["bf16_tflops"] * NOMINAL["tf32"] / NOMINAL["bf16"] / 3.0
+    # float64 products as 34 float16 products of sliced operands
+    sliced_peak = peaks["bf16_tflops"] / 34.0
+    sliced_src = f"sliced float64 = bf16 {peak_kind} / 34 digit products"
     alu_peak = fp64_peak if precision == pk.CTAUX_FP64 else fp32_peak
     alu_src = (f"FP64 = bf16 {peak_kind} x 1.25/2250" if precision == pk.CTAUX_FP64
                else "FP32 = 152 SMs x 128 lanes x 2 x 2.07 GHz")
     dw = {k: work1[k] - work0[k] for k in work1}
     n_sm = min(152, len(chains))   # one CTA (one SM) per chain for the Gamma growth
     elem = 8 if precision == pk.CTAUX_FP64 else 4
+    # float64 prep and flush run on the tensor cores from this capacity on (ctaux_sliced.cuh)
+    sliced = min(c.capacity + c.k_max for c in chains) >= 256
 
     def roof(phase):
         sec = phase_ms[phase] / 1e3
@@ -724,6 +723,8 @@ def measure_form(args, pk, torch, dist, chains, meta, refresh, form, local, worl
             if precision == pk.CTAUX_MIXED:
                 r.update(bound="tensor", peak=tf32x3_peak,
                          peak_source=f"3xTF32 = bf16 {peak_kind} x 1100/2250 / 3 products")
+            elif sliced:
+                r.update(bound="tensor", peak=sliced_peak, peak_source=sliced_src)
             else:
                 r.update(bound="alu", peak=alu_peak, peak_source=alu_src)
             return r
@@ -738,6 +739,8 @@ def measure_form(args, pk, torch, dist, chains, meta, refresh, form, local, worl
                 # product on the CUDA cores
                 r.update(bound="tensor", peak=tf32x3_peak,
                          peak_source=f"3xTF32 = bf16 {peak_kind} x 1100/2250 / 3 products")
+            elif sliced:
+                r.update(bound="tensor", peak=sliced_peak, peak_source=sliced_src)
             else:
                 r.update(bound="alu", peak=alu_peak, peak_source=alu_src)
             return r
@@ -753,16 +756,8 @@ def measure_form(args, pk, torch, dist, chains, meta, refresh, form, local, worl
                         unit="TFLOP/s",
                         peak_source=alu_src + " (estimator flops, interpolations not counted)")
         if nm == "refresh":
-            if form == "mixed_df64":
-                # one compensated double-float multiply-add of the trailing update
-                # is 12 float32 operations (TwoProd 2, cross terms 2, TwoSum 6, 2 adds)
-                return dict(bound="alu", achieved=dw["refresh_flop"] / sec / 1e12,
-                            peak=fp32_peak / 12.0, unit="TFLOP/s",
-                            peak_source="double-float = FP32 peak / 12 float32 operations per "
-                                        "multiply-add (2 m^3 per spin)")
-            return dict(bound="alu", achieved=dw["refresh_flop"] / sec / 1e12, peak=fp64_peak,
-                        unit="TFLOP/s",
-                        peak_source=f"FP64 = bf16 {peak_kind} x 1.25/2250 (2 m^3 per spin)")
+            return dict(bound="tensor", achieved=dw["refresh_flop"] / sec / 1e12, peak=sliced_peak,
+                        unit="TFLOP/s", peak_source=sliced_src + " (2 m^3 per spin)")
         # plan/gather and flush support: latency-bound, no algorithmic roofline
         return dict(bound="latency", achieved=None, peak=None, unit=None, peak_source=None)
 
