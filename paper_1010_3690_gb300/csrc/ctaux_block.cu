@@ -75,6 +75,7 @@ __global__ void __launch_bounds__(256) k_plan(Chain<T>* chains) {
 //   Gcol[n + a][b] = G0(new_a, new_b)          (accumulated onto by the prep products)
 //   N_ext[:, n + a] = e_{n+a}                  (s=0 columns of N_ext are unit vectors)
 constexpr int kGatherNew = 4;   // new vertices per thread and old vertex: one conversion of its time
+constexpr int kGatherSmall = 4096;   // pairs of a panel evaluated directly
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_gather(Chain<T>* chains) {
@@ -88,13 +89,14 @@ __global__ void __launch_bounds__(256) k_gather(Chain<T>* chains) {
   const double* tau = c.tau[buf];
   const int* site = c.site[buf];
   T* Nb = c.N[buf][spin];
-  // Up to two values per thread the launch takes the latency of one evaluation
-  // after another, and g0_eval is the shorter chain (14.1 against 15.9 us with
-  // k_plan at n = 415, k = 64); with more the FP64 pipe bounds the kernel, and
-  // the times are converted once for 2 kGatherNew values (0.27 against
-  // 0.135 ms for 96 chains of n = 415).
+  // Small panels take the latency of one evaluation after another, and g0_eval is
+  // the shorter chain (with k_plan 13.7 against 17.4 us at n = 30, k = 8); in large
+  // ones the FP64 pipe bounds the kernel, and the times are converted once for 2
+  // kGatherNew values (0.27 against 0.135 ms for 96 chains of n = 415, k = 64; one
+  // such chain alone 14.1 against 15.9 us).  The line depends on the chain's own
+  // sizes only: it gives the same bits alone or in a batch.
   const long nC = (long)k_ins * n;
-  const bool single = nC <= (long)gridDim.x * blockDim.x;
+  const bool single = nC <= kGatherSmall;
   if (!single) {
     for (int a = threadIdx.x; a < k_ins; a += blockDim.x) {
       ft[a] = tau_fix(c, tau[n + a]);

@@ -33,7 +33,7 @@ def edge_chain(n_tau, n, k):
     return ch, cfg
 
 
-# n * k: a block's panels with at most two values per thread of the gather, and more
+# n * k: panels of up to 4096 pairs, which the gather evaluates directly, and more
 @pytest.mark.parametrize("n,k", [(90, 32), (700, 128)])
 @pytest.mark.parametrize("n_tau", [2, 5, 1024, 131073])
 def test_edge_times(n_tau, n, k):
