@@ -330,8 +330,8 @@ ctaux_status ctaux_autotune_k(ctaux_ctx *ctx, const int *candidates, int n_candi
  *   index = (product * 16 + min(floor(log2 n), 15)) * 9 + min(floor(log2 k_max), 8),
  * products 0 R~, 1 G_{old,new}, 2 G_{new,new}, 3 flush (4, the measurement product,
  * has one shape: its entries are kept and have no effect; nor have those of 0, 1
- * and 3 for FP64 chains of capacity + k_max 256 and more, whose products run on
- * the tensor cores), picks the shape each chain uses (the table is read on the device for every chain's
+ * and 3 for FP64 chains of capacity + k_max 256 and more, and of 2 with a k_max of
+ * 128 and more too, whose products run on the tensor cores), picks the shape each chain uses (the table is read on the device for every chain's
  * current order, so chains of different sizes in one launch use different
  * shapes).  A new context starts with all zeros (the default shapes).
  * ctaux_autotune_tiles times the variants on the context's own chains: per

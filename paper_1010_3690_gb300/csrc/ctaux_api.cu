@@ -135,6 +135,13 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
       o.push_back(take(rows * 2 * sizeof(int)));
       o.push_back(take(rows * 2 * sizeof(int)));
       o.push_back(take(c.k_max * sizeof(int)));
+      if (c.k_max >= kSlicedNewMinK) {
+        const size_t gt = (size_t)((c.k_max + 127) / 128) * ((c.k_max + 63) / 64);
+        o.push_back(take((c.k_max + 127) / 128 * pl * 4 * kSlicedImageA));
+        o.push_back(take((c.k_max + 127) / 128 * 128 * pl * sizeof(int)));
+        o.push_back(take(gt * sliced_new_slices(c.cap_m) * 8192 * sizeof(double)));
+        o.push_back(take(gt * 16 * sizeof(int)));
+      }
       views[2 * ci + spin].pl = (int)pl;
       views[2 * ci + spin].yc = (int)yc;
       for (int pr = 0; pr < 2; ++pr) {
@@ -152,8 +159,8 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
       }
     }
   }
-  ls.any_sliced = ls.any_sliced_y = 0;
-  ls.any_plain = ls.any_plain_y = 1;
+  ls.any_sliced = ls.any_sliced_y = ls.any_sliced_new = 0;
+  ls.any_plain = ls.any_plain_y = ls.any_plain_new = 1;
   if (jobs.empty()) return CTAUX_OK;
   const size_t o_views = take(views.size() * sizeof(SlicedView)), o_jobs = take(jobs.size() * sizeof(SlicedJob)),
                o_exp = take(pool_exp * sizeof(int)), o_pool = take(pool);
@@ -167,15 +174,17 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
   ctx->allocations.push_back(mem);
   unsigned char* base = reinterpret_cast<unsigned char*>(mem);
   CUDA_TRY(ctx, cudaMemset(mem, 0, o_pool));   // the tickets start at zero
-  int plain = 0, plain_y = 0;
+  int plain = 0, plain_y = 0, plain_new = 0;
   for (int ci = 0; ci < nch; ++ci) {
     if (offs[2 * ci].empty()) {
-      plain = plain_y = 1;
+      plain = plain_y = plain_new = 1;
       continue;
     }
     hc[ci].sliced = 1;
     hc[ci].sliced_y = hc[ci].k_max >= kSlicedYMinK;
     (hc[ci].sliced_y ? ls.any_sliced_y : plain_y) = 1;
+    hc[ci].sliced_new = hc[ci].k_max >= kSlicedNewMinK;
+    (hc[ci].sliced_new ? ls.any_sliced_new : plain_new) = 1;
     for (int spin = 0; spin < 2; ++spin) {
       SlicedView& v = views[2 * ci + spin];
       const std::vector<size_t>& o = offs[2 * ci + spin];
@@ -190,6 +199,12 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
       v.ye = reinterpret_cast<int*>(base + o[10]);
       v.xe = reinterpret_cast<int*>(base + o[11]);
       v.qe = reinterpret_cast<int*>(base + o[12]);
+      if (o.size() > 13) {
+        v.gs = base + o[13];
+        v.ge = reinterpret_cast<int*>(base + o[14]);
+        v.gpart = reinterpret_cast<double*>(base + o[15]);
+        v.gticket = reinterpret_cast<int*>(base + o[16]);
+      }
     }
   }
   CUDA_TRY(ctx, cudaMemcpy(base + o_views, views.data(), views.size() * sizeof(SlicedView), cudaMemcpyHostToDevice));
@@ -205,6 +220,7 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
   ls.any_sliced = 1;
   ls.any_plain = plain;
   ls.any_plain_y = plain_y;
+  ls.any_plain_new = plain_new;
   CUDA_TRY(ctx, configure_sliced(nch, p.max_jobs));
   return CTAUX_OK;
 }
@@ -501,7 +517,7 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
                              cudaMemcpyHostToDevice));
     ctx->tc_maps_dev = reinterpret_cast<TcMaps*>(dm);
   }
-  ls.any_plain = ls.any_plain_y = 1;
+  ls.any_plain = ls.any_plain_y = ls.any_plain_new = 1;
   if constexpr (sizeof(T) == 8) {
     const ctaux_status bs = build_sliced(ctx, hc);
     if (bs != CTAUX_OK) return bs;
@@ -1290,7 +1306,7 @@ ctaux_status ctaux_autotune_tiles(ctaux_ctx* ctx, int n_blocks, int8_t* table_ou
   std::vector<std::pair<int, int>> prods;
   if (!(mixed && ctx->ls.prep_tc))
     for (int ph : {PH_RTILDE, PH_GCOL_OLD, PH_GCOL_NEW})
-      if (ctx->ls.any_plain || ph == PH_GCOL_NEW) prods.push_back({ph, 0});
+      if (ph == PH_GCOL_NEW ? ctx->ls.any_plain_new : ctx->ls.any_plain) prods.push_back({ph, 0});
   if (!(mixed && ctx->ls.use_tc) && ctx->ls.any_plain) prods.push_back({PH_FLUSH, 1});
   const int timer_phase[2] = {1, 3};
   // groups: (octave of the current order, octave of k_max) slots of the table

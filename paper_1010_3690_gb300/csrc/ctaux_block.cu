@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(256) k_gemm(Chain<T>* chains, int n_chains, in
   for (int ci = threadIdx.x; ci < n_chains; ci += blockDim.x) {
     int a, b, q, wd;
     const Chain<T>& c = chains[ci];
-    const bool other = c.sliced && PHASE != PH_GCOL_NEW;   // ctaux_sliced.cu
+    const bool other = PHASE == PH_GCOL_NEW ? c.sliced_new : c.sliced;   // ctaux_sliced.cu
     off[ci] = (!other && chain_tile_var(c, *c.dyn, PHASE) == V)
                   ? gemm_items<T, PHASE>(c, *c.dyn, kchunk, V, a, b, q, wd)
                   : 0;
@@ -1497,7 +1497,7 @@ void launch_block(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st, Pha
     }
     if constexpr (std::is_same<T, double>::value)
       if (ls.any_sliced) nk += launch_sliced_prep(dchains, ls, st);
-    nk += launch_gemm<T>(dchains, ls, PH_GCOL_NEW, st);
+    if (ls.any_plain_new) nk += launch_gemm<T>(dchains, ls, PH_GCOL_NEW, st);
     pt->end(1, st, nk);
   }
   if (fork) {

@@ -172,7 +172,7 @@ struct Chain {
   double fx_scale;           // imaginary time -> fixed-point table position (tau_fix)
   long long fx_beta;         // position of beta
   int fx_bits;               // fraction bits of a position
-  int sliced_y;              // with `sliced`: the flush coefficients Y too
+  int sliced_y, sliced_new;  // with `sliced`: the flush coefficients Y too, and G_{new,new}
 };
 
 // ----------------------------------------------------------------- Philox

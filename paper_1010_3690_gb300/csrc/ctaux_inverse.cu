@@ -27,8 +27,8 @@
 //
 // One chain (two matrices), ms per recomputation, against the float64-pipe
 // elimination with a grid barrier per column that this replaces: 2.8 -> 1.2 at
-// order 431, 44 -> 9.6 at 2000, 1150 -> 108 at 6800 (where 1.06 TFLOP/s of
-// float64 was the bound; now 12 TFLOP/s).
+// order 431, 44 -> 8.0 at 2000, 1150 -> 79 at 6800 (where 1.06 TFLOP/s of
+// float64 was the bound; now 16 TFLOP/s).
 #include <cooperative_groups.h>
 
 #include "ctaux_dev.cuh"

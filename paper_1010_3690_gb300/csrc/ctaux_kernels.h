@@ -143,6 +143,7 @@ struct LaunchShape {
   int max_k;             // largest k_max of the context's chains
   int any_sliced, any_plain;  // float64 form: chains with sliced prep and flush products, and without
   int any_sliced_y, any_plain_y;  // the same for the flush coefficients
+  int any_sliced_new, any_plain_new;  // and for G_{new,new}
   SlicedPlan sliced;
   int tile_mask[PH_COUNT];  // tile variants in the context's table, per product (bit v)
 };

@@ -2,13 +2,13 @@
 // (sliced operands, ctaux_oz.cuh):
 //   prep 0: R~^T[j][a] = sum_{l<n} N[l][j] C[a][l]      -> N_ext[n + a][j]
 //   prep 1: G[i][a]    = sum_{l<n} N[i][l] B[l][a]      -> Gcol[a][i]
+//   prep 2: G[n+a][b]  = sum_{l<n} C[a][l] G[l][b] + G0 -> Gcol[b][n + a]
 //   Y:      Y[a][r]    = sum_q (G - 1)[S_a][P_q] Gamma^{-1}[q][r]
 //   flush:  N'[a][b]   = N[S_a][S_b] + sum_q (-Y)[a][q] N[P_q][S_b]
 // On the float64 pipe (1/64 of the float32 rate) these were nine tenths of a
-// block at 100 sites (per block of two chains: prep 86 -> 7.6 ms with the third
-// product, Y 2.67 -> 0.25, flush 69 -> 2.6; at the 6 x 6 cluster 2.8 -> 0.46, 0.16 ->
-// 0.06 and 1.33 -> 0.10).  Relative error of N after 8 blocks without recomputation,
-// 6 x 6 cluster, sliced / on the float64 pipe: 2.4e-14 / 4.5e-14.
+// block at 100 sites (per block of two chains: prep 86 -> 5.8 ms, Y 2.67 -> 0.25, flush 69 -> 2.6; at the
+// 6 x 6 cluster 2.8 -> 0.41, 0.16 -> 0.06 and 1.33 -> 0.10).  Relative error of N after 8 blocks without recomputation,
+// 6 x 6 cluster, sliced / on the float64 pipe: 2.1e-14 / 4.5e-14.
 // Bound by the MMAs (68 per chunk of 32, 48 clocks each: shared-memory reads at
 // N = 64) and, exposed between parts, by the 4 conversions per output of the
 // eight accumulators that fill the TMEM.  The matrix side (N, N^T or Y) is the tensor cores' A
@@ -146,6 +146,36 @@ __global__ void __launch_bounds__(256) k_slice_panels(const Chain<double>* chain
     const int mx = max_field4(x);
     store_four(v.cs[prod] + ((size_t)(a >> 6) * v.pl + p) * 4 * oz::kImageB, oz::kRowsB, oz::kImageB, a & 63, lane, x, mx);
     if (lane == 0) v.ce[prod][(size_t)a * v.pl + p] = oz::row_exponent(mx);
+  }
+}
+
+// The columns of G_{old,new} of every chain, a warp per (column, part); their inner
+// index is balanced against C's.
+__global__ void __launch_bounds__(256) k_slice_g(const Chain<double>* chains, int n_chains, const SlicedView* views) {
+  __shared__ int off[kMaxChains + 1];
+  for (int ci = threadIdx.x; ci < n_chains; ci += blockDim.x) {
+    const Dyn& d = *chains[ci].dyn;
+    off[ci] = d.status || !chains[ci].sliced_new ? 0 : 2 * ((d.k_ins + 7) / 8) * ((d.n + 127) / 128);
+  }
+  __syncthreads();
+  block_exclusive_scan(off, n_chains);
+  const int total = off[n_chains], warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int u = blockIdx.x; u < total; u += gridDim.x) {
+    const int ci = find_chain(off, n_chains, u);
+    const Chain<double>& c = chains[ci];
+    const int n = c.dyn->n, k_ins = c.dyn->k_ins, parts = (n + 127) / 128;
+    int l = u - off[ci];
+    const int p = l % parts;
+    l /= parts;
+    const int spin = l & 1, b = (l >> 1) * 8 + warp;
+    if (b >= k_ins) continue;
+    const SlicedView& v = views[2 * ci + spin];
+    double x[4];
+    load_four(c.Gcol[spin] + (size_t)b * c.ld, p, lane, n, x);
+    balance_four(x, c, Balance(c, spin, false), p, lane, n);
+    const int mx = max_field4(x);
+    store_four(v.gs + ((size_t)(b >> 7) * v.pl + p) * 4 * oz::kImageA, oz::kRowsA, oz::kImageA, b & 127, lane, x, mx);
+    if (lane == 0) v.ge[(size_t)b * v.pl + p] = oz::row_exponent(mx);
   }
 }
 
@@ -402,6 +432,43 @@ struct PrepSrc {
   }
 };
 
+// G_{new,new}: rows are the columns b of G_{old,new}, columns the rows a of C.
+struct NewSrc {
+  const Chain<double>* chains;
+  const SlicedView* views;
+  int n;
+  __device__ __forceinline__ int count(int i) const {
+    const Dyn& d = *chains[i].dyn;
+    if (!chains[i].sliced_new || d.status || d.k_ins == 0 || d.n == 0) return 0;
+    return 2 * ((d.k_ins + 127) / 128) * ((d.k_ins + 63) / 64) * sliced_new_slices(d.n);
+  }
+  __device__ __forceinline__ ProdItem item(int i, int l) const {
+    const Dyn& d = *chains[i].dyn;
+    ProdItem t;
+    t.ci = i;
+    t.spin = l & 1;
+    l >>= 1;
+    const SlicedView& v = views[2 * i + t.spin];
+    t.prod = 3;
+    t.M = t.N = d.k_ins;
+    t.slices = sliced_new_slices(d.n);
+    const int ct = (t.N + 63) / 64, parts = (d.n + 127) / 128;
+    t.slice = l % t.slices;
+    t.tile = l / t.slices;
+    const int r = t.tile / ct, c = t.tile % ct;
+    const int p0 = (int)((long)parts * t.slice / t.slices), p1 = (int)((long)parts * (t.slice + 1) / t.slices);
+    t.m0 = r * 128;
+    t.n0 = c * 64;
+    t.chunks = min(p1 * 4, (d.n + oz::kK - 1) / oz::kK) - p0 * 4;
+    t.a = v.gs + ((size_t)r * v.pl + p0) * 4 * oz::kImageA;
+    t.b = v.cs[0] + ((size_t)c * v.pl + p0) * 4 * oz::kImageB;
+    t.ea = v.ge + (size_t)t.m0 * v.pl + p0;
+    t.eb = v.ce[0] + (size_t)t.n0 * v.pl + p0;
+    t.es_a = t.es_b = v.pl;
+    return t;
+  }
+};
+
 struct FlushSrc {
   const Chain<double>* chains;
   const SlicedView* views;
@@ -622,12 +689,12 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src) {
         if (t.slices > 1) {   // partial tiles, added in slice order by the last to arrive
           const SlicedView& v = src.views[2 * t.ci + t.spin];
           // (a warp's 32 x 16 share of the tile by itself: no barrier)
-          double* part = v.part[t.prod] + (size_t)t.tile * t.slices * 8192 + cl * 128 + rl;
+          double* part = (t.prod == 3 ? v.gpart : v.part[t.prod]) + (size_t)t.tile * t.slices * 8192 + cl * 128 + rl;
 #pragma unroll
           for (int e = 0; e < kProdCols; ++e) part[(size_t)t.slice * 8192 + e * 128] = z[e];
           __threadfence();
           __syncwarp();
-          int* ticket = v.ticket[t.prod] + t.tile * 16 + warp - 2;
+          int* ticket = (t.prod == 3 ? v.gticket : v.ticket[t.prod]) + t.tile * 16 + warp - 2;
           int arrived = 0;
           if (lane == 0) arrived = atomicAdd(ticket, 1);
           if (__shfl_sync(0xffffffffu, arrived, 0) != t.slices - 1) continue;
@@ -650,8 +717,14 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src) {
       } else {
         double* out = t.prod == 0   ? c.N[d.buf][t.spin] + (size_t)i * ld + d.n
                       : t.prod == 1 ? c.Gcol[t.spin] + i
-                                    : c.Y[t.spin] + i;
-        const size_t cs = t.prod == 0 ? 1 : (size_t)ld;
+                      : t.prod == 2 ? c.Y[t.spin] + i
+                                    : c.Gcol[t.spin] + (size_t)i * ld + d.n;
+        const size_t cs = t.prod == 0 || t.prod == 3 ? 1 : (size_t)ld;
+        if (t.prod == 3) {   // onto G0(new, new)
+#pragma unroll
+          for (int e = 0; e < kProdCols; ++e)
+            if (t.n0 + cl + e < t.N) z[e] += out[t.n0 + cl + e];
+        }
 #pragma unroll
         for (int e = 0; e < kProdCols; ++e)
           if (t.n0 + cl + e < t.N) out[(size_t)(t.n0 + cl + e) * cs] = z[e];
@@ -672,6 +745,7 @@ cudaError_t configure_sliced(int n_chains, int max_jobs) {
   const cudaFuncAttribute dyn = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e = cudaFuncSetAttribute(k_sliced_product<PrepSrc, false>, dyn, prod_smem(max_jobs));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_slice_n, dyn, (int)sizeof(int) * (max_jobs + 1));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sliced_product<NewSrc, false>, dyn, prod_smem(n_chains));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sliced_product<YSrc, false>, dyn, prod_smem(n_chains));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sliced_product<FlushSrc, true>, dyn, prod_smem(n_chains));
   return e;
@@ -688,6 +762,12 @@ int launch_sliced_prep(const Chain<double>* dchains, const LaunchShape& ls, cuda
                                                                          p.pool_exp);
     const PrepSrc src{dchains, p.views, jobs, sp.count, p.pool, p.pool_exp};
     k_sliced_product<PrepSrc, false><<<ls.tc_ctas, kProdThreads, prod_smem(sp.count), st>>>(src);
+  }
+  if (ls.any_sliced_new) {
+    k_slice_g<<<ls.persist_ctas, 256, 0, st>>>(dchains, ls.n_chains, p.views);
+    const NewSrc src{dchains, p.views, ls.n_chains};
+    k_sliced_product<NewSrc, false><<<ls.tc_ctas, kProdThreads, prod_smem(ls.n_chains), st>>>(src);
+    n += 2;
   }
   return n;
 }

@@ -16,6 +16,10 @@ struct SlicedView {
   unsigned char* xs;      // N[P, S] columns: [64 rows][chunk] images
   int *ye, *xe;           // exponents, [row][2]
   int* qe;                // balance of Y's inner index, exponents
+  unsigned char* gs;      // columns of G_{old,new}: [128 rows][chunk] images
+  int* ge;                // their exponents, [row][pl]
+  double* gpart;          // split-K partial tiles of G_{new,new}
+  int* gticket;           // arrivals per tile and epilogue warp
   double* part[2];        // split-K partial tiles of the prep products (128 x 64)
   int* ticket[2];         // arrivals per tile and epilogue warp
   int pl;                 // parts of the inner dimension at the capacity
@@ -79,6 +83,13 @@ constexpr int kSlicedMinOrder = 256;
 // chains of k_max 32, 37.3 / 36.4 for one of 64 at order 415, 164 / 57 for one of 128
 // at order 2085, 2670 / 254 for two of 256 at order 6760.
 constexpr int kSlicedYMinK = 64;
+// k_max from which G_{new,new} is one: us per block of the prep, float64 pipe against
+// sliced, 87 / 108 for one chain of 64 at order 415, 465 / 412 for one of 128 at
+// order 2085, 7480 / 5800 for two of 256 at order 6760.
+constexpr int kSlicedNewMinK = 128;
+// Split of G_{new,new} = C G_{old,new} over its inner dimension: a part or two per
+// slice, since it has few tiles (at most eight per spin).
+__host__ __device__ inline int sliced_new_slices(int n) { return ((n + 127) / 128 + 1) / 2; }
 // Bytes of the strip pool, unless one job needs more.
 constexpr size_t kSlicedPool = (size_t)8 << 30;
 
