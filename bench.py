@@ -709,7 +709,13 @@ def measure_form(args, pk, torch, dist, chains, meta, refresh, form, local, worl
     alu_src = (f"FP64 = bf16 {peak_kind} x 1.25/2250" if precision == pk.CTAUX_FP64
                else "FP32 = 152 SMs x 128 lanes x 2 x 2.07 GHz")
     dw = {k: work1[k] - work0[k] for k in work1}
-    n_sm = min(152, len(chains))   # one CTA (one SM) per chain for the Gamma growth
+    # SMs of the Gamma growth: a cluster per chain while the chains' clusters fit, else one CTA
+    cl = 16 if args.gamma != "lu" and max(c.k_max for c in chains) > 24 else 1
+    while cl > 1 and cl * len(chains) > 152:
+        cl //= 2
+    if cl < (2 if precision == pk.CTAUX_FP64 else 4):
+        cl = 1
+    n_sm = min(152, cl * len(chains))
     elem = 8 if precision == pk.CTAUX_FP64 else 4
     # float64 prep and flush run on the tensor cores from this capacity on (ctaux_sliced.cuh)
     sliced = min(c.capacity + c.k_max for c in chains) >= 256
@@ -748,7 +754,7 @@ def measure_form(args, pk, torch, dist, chains, meta, refresh, form, local, worl
             a = dw["gamma_flop"] / sec / 1e12
             return dict(bound="alu", achieved=a, peak=alu_peak, unit="TFLOP/s",
                         peak_source=alu_src + "; whole GPU (the Gamma chain of a chain runs on "
-                                              "one SM: frac_of_active_sms is against the "
+                                              "a cluster of SMs: frac_of_active_sms is against the "
                                               f"{n_sm} SMs in use)",
                         frac_of_active_sms=a / (alu_peak * n_sm / 152.0))
         if nm == "measure":
