@@ -440,12 +440,12 @@ __global__ void __launch_bounds__(256) k_inv_cols(const InvView* views, const in
 // run while it adds to X on the float64 pipe.  Per tile: 34 x 2 MMAs of 48
 // clocks (128 x 64 x 16, bound by shared-memory reads of A and B) against 8192
 // float64 additions, 19 clocks per warp.  X's loads and additions hide behind
-// the next tile's MMAs once the tile has been sent for (834 -> 740 us per rank-128
-// product at order 6760, both spins); what is left open is the emptying of the
-// accumulators, bound by the conversions to integers (740 -> 660 us with four of
-// them per element in place of six; 590 with none, where shared memory, reads for
-// the MMAs and writes of the bulk copies, is the bound).  Releasing the accumulators
-// group by group took 694: its shorter loads wait more often.
+// the next tile's MMAs once the tile has been sent for (830 -> 741 us per rank-128
+// product at order 6760, both spins, caches cold); what is left open is the
+// emptying of the accumulators, with its conversions to integers (741 -> 732 us
+// with four of them per element in place of six).  With the emptying cut to a
+// quarter it took 590 us: shared memory, reads for the MMAs and writes of the bulk
+// copies, is the bound there.
 constexpr int kUpdStages = 2, kUpdThreads = 576;
 constexpr int kUpdCols = 16;   // columns of an epilogue warp
 constexpr int kUpdStageBytes = oz::kImageA + oz::kImageB;
