@@ -323,8 +323,8 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
   // from-scratch recomputation: launch shapes for all chains and for one
   std::vector<int> lds;
   for (const auto& cp : ctx->chains) lds.insert(lds.end(), 2, round_up(cp.capacity + cp.k_max, 32));
-  CUDA_TRY(ctx, inv_configure({max_ld, max_ld}, ctx->sm_count, &ls.inv_one));
-  CUDA_TRY(ctx, inv_configure(lds, ctx->sm_count, &ls.inv_all));
+  CUDA_TRY(ctx, inv_configure({max_ld, max_ld}, ctx->sm_count, false, &ls.inv_one));
+  CUDA_TRY(ctx, inv_configure(lds, ctx->sm_count, false, &ls.inv_all));
   std::vector<InvView> host_views(items);
 
   for (size_t ci = 0; ci < ctx->chains.size(); ++ci) {

@@ -20,6 +20,18 @@
 //     runs while they travel.
 //   k_inv_rows    the pivot rows of the other columns, sliced (ctaux_oz.cuh).
 //   k_inv_update  the rank-32 product on the float16 tensor cores.
+// Balance.  The product's error is relative to the largest element of a row of P'
+// and of a column of X[R, J].  A pivot row's own scale r goes into its inner index
+// as 1 / r in P' and as r in X[R, J], so in a matrix whose rows differ in scale the
+// index with the largest multipliers loses the digits of exactly its own pivot row
+// (rows scaled by 2^-27 to 2^27, order 64: error 1e-8 in place of 2e-14).  Inner
+// index k is therefore scaled by the power of two 2^s_k, s_k = max_i (exponent of
+// P'[i][k] - largest exponent in row i) <= 0, taken off P' and put on X[R, J]: the
+// least that keeps every row's largest element, so that what an index adds to the
+// error is bounded by its own terms.  It costs an exchange per panel in the cluster
+// (order 310: 773 -> 794 us).
+// N^{-1} = [e^V / (e^V - 1) - G0] (e^V - 1) has rows of one scale and goes without;
+// scaled columns cancel by themselves.
 // From order 1024 on, two levels: the rank-32 products of four panels stay
 // inside 128 columns, the rest of the matrix follows with one rank-128 product
 // (k_inv_cols slices the 128 columns).  That reads and writes X, and runs the
@@ -41,6 +53,7 @@ namespace {
 
 constexpr int kMaxWidth = oz::kK;
 constexpr int kMaxCluster = 16;
+constexpr int kNoShift = -(1 << 16);   // below every difference of exponents
 
 // Pivot key: the upper 32 bits of the float64 pattern of a magnitude (sign 0,
 // the whole exponent, 20 significand bits) order like the magnitude for every
@@ -134,7 +147,7 @@ __device__ __forceinline__ void st_async(uint32_t addr, unsigned long long v, ui
 // takes 19 clocks of the float64 pipe per column and 32 rows of a CTA, which
 // bounds the step from about 200 rows per CTA on.  Keeping the update to the
 // columns on the right halves that part.
-template <int THREADS>
+template <int THREADS, bool BALANCE>
 __global__ void __launch_bounds__(THREADS, THREADS == 512 ? 1 : 3)
 k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows_cap) {
   constexpr int kWarps = THREADS / 32;
@@ -154,8 +167,10 @@ k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows
   double* crow = Ps + (size_t)width * rs;                      // [3][kMaxCluster][kMaxWidth]
   unsigned long long* ckey = reinterpret_cast<unsigned long long*>(crow + 3 * kMaxCluster * kMaxWidth);
   int8_t* us = reinterpret_cast<int8_t*>(ckey + 3 * kMaxCluster);   // [rs] 0 free, 1 pivoted before, 2 + k in step k
+  int* shifts = reinterpret_cast<int*>(us + ((rs + 15) & ~15));     // with balance: [kMaxCluster][kMaxWidth]
   __shared__ uint32_t wmag[kWarps], wrow[kWarps];
   __shared__ double cand_row[kMaxWidth];
+  __shared__ int shift[kMaxWidth];
   __shared__ uint64_t landed[3];   // candidates of a generation: one local arrival and their bytes
   __shared__ volatile int gave_up;
   const uint32_t bytes = ncta * (uint32_t)(sizeof(double) * kMaxWidth + sizeof(unsigned long long));
@@ -296,6 +311,40 @@ k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows
     }
   }
   __syncthreads();
+  if constexpr (BALANCE) {
+    // ---- balance of the inner index: the CTA's rows, then all CTAs'
+    if (tid < kMaxWidth) shift[tid] = kNoShift;
+    __syncthreads();
+    for (int e = tid; e < ((nr + 31) & ~31) * 4; e += THREADS) {   // the whole warp
+      const int r = (e >> 7) * 32 + lane, ch = (e >> 5) & 3;
+      const int step = r < nr ? max((int)us[r] - 2, 0) : bw;
+      int mx = 0;
+      for (int k = step; k < bw; ++k) mx = max(mx, oz::exp_field((uint32_t)__double2hiint(Ps[(size_t)k * rs + r])));
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        const int k = ch * 8 + t;
+        const int f = k >= step && k < bw ? oz::exp_field((uint32_t)__double2hiint(Ps[(size_t)k * rs + r])) : 0;
+        // a row that is not finite has products that are not finite in any case
+        const int s = __reduce_max_sync(0xffffffffu, f != 0 && mx != 0x7ff ? f - mx : kNoShift);
+        if (lane == 0) atomicMax(shift + k, s);
+      }
+    }
+    __syncthreads();
+    for (uint32_t w = (uint32_t)warp; w < ncta; w += kWarps)
+      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(map_rank(tc::smem_u32(shifts + rank * kMaxWidth + lane), w)),
+                   "r"(shift[lane])
+                   : "memory");
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+    if (tid < kMaxWidth) {
+      int s = kNoShift;
+      for (uint32_t w = 0; w < ncta; ++w) s = max(s, shifts[w * kMaxWidth + tid]);
+      shift[tid] = s == kNoShift ? 0 : s;
+      if (rank == 0) v.balance[tid] = shift[tid];
+    }
+    __syncthreads();
+  }
   cluster_arrive();   // no CTA exits while another may still store to it
   // ---- L, and the slices of F: four threads per row, 8 columns (one 16-byte
   // chunk of every slice) each
@@ -305,16 +354,20 @@ k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows
     const int step = (int)us[r] - 2;   // of a pivot row of this panel
     if (step >= 0)
       for (int k = ch * 8; k < min(step, ch * 8 + 8); ++k) v.L[step * kMaxWidth + k] = Ps[(size_t)k * rs + r];
-    int mx = 0;
-    for (int k = max(step, 0); k < bw; ++k)
-      mx = max(mx, oz::exp_field((uint32_t)__double2hiint(Ps[(size_t)k * rs + r])));
+    int mx = 0, top = 0;   // the largest exponent field, balanced, and as it is
+    for (int k = max(step, 0); k < bw; ++k) {
+      const int f = oz::exp_field((uint32_t)__double2hiint(Ps[(size_t)k * rs + r]));
+      top = max(top, f);
+      if (BALANCE && f) mx = max(mx, f - shift[k]);
+    }
+    if (!BALANCE || top == 0x7ff) mx = top;
     const int row = r0 + r;
     unsigned char* img = v.As + (size_t)(row >> 7) * v.chunks * oz::kImageA + oz::chunk_offset(row & 127, ch);
     long long y[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
       const int k = ch * 8 + t;
-      y[t] = oz::biased_digits(k < bw && k >= step ? Ps[(size_t)k * rs + r] : 0.0, mx);
+      y[t] = oz::biased_digits(k < bw && k >= step ? Ps[(size_t)k * rs + r] : 0.0, mx, BALANCE && top != 0x7ff ? -shift[k] : 0);
     }
     oz::store_chunk(img, oz::kRowsA, y);
     if (ch == 0) v.ea[row] = oz::row_exponent(mx);
@@ -333,6 +386,7 @@ struct InvRange {
 // warp per column, a lane per pivot row.  Rank 32: y_k, the column at pivot row k
 // just before step k, y_k = X[R_k][j] + sum_{l<k} L[k][l] y_l; the panel's own
 // column c0 + k starts from the unit vector e_k.
+template <bool BALANCE>
 __global__ void __launch_bounds__(256) k_inv_rows(const InvView* views, const int* orders, int items,
                                                   InvRange g) {
   __shared__ int off[2 * kMaxChains + 1];
@@ -376,12 +430,18 @@ __global__ void __launch_bounds__(256) k_inv_rows(const InvView* views, const in
 #pragma unroll
     for (int c = 0; c < 4; ++c) mx = max(mx, oz::exp_field((uint32_t)__double2hiint(x[c])));
     mx = __reduce_max_sync(0xffffffffu, mx);
+    int shift = 0;
+    if (BALANCE && mx != 0 && mx != 0x7ff) {   // (rank 32: x[0] alone)
+      shift = lane < bw ? v.balance[lane] : 0;
+      const int f = oz::exp_field((uint32_t)__double2hiint(x[0]));
+      mx = __reduce_max_sync(0xffffffffu, f ? f + shift : kNoShift);
+    }
     unsigned char* img = v.Bs + (size_t)(j >> 6) * v.chunks * oz::kImageB +
                          oz::chunk_offset(j & 63, lane >> 3) + (lane & 7) * 2;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       if (c >= nc) break;
-      const long long y = oz::biased_digits(x[c], mx);
+      const long long y = oz::biased_digits(x[c], mx, shift);
 #pragma unroll
       for (int i = 0; i < oz::kSlices; ++i)
         *reinterpret_cast<uint16_t*>(img + (size_t)c * oz::kImageB + (size_t)i * oz::kRowsB * 64) =
@@ -636,9 +696,10 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
 
 constexpr int upd_smem() { return kUpdStages * kUpdStageBytes + 1024; }
 
-int panel_smem_bytes(int width, int rows) {
+int panel_smem_bytes(int width, int rows, bool balance) {
   return (int)(sizeof(double) * ((size_t)width * rows + 3 * kMaxCluster * kMaxWidth) +
-               sizeof(unsigned long long) * 3 * kMaxCluster + (size_t)((rows + 15) & ~15));
+               sizeof(unsigned long long) * 3 * kMaxCluster + (size_t)((rows + 15) & ~15) +
+               (balance ? sizeof(int) * kMaxCluster * kMaxWidth : 0));
 }
 
 }  // namespace
@@ -649,9 +710,10 @@ int panel_smem_bytes(int width, int rows) {
 // to order 1084: 13.0 ms, 14.3 with 4; larger clusters pay where a batch's last,
 // largest matrices are left), 4 beyond 256 matrices, whose rows fill the float64
 // pipes of all SMs anyway.
-cudaError_t inv_configure(const std::vector<int>& lds, int sm_count, InvShape* out) {
+cudaError_t inv_configure(const std::vector<int>& lds, int sm_count, bool balance, InvShape* out) {
   InvShape s{};
   s.sm_count = sm_count;
+  s.balance = balance;
   int max_ld = 1;
   for (int ld : lds) max_ld = ld > max_ld ? ld : max_ld;
   s.chunks = inv_chunks(max_ld);
@@ -660,13 +722,15 @@ cudaError_t inv_configure(const std::vector<int>& lds, int sm_count, InvShape* o
     return e;
   };
   const int most = 220 * 1024;
-  cudaError_t e = cudaFuncSetAttribute(k_inv_panel<512>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess) e = attrs(k_inv_panel<512>, most);
-  if (e == cudaSuccess) e = attrs(k_inv_panel<256>, most);
+  auto* panel512 = balance ? k_inv_panel<512, true> : k_inv_panel<512, false>;
+  auto* panel256 = balance ? k_inv_panel<256, true> : k_inv_panel<256, false>;
+  cudaError_t e = cudaFuncSetAttribute(panel512, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) e = attrs(panel512, most);
+  if (e == cudaSuccess) e = attrs(panel256, most);
   if (e == cudaSuccess) e = attrs(k_inv_update<false>, upd_smem());
   if (e == cudaSuccess) e = attrs(k_inv_update<true>, upd_smem());
   if (e != cudaSuccess) return e;
-  auto smem_of = [&](int cluster) { return panel_smem_bytes(s.width, (max_ld + cluster - 1) / cluster); };
+  auto smem_of = [&](int cluster) { return panel_smem_bytes(s.width, (max_ld + cluster - 1) / cluster, balance); };
   // 16 CTAs need a GPC with that many free SMs
   int largest = 16;
   {
@@ -681,7 +745,7 @@ cudaError_t inv_configure(const std::vector<int>& lds, int sm_count, InvShape* o
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, k_inv_panel<512>, &cfg);
+    e = cudaOccupancyMaxActiveClusters(&n, panel512, &cfg);
     if (e != cudaSuccess) return e;
     if (n == 0) largest = 8;
   }
@@ -707,7 +771,8 @@ int launch_inverse(const InvView* views, const int* orders, int items, int max_o
   auto update = [&](int c0, int width, int j0, int j1) {
     const InvRange g{c0, width, j0, j1};
     const long cols = (j1 < max_order ? j1 : max_order) - j0;
-    k_inv_rows<<<grid(items * ((cols + 7) / 8), 8 * sms), 256, 0, st>>>(views, orders, items, g);
+    auto* rows = sh.balance ? k_inv_rows<true> : k_inv_rows<false>;
+    rows<<<grid(items * ((cols + 7) / 8), 8 * sms), 256, 0, st>>>(views, orders, items, g);
     const int ug = grid(items * rb * ((cols + 63) / 64), sms);
     if (width > oz::kK) k_inv_update<true><<<ug, kUpdThreads, upd_smem(), st>>>(views, orders, items, g);
     else k_inv_update<false><<<ug, kUpdThreads, upd_smem(), st>>>(views, orders, items, g);
@@ -728,9 +793,9 @@ int launch_inverse(const InvView* views, const int* orders, int items, int max_o
       at.val.clusterDim.y = at.val.clusterDim.z = 1;
       cfg.attrs = &at;
       cfg.numAttrs = 1;
-      const cudaError_t e =
-          pn.threads == 512 ? cudaLaunchKernelEx(&cfg, k_inv_panel<512>, views, orders, c0, sh.width, pn.rows)
-                            : cudaLaunchKernelEx(&cfg, k_inv_panel<256>, views, orders, c0, sh.width, pn.rows);
+      auto* fn = pn.threads == 512 ? (sh.balance ? k_inv_panel<512, true> : k_inv_panel<512, false>)
+                                   : (sh.balance ? k_inv_panel<256, true> : k_inv_panel<256, false>);
+      const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, views, orders, c0, sh.width, pn.rows);
       n += 1;
       if (e != cudaSuccess) {
         *err = e;

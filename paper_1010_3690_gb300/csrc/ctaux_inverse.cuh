@@ -23,6 +23,8 @@ struct InvView {
   int* pcol;            // column at which a row was pivoted, -1 if not yet
   double* piv;          // pivots, in column order
   double* L;            // [32][32] multipliers of the current panel's pivot rows
+  int* balance;         // [32] balance of the current panel (ctaux_inverse.cu); null where the
+                        // matrix is known to have rows of one scale
   int* status;          // DS_SINGULAR and DS_TIMEOUT bits
 };
 
@@ -66,10 +68,12 @@ struct InvShape {
   int width;                     // panel width (32; 16 or 8 where a panel would not fit)
   int chunks;                    // 4: two levels
   int sm_count;
+  bool balance;
   std::vector<InvPanel> panels;  // of each panel: fewer matrices reach the later ones
 };
-// lds: the leading dimension of every matrix.
-cudaError_t inv_configure(const std::vector<int>& lds, int sm_count, InvShape* out);
+// lds: the leading dimension of every matrix.  balance: for matrices whose rows may
+// differ in scale (one level only); their views then have room for it.
+cudaError_t inv_configure(const std::vector<int>& lds, int sm_count, bool balance, InvShape* out);
 
 // Inverts the matrices views[0..items) of orders orders[0..items) (device; 0 =
 // leave out), none above max_order: afterwards inv[c][perm[j]] = X[perm[c]][j].

@@ -21,7 +21,8 @@ constexpr int kM = CTAUX_NOALLOC_MAX_M;
 // the order and the view.
 constexpr size_t kWork = ((size_t)kM * kM + (size_t)kM * 114 + 1024) * sizeof(double);   // ld^2 + inv_extra_doubles(kM, 1)
 constexpr size_t kPerm = kWork, kPcol = kPerm + kM * sizeof(int), kUsed = kPcol + kM * sizeof(int),
-                 kStatus = kUsed + kM, kOrder = kStatus + 16, kView = kOrder + 16, kEnd = kView + sizeof(InvView);
+                 kStatus = kUsed + kM, kOrder = kStatus + 16, kBalance = kOrder + 16, kView = kBalance + 32 * sizeof(int),
+                 kEnd = kView + sizeof(InvView);
 static_assert(kEnd <= CTAUX_NOALLOC_SCRATCH_BYTES, "scratch size in the header");
 
 // Shared by every call on a device; held by each device that loads the library.
@@ -95,7 +96,7 @@ extern "C" ctaux_status ctaux_invert_noalloc(const double* d_a, int lda, double*
   std::call_once(s.once, [&s, dev]() {
     s.err = cudaGetSymbolAddress(reinterpret_cast<void**>(&s.scratch), g_noalloc_scratch);
     if (s.err == cudaSuccess) s.err = cudaDeviceGetAttribute(&s.sms, cudaDevAttrMultiProcessorCount, dev);
-    if (s.err == cudaSuccess) s.err = inv_configure({kM}, s.sms, &s.shape);
+    if (s.err == cudaSuccess) s.err = inv_configure({kM}, s.sms, true, &s.shape);
   });
   if (s.err != cudaSuccess || !s.scratch) return CTAUX_ECUDA;
   InvView v{};
@@ -104,6 +105,7 @@ extern "C" ctaux_status ctaux_invert_noalloc(const double* d_a, int lda, double*
   v.pcol = reinterpret_cast<int*>(s.scratch + kPcol);
   v.used = reinterpret_cast<int8_t*>(s.scratch + kUsed);
   v.status = reinterpret_cast<int*>(s.scratch + kStatus);
+  v.balance = reinterpret_cast<int*>(s.scratch + kBalance);   // a caller's rows may differ in scale
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   k_noalloc_load<<<m, 256, 0, st>>>(d_a, lda, m, v, s.scratch);
   cudaError_t e = cudaSuccess;

@@ -47,13 +47,14 @@ __device__ __forceinline__ int row_exponent(int max_field) {
   return max_field == 0x7ff ? kNonFinite : max_field - 1022;
 }
 
-// x as a fixed-point integer, x ~ q 2^(e - 55), |q| <= 2^55, plus the bias
+// x 2^shift as a fixed-point integer, ~ q 2^(e - 55), |q| <= 2^55, plus the bias
 // that makes the six low bytes the digits + 128 (the digits are balanced); the
-// seventh digit is the (signed) rest.  Subnormal x count as zero.
-__device__ __forceinline__ long long biased_digits(double x, int max_field) {
+// seventh digit is the (signed) rest.  max_field: the row's largest exponent
+// field, its shift added.  Subnormal x count as zero.
+__device__ __forceinline__ long long biased_digits(double x, int max_field, int shift = 0) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
   const int ex = (int)(bits >> 52) & 0x7ff;
-  const int t = max_field - ex;   // >= 0
+  const int t = max_field - ex - shift;   // >= 0
   unsigned long long q = 0;
   if (ex != 0 && t < 56) {
     const unsigned long long v = ((bits & 0xfffffffffffffull) | 0x10000000000000ull) << 2;
