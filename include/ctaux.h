@@ -368,8 +368,9 @@ ctaux_status ctaux_synchronize(ctaux_ctx *ctx);
  *
  * Inverts the m x m float64 matrix d_a (column-major, leading dimension lda,
  * device memory) by Gauss-Jordan elimination with partial pivoting -- the
- * arithmetic of the FP64 recomputation that ctaux_recompute runs -- and
- * writes the inverse to d_inv (leading dimension ld_inv, device memory) and
+ * arithmetic of the FP64 recomputation that ctaux_recompute runs, with its
+ * products balanced so that rows of different scale keep float64 accuracy --
+ * and writes the inverse to d_inv (leading dimension ld_inv, device memory) and
  * log|det d_a| to *d_logdet (device memory, may be NULL).  Asynchronous on
  * cuda_stream (NULL = legacy default stream).  A singular input gives -inf in
  * *d_logdet and non-finite entries in d_inv.  The caller owns d_a, d_inv and

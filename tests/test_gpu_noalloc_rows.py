@@ -67,8 +67,9 @@ def _scales(kind, m):
         c = one.copy()
         c[m - 3] = 2.0 ** 27
         return spread(20), c
-    assert kind == "low"   # near and below the smallest normal number
-    return 2.0 ** rng.integers(-6, 7, m), np.full(m, 2.0 ** -1010)
+    near = 2.0 ** rng.integers(-6, 7, m)   # of the smallest and the largest normal number
+    end = 2.0 ** (-1010 if kind.startswith("low") else 1005)
+    return (near * end, one) if kind.endswith("rows") else (near, one * end)
 
 
 def _invert(a):
@@ -103,7 +104,8 @@ def _check(m, kind):
 
 @pytest.mark.parametrize("m", [40, 137, 257])
 @pytest.mark.parametrize("kind", ["rows0", "rows13", "rows27", "rows53", "columns", "both", "similar",
-                                  "ascending", "half_column"])
+                                  "ascending", "half_column", "low", "high",
+                                  "low_rows", "high_rows"])
 def test_rows_and_columns_of_different_scale(m, kind):
     _check(m, kind)
 
