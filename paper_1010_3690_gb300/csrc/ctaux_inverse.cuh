@@ -57,6 +57,14 @@ __host__ __device__ inline void inv_layout(double* work, int ld, int chunks, Inv
   v.L = v.piv + lp;
 }
 
+// Column of the inverse that column j of X holds.  After a bounded wait gave up
+// (status beyond `singular`, a zero pivot's bit), perm may hold rows of an earlier,
+// larger matrix, and what X holds is of no use: every column then stays in its place,
+// inside the caller's matrix.
+__host__ __device__ inline int inv_column(int status, int singular, const int* perm, int j) {
+  return (status & ~singular) ? j : perm[j];
+}
+
 // Launch parameters of the inversion of a set of matrices.
 struct InvPanel {
   int cluster;     // CTAs of a matrix's cluster (2 to 16)

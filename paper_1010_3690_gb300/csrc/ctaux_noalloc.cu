@@ -92,13 +92,14 @@ __global__ void __launch_bounds__(256) k_noalloc_rows(int m, InvView v, int* row
 }
 
 // The inverse in the caller's order, and log|det| (the pivots' logarithms, in a
-// fixed order).  NaN where a bounded wait of the inversion gave up.
+// fixed order).  All NaN where a bounded wait of the inversion gave up.
 __global__ void __launch_bounds__(256) k_noalloc_store(double* __restrict__ Ainv, int ldi, int m, InvView v,
                                                        const int* __restrict__ col_exp,
                                                        const int* __restrict__ row_exp, double* logdet) {
-  const double poison = (*v.status & ~DS_SINGULAR) ? nan("") : 0.0;
+  const int status = *v.status;
+  const double poison = (status & ~DS_SINGULAR) ? nan("") : 0.0;
   for (int j = blockIdx.x; j < m; j += gridDim.x) {
-    const int pj = v.perm[j], re = row_exp[pj];
+    const int pj = inv_column(status, DS_SINGULAR, v.perm, j), re = row_exp[pj];
     for (int c = threadIdx.x; c < m; c += blockDim.x) {
       const double x = v.X[(size_t)j * v.ld + v.perm[c]] + poison;   // inv[c][perm[j]]
       const int e = re + col_exp[c];
