@@ -216,12 +216,11 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
   p.pool_exp = reinterpret_cast<int*>(base + o_exp);
   p.strips = ctx->strips.data();
   p.n_strips = (int)ctx->strips.size();
-  for (const SlicedStrip& s : ctx->strips) p.max_jobs = std::max(p.max_jobs, s.count);
   ls.any_sliced = 1;
   ls.any_plain = plain;
   ls.any_plain_y = plain_y;
   ls.any_plain_new = plain_new;
-  CUDA_TRY(ctx, configure_sliced(nch, p.max_jobs));
+  CUDA_TRY(ctx, configure_sliced());
   return CTAUX_OK;
 }
 
@@ -289,11 +288,11 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
                  sizeof(short) * ((max_ld + 7) & ~7) + sizeof(uint32_t) * ((max_ld + 31) / 32) +
                  sizeof(double) * 2 * max_k + sizeof(double) * 2 * max_k + ((max_ld + 15) & ~15) + 64;
   size_t gam = ((sizeof(T) * 2 * (size_t)max_k * (max_k + 1)) + 15) & ~size_t(15);
-  ls.gamma_in_smem = (fixed + gam <= 200 * 1024) ? 1 : 0;
+  ls.gamma_in_smem = (fixed + gam <= kPropSmem) ? 1 : 0;
   ls.prop_smem = (int)(fixed + (ls.gamma_in_smem ? gam : 0));
   ls.gamma_lu = P.gamma_form == CTAUX_GAMMA_LU ? 1 : 0;
   ls.max_k = max_k;
-  CUDA_TRY(ctx, configure_block_kernels<T>(ls));
+  CUDA_TRY(ctx, configure_block_kernels<T>());
   int max_cap = 0;
   for (const auto& cp : ctx->chains) max_cap = std::max(max_cap, cp.capacity + cp.k_max);
   CUDA_TRY(ctx, configure_gamma_cluster<T>(ls, max_cap, ctx->sm_count));

@@ -1471,8 +1471,8 @@ void launch_g0_pairs(const double* plain, int n_tau, long entries, double2* g0, 
 
 // ----------------------------------------------------------- launchers
 template <typename T>
-int lu_inverse_smem(const LaunchShape& ls) {
-  return (int)(sizeof(T) * 32 * (size_t)ls.max_k);
+int lu_inverse_smem(int max_k) {
+  return (int)(sizeof(T) * 32 * (size_t)max_k);
 }
 
 template <typename T>
@@ -1519,7 +1519,7 @@ void launch_block(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st, Pha
     else k_proposals<T, false><<<nch, 256, ls.prop_smem, st>>>(dchains);
   }
   if (ls.gamma_lu)
-    k_lu_inverse<T><<<dim3((ls.max_k + 31) / 32, 2, nch), 32, lu_inverse_smem<T>(ls), st>>>(dchains);
+    k_lu_inverse<T><<<dim3((ls.max_k + 31) / 32, 2, nch), 32, lu_inverse_smem<T>(ls.max_k), st>>>(dchains);
   pt->end(2, st, ls.gamma_lu ? 2 : 1);
   bool tc = false;
   if constexpr (std::is_same<T, float>::value) tc = ls.use_tc != 0;
@@ -1560,13 +1560,13 @@ void launch_block(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st, Pha
 }
 
 template <typename T>
-cudaError_t configure_block_kernels(const LaunchShape& ls) {
+cudaError_t configure_block_kernels() {
   const cudaFuncAttribute dyn = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(k_proposals_smem<T, false>, dyn, ls.prop_smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_proposals<T, false>, dyn, ls.prop_smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_proposals_smem<T, true>, dyn, ls.prop_smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_proposals<T, true>, dyn, ls.prop_smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lu_inverse<T>, dyn, lu_inverse_smem<T>(ls));
+  cudaError_t e = cudaFuncSetAttribute(k_proposals_smem<T, false>, dyn, kPropSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_proposals<T, false>, dyn, kPropSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_proposals_smem<T, true>, dyn, kPropSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_proposals<T, true>, dyn, kPropSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lu_inverse<T>, dyn, lu_inverse_smem<T>(kMaxK));
   return e;
 }
 
@@ -1574,7 +1574,7 @@ template void launch_block<double>(Chain<double>*, const LaunchShape&, cudaStrea
                                    const TcMaps*, const BlockFork*);
 template void launch_block<float>(Chain<float>*, const LaunchShape&, cudaStream_t, PhaseTimer*,
                                   const TcMaps*, const BlockFork*);
-template cudaError_t configure_block_kernels<double>(const LaunchShape&);
-template cudaError_t configure_block_kernels<float>(const LaunchShape&);
+template cudaError_t configure_block_kernels<double>();
+template cudaError_t configure_block_kernels<float>();
 
 }  // namespace ctaux

@@ -148,6 +148,11 @@ struct LaunchShape {
   int tile_mask[PH_COUNT];  // tile variants in the context's table, per product (bit v)
 };
 
+// Largest dynamic shared memory of the proposals of one CTA.  A kernel's limit holds
+// for the process, not for a context: every configure_* sets one that no context
+// exceeds, and the launches ask for what their context needs.
+constexpr int kPropSmem = 200 * 1024;
+
 // Row stride of a CTA's share of Gamma^{-1} in the cluster form: four lanes per
 // row read consecutive elements of a warp's eight rows without bank conflicts.
 __host__ __device__ inline int gamma_share_stride(int k, size_t element) {
@@ -215,7 +220,7 @@ template <typename T>
 void launch_block(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st, PhaseTimer* pt,
                   const TcMaps* maps, const BlockFork* fork = nullptr);
 template <typename T>
-cudaError_t configure_block_kernels(const LaunchShape& ls);
+cudaError_t configure_block_kernels();
 size_t refresh_work_doubles(int ld);
 size_t refresh_work_one(int ld);
 template <typename T>
@@ -258,7 +263,7 @@ template <typename T>
 cudaError_t configure_gamma_cluster(LaunchShape& ls, int max_cap, int sm_count);
 template <typename T>
 cudaError_t launch_gamma_cluster(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st);
-cudaError_t configure_sliced(int n_chains, int max_jobs);
+cudaError_t configure_sliced();
 // The prep products R~ and G_{old,new}, and the flush product, of the sliced
 // chains; return the kernels launched.
 int launch_sliced_prep(const Chain<double>* dchains, const LaunchShape& ls, cudaStream_t st);

@@ -741,13 +741,15 @@ int prod_smem(int n) { return kProdStages * kProdStageBytes + 1024 + (int)sizeof
 
 }  // namespace
 
-cudaError_t configure_sliced(int n_chains, int max_jobs) {
+// The limits hold for the process: for the most chains and jobs (four per chain).
+cudaError_t configure_sliced() {
   const cudaFuncAttribute dyn = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(k_sliced_product<PrepSrc, false>, dyn, prod_smem(max_jobs));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_slice_n, dyn, (int)sizeof(int) * (max_jobs + 1));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sliced_product<NewSrc, false>, dyn, prod_smem(n_chains));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sliced_product<YSrc, false>, dyn, prod_smem(n_chains));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sliced_product<FlushSrc, true>, dyn, prod_smem(n_chains));
+  constexpr int kMaxJobs = 4 * kMaxChains;
+  cudaError_t e = cudaFuncSetAttribute(k_sliced_product<PrepSrc, false>, dyn, prod_smem(kMaxJobs));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_slice_n, dyn, (int)sizeof(int) * (kMaxJobs + 1));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sliced_product<NewSrc, false>, dyn, prod_smem(kMaxChains));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sliced_product<YSrc, false>, dyn, prod_smem(kMaxChains));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sliced_product<FlushSrc, true>, dyn, prod_smem(kMaxChains));
   return e;
 }
 

@@ -45,7 +45,6 @@ struct SlicedPlan {
   int* pool_exp = nullptr;
   const SlicedStrip* strips = nullptr;
   int n_strips = 0;
-  int max_jobs = 0;                    // of a strip
 };
 
 constexpr size_t kSlicedImageA = 7 * 128 * 64, kSlicedImageB = 7 * 64 * 64;   // oz::kImageA, oz::kImageB
