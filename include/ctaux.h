@@ -146,7 +146,13 @@ typedef struct {
                                          CTAUX_ETIMEOUT; 0 = 2^24 (seconds).  A negative value
                                          is a test of that path: the MMA issuer first waits
                                          -tc_wait_limit polls on a barrier that nothing
-                                         completes, so every flush reports CTAUX_ETIMEOUT */
+                                         completes, so every flush reports CTAUX_ETIMEOUT.
+                                         FP64 form: the same for the products on the tensor
+                                         cores (capacity + k_max of 256 and more); the test
+                                         lasts until a chain's second recomputation
+                                         (ctaux_set_config counts as one).  A launch that
+                                         gives up stops all its chains; ctaux_set_config
+                                         makes a chain usable again */
   int gamma_form;                     /* CTAUX_GAMMA_INVERSE (0) or CTAUX_GAMMA_LU (1); the
                                          same Markov chain either way (ratios equal up to
                                          rounding) */

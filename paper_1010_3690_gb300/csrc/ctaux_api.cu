@@ -543,7 +543,7 @@ ctaux_status check_device_status(ctaux_ctx* ctx) {
       return set_err(ctx, CTAUX_ESINGULAR, "chain %zu: zero pivot in the FP64 recomputation", ci);
     if (st & DS_INDEX) return set_err(ctx, CTAUX_EINVAL, "chain %zu: vertex selection out of range", ci);
     if (st & DS_TIMEOUT)
-      return set_err(ctx, CTAUX_ETIMEOUT, "chain %zu: a bounded wait of the tensor-core flush gave up", ci);
+      return set_err(ctx, CTAUX_ETIMEOUT, "chain %zu: a bounded wait of a kernel gave up", ci);
     if (st) return set_err(ctx, CTAUX_ENUMERIC, "chain %zu: device status %d", ci, st);
     int ex = 0;
     CUDA_TRY(ctx, cudaMemcpy(&ex, &dp->drift_exceeded, sizeof(int), cudaMemcpyDeviceToHost));

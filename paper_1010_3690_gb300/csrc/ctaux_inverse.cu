@@ -568,6 +568,11 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
   uint32_t issued = 0;
+  auto fail = [&]() {   // tiles of any matrix may stay undone
+    err_s = 1;
+    for (int i = 0; i < items; ++i)
+      if (orders[i] > 0) atomicOr(views[i].status, DS_TIMEOUT);
+  };
 
   if (warp == 0 && lane == 0) {
     for (int w = blockIdx.x; w < total && !err_s; w += gridDim.x) {
@@ -588,8 +593,7 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
         ++issued;
       }
       if (!ok) {
-        err_s = 1;
-        atomicOr(v.status, DS_TIMEOUT);
+        fail();
         break;
       }
     }
@@ -617,8 +621,7 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
         __syncwarp();
       }
       if (!ok) {
-        err_s = 1;
-        if (lane == 0) atomicOr(views[t.it].status, DS_TIMEOUT);
+        if (lane == 0) fail();
         break;
       }
       if (oz::elect_one()) mma_commit(smem_u32(&accfull));
@@ -631,7 +634,6 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
     const int quarter = warp & 3, group = (warp - 2) >> 2;
     uint32_t q = 0;
     for (int w = blockIdx.x; w < total; w += gridDim.x, ++q) {
-      if (__any_sync(0xffffffffu, err_s != 0)) break;
       const UpdTile t = upd_tile(off, orders, items, w, g.j0);
       const InvView& v = views[t.it];
       const int ld = v.ld, i = t.i0 + quarter * 32 + lane, jb = t.j0 + group * kUpdCols;
@@ -646,11 +648,8 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
         if (pi < t.m && pj < je)
           asm volatile("prefetch.global.L2 [%0];" ::"l"(v.X + (size_t)pj * ld + pi));
       }
-      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&accfull), q & 1))) {
-        if (lane == 0) {
-          err_s = 1;
-          atomicOr(v.status, DS_TIMEOUT);
-        }
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&accfull), q & 1, err_s ? 1u : kWaitLimit))) {
+        if (lane == 0) fail();
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");

@@ -398,6 +398,8 @@ struct PrepSrc {
   int n;
   const unsigned char* pool;
   const int* pool_exp;
+  __device__ __forceinline__ int chain(int i) const { return jobs[i].ci; }
+  __device__ __forceinline__ bool takes(int) const { return true; }
   __device__ __forceinline__ int count(int i) const {
     const Dyn& d = *chains[jobs[i].ci].dyn;
     if (d.status || d.k_ins == 0 || d.n == 0) return 0;
@@ -437,6 +439,8 @@ struct NewSrc {
   const Chain<double>* chains;
   const SlicedView* views;
   int n;
+  __device__ __forceinline__ int chain(int i) const { return i; }
+  __device__ __forceinline__ bool takes(int i) const { return chains[i].sliced_new; }
   __device__ __forceinline__ int count(int i) const {
     const Dyn& d = *chains[i].dyn;
     if (!chains[i].sliced_new || d.status || d.k_ins == 0 || d.n == 0) return 0;
@@ -473,6 +477,8 @@ struct FlushSrc {
   const Chain<double>* chains;
   const SlicedView* views;
   int n;
+  __device__ __forceinline__ int chain(int i) const { return i; }
+  __device__ __forceinline__ bool takes(int i) const { return chains[i].sliced; }
   __device__ __forceinline__ int count(int i) const {
     const int nn = flush_rows(chains[i]);
     return 2 * ((nn + 127) / 128) * ((nn + 63) / 64);
@@ -504,6 +510,8 @@ struct YSrc {
   const Chain<double>* chains;
   const SlicedView* views;
   int n;
+  __device__ __forceinline__ int chain(int i) const { return i; }
+  __device__ __forceinline__ bool takes(int i) const { return chains[i].sliced_y; }
   __device__ __forceinline__ int count(int i) const {
     const int nn = chains[i].sliced_y ? flush_rows(chains[i]) : 0;
     return nn ? 2 * ((nn + 127) / 128) * ((chains[i].dyn->k_acc + 63) / 64) : 0;
@@ -533,12 +541,17 @@ struct YSrc {
   }
 };
 
+// A wait of more than wl polls gives up: the CTA stops, and every chain of the launch
+// gets DS_TIMEOUT, since the CTA may leave items of any of them undone and a CTA that
+// starts later finds other work lists.  With `stall` set (a test of this path) the MMA
+// issuer of CTA 0 first waits on a barrier that nothing completes, until the chain of
+// its first item has been recomputed twice.
 template <class Src, bool FLUSH>
-__global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src) {
+__global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src, uint32_t wl, int stall) {
   extern __shared__ __align__(1024) unsigned char prod_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)prod_raw + 1023) & ~(uintptr_t)1023);
   int* off = reinterpret_cast<int*>(base + kProdStages * kProdStageBytes);
-  __shared__ uint64_t full[kProdStages], empty[kProdStages], accfull, accempty, drain;
+  __shared__ uint64_t full[kProdStages], empty[kProdStages], accfull, accempty, drain, never;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int err_s;
   for (int i = threadIdx.x; i < src.n; i += blockDim.x) off[i] = src.count(i);
@@ -551,9 +564,10 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src) {
     const int i = find_chain(off, src.n, w);
     return src.item(i, w - off[i]);
   };
-  auto fail = [&](int ci) {
+  auto fail = [&]() {
     err_s = 1;
-    atomicOr(&src.chains[ci].dyn->status, DS_TIMEOUT);
+    for (int i = 0; i < src.n; ++i)
+      if (src.takes(i)) atomicOr(&src.chains[src.chain(i)].dyn->status, DS_TIMEOUT);
   };
 
   if (warp == 1) {
@@ -569,6 +583,7 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src) {
     mbar_init(smem_u32(&accfull), 1);
     mbar_init(smem_u32(&accempty), 16);
     mbar_init(smem_u32(&drain), 1);
+    mbar_init(smem_u32(&never), 1);
     err_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -585,7 +600,7 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src) {
       bool ok = true;
       for (int c = 0; c < t.chunks; ++c) {
         const uint32_t s = issued % kProdStages, use = issued / kProdStages;
-        ok = use == 0 || mbar_wait(smem_u32(empty + s), (use - 1) & 1);
+        ok = use == 0 || mbar_wait(smem_u32(empty + s), (use - 1) & 1, wl);
         if (!ok) break;
         const uint32_t fb = smem_u32(full + s), dst = smem_u32(base + s * kProdStageBytes);
         mbar_expect_tx(fb, kProdStageBytes);
@@ -594,7 +609,7 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src) {
         ++issued;
       }
       if (!ok) {
-        fail(t.ci);
+        fail();
         break;
       }
     }
@@ -604,14 +619,18 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src) {
   } else if (warp == 1) {   // all lanes wait, one issues
     uint32_t q = 0, taken = 0;
     bool ok = true;
+    if (stall && blockIdx.x == 0 && src.chains[item(0).ci].dyn->refreshes < 2)
+      ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&never), 0, wl));
+    if (!ok && lane == 0) fail();
+    __syncwarp();
     for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
       if (__any_sync(0xffffffffu, err_s != 0)) break;
       const ProdItem t = item(w);
       for (int c0 = 0; c0 < t.chunks && ok; c0 += 4, ++q) {
-        ok = __all_sync(0xffffffffu, q == 0 || mbar_wait(smem_u32(&accempty), (q - 1) & 1));
+        ok = __all_sync(0xffffffffu, q == 0 || mbar_wait(smem_u32(&accempty), (q - 1) & 1, wl));
         for (int c = c0; c < min(t.chunks, c0 + 4) && ok; ++c, ++taken) {
           const uint32_t s = taken % kProdStages;
-          ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(full + s), (taken / kProdStages) & 1));
+          ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(full + s), (taken / kProdStages) & 1, wl));
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t a = smem_u32(base + s * kProdStageBytes);
@@ -625,7 +644,8 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src) {
         if (ok && oz::elect_one()) mma_commit(smem_u32(&accfull));
         __syncwarp();
       }
-      if (!ok && lane == 0) fail(t.ci);
+      if (!ok && lane == 0) fail();
+      __syncwarp();
     }
     if (oz::elect_one()) mma_commit(smem_u32(&drain));   // every MMA issued completes before the TMEM is freed
     __syncwarp();
@@ -657,7 +677,7 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src) {
       bool ok = true;
       for (int c0 = 0; c0 < t.chunks; c0 += 4, ++q, ++pa, ++pb) {
         const int ea = *pa - 54;
-        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&accfull), q & 1, err_s ? 1u : kWaitLimit));
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&accfull), q & 1, err_s ? 1u : wl));
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         long long S[kProdCols];
@@ -682,7 +702,7 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src) {
         for (int e = 0; e < kProdCols; ++e) z[e] += oz::scaled_double(S[e], ea + pb[(size_t)e * t.es_b]);
       }
       if (!ok) {
-        if (lane == 0) fail(t.ci);
+        if (lane == 0) fail();
         break;
       }
       if constexpr (!FLUSH) {
@@ -753,6 +773,15 @@ cudaError_t configure_sliced() {
   return e;
 }
 
+namespace {
+template <class Src, bool FLUSH>
+void launch_product(const Src& src, const LaunchShape& ls, cudaStream_t st) {
+  const int lim = ls.tc_wait_limit;
+  const uint32_t wl = lim > 0 ? (uint32_t)lim : lim < 0 ? (uint32_t)(-(int64_t)lim) : kWaitLimit;
+  k_sliced_product<Src, FLUSH><<<ls.tc_ctas, kProdThreads, prod_smem(src.n), st>>>(src, wl, lim < 0 ? 1 : 0);
+}
+}  // namespace
+
 int launch_sliced_prep(const Chain<double>* dchains, const LaunchShape& ls, cudaStream_t st) {
   const SlicedPlan& p = ls.sliced;
   int n = 1;
@@ -763,12 +792,12 @@ int launch_sliced_prep(const Chain<double>* dchains, const LaunchShape& ls, cuda
     k_slice_n<<<ls.persist_ctas, 256, sizeof(int) * (sp.count + 1), st>>>(dchains, p.views, jobs, sp.count, p.pool,
                                                                          p.pool_exp);
     const PrepSrc src{dchains, p.views, jobs, sp.count, p.pool, p.pool_exp};
-    k_sliced_product<PrepSrc, false><<<ls.tc_ctas, kProdThreads, prod_smem(sp.count), st>>>(src);
+    launch_product<PrepSrc, false>(src, ls, st);
   }
   if (ls.any_sliced_new) {
     k_slice_g<<<ls.persist_ctas, 256, 0, st>>>(dchains, ls.n_chains, p.views);
     const NewSrc src{dchains, p.views, ls.n_chains};
-    k_sliced_product<NewSrc, false><<<ls.tc_ctas, kProdThreads, prod_smem(ls.n_chains), st>>>(src);
+    launch_product<NewSrc, false>(src, ls, st);
     n += 2;
   }
   return n;
@@ -778,14 +807,14 @@ int launch_sliced_y(const Chain<double>* dchains, const LaunchShape& ls, cudaStr
   k_balance_y<<<ls.persist_ctas, 256, 0, st>>>(dchains, ls.n_chains, ls.sliced.views);
   k_slice_y<<<ls.persist_ctas, 256, 0, st>>>(dchains, ls.n_chains, ls.sliced.views);
   const YSrc src{dchains, ls.sliced.views, ls.n_chains};
-  k_sliced_product<YSrc, false><<<ls.tc_ctas, kProdThreads, prod_smem(ls.n_chains), st>>>(src);
+  launch_product<YSrc, false>(src, ls, st);
   return 3;
 }
 
 int launch_sliced_flush(const Chain<double>* dchains, const LaunchShape& ls, cudaStream_t st) {
   k_slice_flush<<<ls.persist_ctas, 256, 0, st>>>(dchains, ls.n_chains, ls.sliced.views);
   const FlushSrc src{dchains, ls.sliced.views, ls.n_chains};
-  k_sliced_product<FlushSrc, true><<<ls.tc_ctas, kProdThreads, prod_smem(ls.n_chains), st>>>(src);
+  launch_product<FlushSrc, true>(src, ls, st);
   return 2;
 }
 
