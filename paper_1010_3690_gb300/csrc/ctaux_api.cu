@@ -34,6 +34,8 @@ struct ctaux_ctx {
   std::string err;
   int max_ld = 0;
   std::vector<SlicedStrip> strips;   // of ls.sliced
+  // arrival counters of a chain's split products (device address, bytes)
+  std::vector<std::vector<std::pair<void*, size_t>>> tickets;
   // CUDA graphs of one block (with its near-tie launch), of one measurement,
   // and of one block with the previous block's measurement beside it (on the
   // side stream), captured on first use on a private stream, with their
@@ -193,6 +195,7 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
         v.ce[pr] = reinterpret_cast<int*>(base + o[4 * pr + 1]);
         v.part[pr] = reinterpret_cast<double*>(base + o[4 * pr + 2]);
         v.ticket[pr] = reinterpret_cast<int*>(base + o[4 * pr + 3]);
+        ctx->tickets[ci].push_back({v.ticket[pr], o[4 * pr + 4] - o[4 * pr + 3]});
       }
       v.ys = base + o[8];
       v.xs = base + o[9];
@@ -204,6 +207,8 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
         v.ge = reinterpret_cast<int*>(base + o[14]);
         v.gpart = reinterpret_cast<double*>(base + o[15]);
         v.gticket = reinterpret_cast<int*>(base + o[16]);
+        const size_t tiles = (size_t)((hc[ci].k_max + 127) / 128) * ((hc[ci].k_max + 63) / 64);
+        ctx->tickets[ci].push_back({v.gticket, tiles * 16 * sizeof(int)});
       }
     }
   }
@@ -318,6 +323,7 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
     ls.tie_grid = ctx->sm_count;
     ls.tie_iters = P.tie_refine_iters == 0 ? 12 : std::max(0, P.tie_refine_iters);
   }
+  ctx->tickets.resize(ctx->chains.size());
   std::vector<TcMaps> host_maps(mixed_tc ? 2 * ctx->chains.size() : 0);
   // from-scratch recomputation: launch shapes for all chains and for one
   std::vector<int> lds;
@@ -410,6 +416,8 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
       c.ticket[spin] = dalloc<int>(ctx, kMaxPartials, &err);
       c.vpart[spin] = dalloc<T>(ctx, meas_v_partials(c.cap_m, P.n_anchors, sizeof(T) == 8), &err);
       c.vticket[spin] = dalloc<int>(ctx, meas_v_tickets(c.cap_m, P.n_anchors), &err);
+      ctx->tickets[ci].push_back({c.ticket[spin], kMaxPartials * sizeof(int)});
+      ctx->tickets[ci].push_back({c.vticket[spin], meas_v_tickets(c.cap_m, P.n_anchors) * sizeof(int)});
     }
     c.gamma_lu = P.gamma_form == CTAUX_GAMMA_LU ? 1 : 0;
     c.kp = round_up(cp.k_max, 32);
@@ -1028,6 +1036,10 @@ ctaux_status ctaux_set_config(ctaux_ctx* ctx, int chain, const double* tau, cons
     CUDA_TRY(ctx, cudaMemcpy(ds, s8.data(), n, cudaMemcpyHostToDevice));
     CUDA_TRY(ctx, cudaMemcpy(db, bv.data(), n * sizeof(int64_t), cudaMemcpyHostToDevice));
   }
+  // a chain that had stopped (a bounded wait that gave up, beside whose kernel others
+  // may have seen the status or not) can hold split products half arrived
+  if (d.status)
+    for (const auto& tk : ctx->tickets[chain]) CUDA_TRY(ctx, cudaMemset(tk.first, 0, tk.second));
   d.n = n;
   d.t = t;
   d.status = 0;

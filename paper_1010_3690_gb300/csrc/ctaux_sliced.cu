@@ -543,9 +543,10 @@ struct YSrc {
 
 // A wait of more than wl polls gives up: the CTA stops, and every chain of the launch
 // gets DS_TIMEOUT, since the CTA may leave items of any of them undone and a CTA that
-// starts later finds other work lists.  With `stall` set (a test of this path) the MMA
-// issuer of CTA 0 first waits on a barrier that nothing completes, until the chain of
-// its first item has been recomputed twice.
+// starts later finds other work lists (split-K arrivals are then incomplete;
+// ctaux_set_config clears them with the status).  With `stall` set (a test of this
+// path) the MMA issuer of CTA 0 first waits on a barrier that nothing completes, until
+// the chain of its first item has been recomputed twice.
 template <class Src, bool FLUSH>
 __global__ void __launch_bounds__(kProdThreads, 1) k_sliced_product(Src src, uint32_t wl, int stall) {
   extern __shared__ __align__(1024) unsigned char prod_raw[];

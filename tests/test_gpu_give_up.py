@@ -3,6 +3,7 @@ test setting of tc_wait_limit lets one CTA wait on a barrier that nothing comple
 """
 import dataclasses
 
+import numpy as np
 import pytest
 
 from workloads import configs
@@ -36,3 +37,31 @@ def test_every_chain_of_a_product_that_gave_up_reports_it(k, n_chains):
         _give_up(ctx, cfgs)
         assert all(ctx.stats(i)["status"] & 8 for i in range(n_chains))
         assert all(len(ctx.trace(i)) == 0 for i in range(n_chains))
+
+
+@pytest.mark.parametrize("k,n_chains", [(64, 1), (64, 8), (160, 2)])
+def test_chains_recover_from_a_product_that_gave_up(k, n_chains):
+    """After ctaux_set_config they go on as in a context where nothing happened: no
+    half-arrived split product is left."""
+    chains, cfgs = _chains(k, n_chains)
+    kw = dict(refresh_every=0, trace_capacity=4 * k)
+    with pk.Context(chains, **kw) as ctx:
+        for i, cfg in enumerate(cfgs):
+            ctx.set_config(i, **cfg)
+        ctx.sweep(3)
+        ctx.synchronize()
+        clean = [ctx.trace(i) for i in range(n_chains)]
+    with pk.Context(chains, tc_wait_limit=-20000, **kw) as ctx:
+        _give_up(ctx, cfgs)
+        for i, cfg in enumerate(cfgs):
+            try:
+                ctx.set_config(i, **cfg)
+            except pk.CtauxError as e:             # reports the chains that still wait
+                assert e.code == 7 and i + 1 < n_chains
+        ctx.sweep(3)
+        ctx.synchronize()
+        for i in range(n_chains):
+            tr = ctx.trace(i)
+            assert len(tr) == len(clean[i])
+            for name in tr.dtype.names:
+                np.testing.assert_array_equal(tr[name], clean[i][name])
