@@ -6,6 +6,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -325,11 +326,18 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
   }
   ctx->tickets.resize(ctx->chains.size());
   std::vector<TcMaps> host_maps(mixed_tc ? 2 * ctx->chains.size() : 0);
-  // from-scratch recomputation: launch shapes for all chains and for one
+  // from-scratch recomputation
+  InvDevice inv_dev{};
+  CUDA_TRY(ctx, inv_device(ctx->sm_count, false, &inv_dev));
   std::vector<int> lds;
-  for (const auto& cp : ctx->chains) lds.insert(lds.end(), 2, round_up(cp.capacity + cp.k_max, 32));
-  CUDA_TRY(ctx, inv_configure({max_ld, max_ld}, ctx->sm_count, false, &ls.inv_one));
-  CUDA_TRY(ctx, inv_configure(lds, ctx->sm_count, false, &ls.inv_all));
+  std::map<int, int> place;
+  for (const auto& cp : ctx->chains) {
+    const int ld = round_up(cp.capacity + cp.k_max, 32);
+    lds.insert(lds.end(), 2, ld);
+    if (place.emplace(ld, (int)ls.inv_one.size()).second) ls.inv_one.push_back(inv_shapes({ld, ld}, inv_dev)[0]);
+    ls.inv_one_of.push_back(place[ld]);
+  }
+  ls.inv_all = inv_shapes(lds, inv_dev);
   std::vector<InvView> host_views(items);
 
   for (size_t ci = 0; ci < ctx->chains.size(); ++ci) {
@@ -460,7 +468,8 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
     if (c.pcol) CUDA_TRY(ctx, cudaMemset(c.pcol, 0xFF, 2 * ld * sizeof(int)));
     for (int spin = 0; spin < 2; ++spin) {
       InvView& v = host_views[2 * ci + spin];
-      inv_layout(c.work + spin * refresh_work_one((int)ld), (int)ld, ls.inv_all.chunks, v);
+      inv_layout(c.work + spin * refresh_work_one((int)ld), (int)ld, inv_chunks((int)ld), v);
+      v.width = inv_width((int)ld, inv_dev);
       v.perm = c.perm + spin * ld;
       v.used = c.used + spin * ld;
       v.pcol = c.pcol + spin * ld;
@@ -510,7 +519,7 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
   }
   {
     InvView* dv = dalloc<InvView>(ctx, items, &err);
-    ls.inv_orders = dalloc<int>(ctx, items, &err);
+    ls.inv_orders = dalloc<int>(ctx, (size_t)items * (1 + ls.inv_all.size()), &err);
     if (err != cudaSuccess)
       return set_err(ctx, CTAUX_ENOMEM, "device allocation failed: %s", cudaGetErrorString(err));
     CUDA_TRY(ctx, cudaMemcpy(dv, host_views.data(), items * sizeof(InvView), cudaMemcpyHostToDevice));

@@ -32,7 +32,7 @@
 // (order 310: 773 -> 794 us).
 // N^{-1} = [e^V / (e^V - 1) - G0] (e^V - 1) has rows of one scale and goes without;
 // scaled columns cancel by themselves.
-// From order 1024 on, two levels: the rank-32 products of four panels stay
+// From leading dimension 1024 on (kInvTwoLevel), two levels: the rank-32 products of four panels stay
 // inside 128 columns, the rest of the matrix follows with one rank-128 product
 // (k_inv_cols slices the 128 columns).  That reads and writes X, and runs the
 // float64 epilogue, once per 128 columns instead of four times.
@@ -381,30 +381,43 @@ k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows
 struct InvRange {
   int c0, width, j0, j1;
 };
+// The columns of matrix i, of order m, in the product of rank 32 with the panel from c0
+// on: all, or the panel's own 128 in two levels.
+__device__ __forceinline__ InvRange inv_range(const InvView* views, const InvSet& set, int i, int m, int c0) {
+  const bool two = set.mixed ? views[i].chunks > 1 : set.two_level;
+  const int j0 = two ? c0 & ~127 : 0;
+  return InvRange{c0, set.width, j0, two ? min(m, j0 + 128) : m};
+}
+// Whether it takes part in the product of rank 128: not where no column lies outside.
+__device__ __forceinline__ bool inv_wide(const InvView* views, const InvSet& set, int i, int m, int c0) {
+  return m > c0 && m > 128 && (!set.mixed || views[i].chunks > 1);
+}
 
 // The pivot rows of the panel, in the columns of the range, as slice images: a
 // warp per column, a lane per pivot row.  Rank 32: y_k, the column at pivot row k
 // just before step k, y_k = X[R_k][j] + sum_{l<k} L[k][l] y_l; the panel's own
 // column c0 + k starts from the unit vector e_k.
 template <bool BALANCE>
-__global__ void __launch_bounds__(256) k_inv_rows(const InvView* views, const int* orders, int items,
-                                                  InvRange g) {
+__global__ void __launch_bounds__(256) k_inv_rows(const InvView* views, const int* orders, int items, InvSet set,
+                                                  int c0, bool wide) {
   __shared__ int off[2 * kMaxChains + 1];
   for (int i = threadIdx.x; i < items; i += blockDim.x) {
     const int m = orders[i];
-    off[i] = m > g.c0 ? (min(m, g.j1) - g.j0 + 7) / 8 : 0;
+    const InvRange g = inv_range(views, set, i, m, c0);
+    off[i] = wide ? (inv_wide(views, set, i, m, c0) ? (m + 7) / 8 : 0) : m > c0 ? (g.j1 - g.j0 + 7) / 8 : 0;
   }
   __syncthreads();
   block_exclusive_scan(off, items);
   const int total = off[items], lane = threadIdx.x & 31;
-  const bool wide = g.width > oz::kK;
   for (int u = blockIdx.x; u < total; u += gridDim.x) {
     const int it = find_chain(off, items, u);
     const InvView& v = views[it];
-    const int m = orders[it], bw = min(g.width, m - g.c0);
+    const int m = orders[it];
+    const InvRange g = wide ? InvRange{c0, 128, 0, m} : inv_range(views, set, it, m, c0);
+    const int bw = min(g.width, m - g.c0);
     const int j = g.j0 + (u - off[it]) * 8 + (threadIdx.x >> 5);
     const bool own = j >= g.c0 && j < g.c0 + bw;
-    if (j >= min(m, g.j1) || (wide && own)) continue;   // the whole warp
+    if (j >= g.j1 || (wide && own)) continue;   // the whole warp
     const int nc = (bw + oz::kK - 1) / oz::kK;
     double x[4];
     int mx = 0;
@@ -454,11 +467,13 @@ __global__ void __launch_bounds__(256) k_inv_rows(const InvView* views, const in
 // The columns [c0, c0 + 128) of X as slice images, one exponent per row: a CTA
 // stages 16 rows in shared memory, a thread then writes a 16-byte chunk of
 // every slice of a row.
-__global__ void __launch_bounds__(256) k_inv_cols(const InvView* views, const int* orders, int items, int c0) {
+__global__ void __launch_bounds__(256) k_inv_cols(const InvView* views, const int* orders, int items,
+                                                  InvSet set, int c0) {
   __shared__ int off[2 * kMaxChains + 1];
   __shared__ double xs[128][17];
   __shared__ int mxs[16];
-  for (int i = threadIdx.x; i < items; i += blockDim.x) off[i] = orders[i] > c0 ? (orders[i] + 15) / 16 : 0;
+  for (int i = threadIdx.x; i < items; i += blockDim.x)
+    off[i] = inv_wide(views, set, i, orders[i], c0) ? (orders[i] + 15) / 16 : 0;
   __syncthreads();
   block_exclusive_scan(off, items);
   const int total = off[items], r = threadIdx.x & 15, ch = threadIdx.x >> 4;
@@ -513,26 +528,29 @@ constexpr int kUpdStageBytes = oz::kImageA + oz::kImageB;
 struct UpdTile {
   int it, m, i0, j0;
 };
-__device__ __forceinline__ UpdTile upd_tile(const int* off, const int* orders, int items, int w, int j0) {
+template <bool WIDE>
+__device__ __forceinline__ UpdTile upd_tile(const int* off, const InvView* views, const int* orders, int items,
+                                            const InvSet& set, int w, int c0) {
   UpdTile t;
   t.it = find_chain(off, items, w);
   t.m = orders[t.it];
   const int tm = (t.m + 127) / 128, l = w - off[t.it];
   t.i0 = (l % tm) * 128;
-  t.j0 = j0 + (l / tm) * 64;
+  t.j0 = (WIDE ? 0 : inv_range(views, set, t.it, t.m, c0).j0) + (l / tm) * 64;
   return t;
 }
 
 // WIDE: rank 128 (up to four image pairs per tile), else rank 32.
 template <bool WIDE>
 __global__ void __launch_bounds__(kUpdThreads, 1)
-k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
+k_inv_update(const InvView* views, const int* orders, int items, InvSet set, int c0) {
   using namespace tc;
   __shared__ int off[2 * kMaxChains + 1];
   for (int i = threadIdx.x; i < items; i += blockDim.x) {
-    const int m = orders[i];
-    const int cols = min(m, g.j1) - g.j0;
-    off[i] = m > g.c0 && !(WIDE && cols <= min(g.width, m - g.c0)) ? ((m + 127) / 128) * ((cols + 63) / 64) : 0;
+    const int m = orders[i], tm = (m + 127) / 128;
+    const InvRange g = inv_range(views, set, i, m, c0);
+    off[i] = WIDE ? (inv_wide(views, set, i, m, c0) ? tm * ((m + 63) / 64) : 0)
+                  : m > c0 ? tm * ((g.j1 - g.j0 + 63) / 64) : 0;
   }
   __syncthreads();
   block_exclusive_scan(off, items);
@@ -576,9 +594,9 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
 
   if (warp == 0 && lane == 0) {
     for (int w = blockIdx.x; w < total && !err_s; w += gridDim.x) {
-      const UpdTile t = upd_tile(off, orders, items, w, g.j0);
+      const UpdTile t = upd_tile<WIDE>(off, views, orders, items, set, w, c0);
       const InvView& v = views[t.it];
-      const int nc = WIDE ? (min(g.width, t.m - g.c0) + oz::kK - 1) / oz::kK : 1;
+      const int nc = WIDE ? (min(128, t.m - c0) + oz::kK - 1) / oz::kK : 1;
       const unsigned char* sa = v.As + (size_t)(t.i0 >> 7) * v.chunks * oz::kImageA;
       const unsigned char* sb = v.Bs + (size_t)(t.j0 >> 6) * v.chunks * oz::kImageB;
       bool ok = true;
@@ -604,8 +622,8 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
     uint32_t q = 0, taken = 0;
     for (int w = blockIdx.x; w < total; w += gridDim.x, ++q) {
       if (__any_sync(0xffffffffu, err_s != 0)) break;
-      const UpdTile t = upd_tile(off, orders, items, w, g.j0);
-      const int nc = WIDE ? (min(g.width, t.m - g.c0) + oz::kK - 1) / oz::kK : 1;
+      const UpdTile t = upd_tile<WIDE>(off, views, orders, items, set, w, c0);
+      const int nc = WIDE ? (min(128, t.m - c0) + oz::kK - 1) / oz::kK : 1;
       bool ok = __all_sync(0xffffffffu, q == 0 || mbar_wait(smem_u32(&accempty), (q - 1) & 1));
       for (int c = 0; c < nc && ok; ++c, ++taken) {
         const uint32_t s = taken % kUpdStages;
@@ -634,10 +652,11 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
     const int quarter = warp & 3, group = (warp - 2) >> 2;
     uint32_t q = 0;
     for (int w = blockIdx.x; w < total; w += gridDim.x, ++q) {
-      const UpdTile t = upd_tile(off, orders, items, w, g.j0);
+      const UpdTile t = upd_tile<WIDE>(off, views, orders, items, set, w, c0);
       const InvView& v = views[t.it];
+      const InvRange g = WIDE ? InvRange{c0, 128, 0, t.m} : inv_range(views, set, t.it, t.m, c0);
       const int ld = v.ld, i = t.i0 + quarter * 32 + lane, jb = t.j0 + group * kUpdCols;
-      const int cn = min(g.c0 + g.width, t.m), je = min(g.j1, t.m);
+      const int cn = min(g.c0 + g.width, t.m), je = g.j1;
       const bool row_ok = i < t.m;
       const int pci = row_ok ? v.pcol[i] : -1;
       const bool load = row_ok && !(pci >= g.c0 && pci < cn);   // pivot rows start from zero
@@ -693,6 +712,7 @@ k_inv_update(const InvView* views, const int* orders, int items, InvRange g) {
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }
 
+constexpr int kPanelSmem = 220 * 1024;
 constexpr int upd_smem() { return kUpdStages * kUpdStageBytes + 1024; }
 
 int panel_smem_bytes(int width, int rows, bool balance) {
@@ -709,106 +729,112 @@ int panel_smem_bytes(int width, int rows, bool balance) {
 // to order 1084: 13.0 ms, 14.3 with 4; larger clusters pay where a batch's last,
 // largest matrices are left), 4 beyond 256 matrices, whose rows fill the float64
 // pipes of all SMs anyway.
-cudaError_t inv_configure(const std::vector<int>& lds, int sm_count, bool balance, InvShape* out) {
-  InvShape s{};
-  s.sm_count = sm_count;
-  s.balance = balance;
-  int max_ld = 1;
-  for (int ld : lds) max_ld = ld > max_ld ? ld : max_ld;
-  s.chunks = inv_chunks(max_ld);
+cudaError_t inv_device(int sm_count, bool balance, InvDevice* out) {
+  *out = InvDevice{sm_count, 16, balance};
   auto attrs = [&](auto* fn, int bytes) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    return e;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   };
-  const int most = 220 * 1024;
   auto* panel512 = balance ? k_inv_panel<512, true> : k_inv_panel<512, false>;
   auto* panel256 = balance ? k_inv_panel<256, true> : k_inv_panel<256, false>;
   cudaError_t e = cudaFuncSetAttribute(panel512, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess) e = attrs(panel512, most);
-  if (e == cudaSuccess) e = attrs(panel256, most);
+  if (e == cudaSuccess) e = attrs(panel512, kPanelSmem);
+  if (e == cudaSuccess) e = attrs(panel256, kPanelSmem);
   if (e == cudaSuccess) e = attrs(k_inv_update<false>, upd_smem());
   if (e == cudaSuccess) e = attrs(k_inv_update<true>, upd_smem());
   if (e != cudaSuccess) return e;
-  auto smem_of = [&](int cluster) { return panel_smem_bytes(s.width, (max_ld + cluster - 1) / cluster, balance); };
   // 16 CTAs need a GPC with that many free SMs
-  int largest = 16;
-  {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(16);
-    cfg.blockDim = dim3(512);
-    cfg.dynamicSmemBytes = most;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = 16;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, panel512, &cfg);
-    if (e != cudaSuccess) return e;
-    if (n == 0) largest = 8;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(16);
+  cfg.blockDim = dim3(512);
+  cfg.dynamicSmemBytes = kPanelSmem;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 16;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  e = cudaOccupancyMaxActiveClusters(&n, panel512, &cfg);
+  if (n == 0) out->largest = 8;
+  return e;
+}
+
+int inv_width(int ld, const InvDevice& dev) {
+  int width = kMaxWidth;
+  while (width > 4 && panel_smem_bytes(width, (ld + dev.largest - 1) / dev.largest, dev.balance) > kPanelSmem) width /= 2;
+  return width;
+}
+
+std::vector<InvShape> inv_shapes(const std::vector<int>& lds, const InvDevice& dev) {
+  std::vector<InvShape> out;
+  for (int width = kMaxWidth; width >= 4; width /= 2) {
+    InvShape s{dev, InvSet{width, false, false}, false, {}};
+    int max_ld = 0;
+    for (int ld : lds)
+      if (inv_width(ld, dev) == width) {
+        max_ld = ld > max_ld ? ld : max_ld;
+        (inv_chunks(ld) > 1 ? s.set.two_level : s.one_level) = true;
+      }
+    if (max_ld == 0) continue;
+    s.set.mixed = s.set.two_level && s.one_level;
+    auto smem_of = [&](int cluster) { return panel_smem_bytes(width, (max_ld + cluster - 1) / cluster, dev.balance); };
+    for (int c0 = 0; c0 < max_ld; c0 += width) {
+      int active = 0;
+      for (int ld : lds) active += ld > c0 && inv_width(ld, dev) == width;
+      int cl = active <= 8 ? dev.largest : active <= 256 ? 8 : 4;
+      while (cl < dev.largest && smem_of(cl) > kPanelSmem) cl *= 2;
+      s.panels.push_back(InvPanel{cl, cl == 16 ? 512 : 256, (max_ld + cl - 1) / cl, smem_of(cl)});
+    }
+    out.push_back(s);
   }
-  s.width = kMaxWidth;
-  while (s.width > 4 && smem_of(largest) > most) s.width /= 2;
-  for (int c0 = 0; c0 < max_ld; c0 += s.width) {
-    int active = 0;
-    for (int ld : lds) active += ld > c0;
-    int cl = active <= 8 ? largest : active <= 256 ? 8 : 4;
-    while (cl < largest && smem_of(cl) > most) cl *= 2;
-    s.panels.push_back(InvPanel{cl, cl == 16 ? 512 : 256, (max_ld + cl - 1) / cl, smem_of(cl)});
-  }
-  *out = s;
-  return cudaSuccess;
+  return out;
 }
 
 int launch_inverse(const InvView* views, const int* orders, int items, int max_order,
                    const InvShape& sh, cudaStream_t st, cudaError_t* err) {
   int n = 0;
+  const int reach = (int)sh.panels.size() * sh.set.width;   // no order of this set is above it
+  max_order = max_order < reach ? max_order : reach;
   auto grid = [&](long units, long most) { return (int)(units < most ? units : most); };
-  const long rb = (max_order + 127) / 128, sms = sh.sm_count;
-  // the product of panel [c0, c0 + width) with the columns [j0, j1)
-  auto update = [&](int c0, int width, int j0, int j1) {
-    const InvRange g{c0, width, j0, j1};
-    const long cols = (j1 < max_order ? j1 : max_order) - j0;
-    auto* rows = sh.balance ? k_inv_rows<true> : k_inv_rows<false>;
-    rows<<<grid(items * ((cols + 7) / 8), 8 * sms), 256, 0, st>>>(views, orders, items, g);
+  const long rb = (max_order + 127) / 128, sms = sh.dev.sm_count;
+  // the product of the panel from c0 on with up to `cols` columns of a matrix
+  auto update = [&](int c0, bool wide, long cols) {
+    auto* rows = sh.dev.balance ? k_inv_rows<true> : k_inv_rows<false>;
+    rows<<<grid(items * ((cols + 7) / 8), 8 * sms), 256, 0, st>>>(views, orders, items, sh.set, c0, wide);
     const int ug = grid(items * rb * ((cols + 63) / 64), sms);
-    if (width > oz::kK) k_inv_update<true><<<ug, kUpdThreads, upd_smem(), st>>>(views, orders, items, g);
-    else k_inv_update<false><<<ug, kUpdThreads, upd_smem(), st>>>(views, orders, items, g);
+    if (wide) k_inv_update<true><<<ug, kUpdThreads, upd_smem(), st>>>(views, orders, items, sh.set, c0);
+    else k_inv_update<false><<<ug, kUpdThreads, upd_smem(), st>>>(views, orders, items, sh.set, c0);
     n += 2;
   };
-  const int outer = sh.chunks == 4 ? 128 : sh.width;
-  for (int o0 = 0; o0 < max_order; o0 += outer) {
-    for (int c0 = o0; c0 < o0 + outer && c0 < max_order; c0 += sh.width) {
-      const InvPanel& pn = sh.panels[c0 / sh.width];
-      cudaLaunchConfig_t cfg{};
-      cfg.gridDim = dim3((unsigned)(items * pn.cluster));
-      cfg.blockDim = dim3((unsigned)pn.threads);
-      cfg.dynamicSmemBytes = (size_t)pn.smem;
-      cfg.stream = st;
-      cudaLaunchAttribute at{};
-      at.id = cudaLaunchAttributeClusterDimension;
-      at.val.clusterDim.x = (unsigned)pn.cluster;
-      at.val.clusterDim.y = at.val.clusterDim.z = 1;
-      cfg.attrs = &at;
-      cfg.numAttrs = 1;
-      auto* fn = pn.threads == 512 ? (sh.balance ? k_inv_panel<512, true> : k_inv_panel<512, false>)
-                                   : (sh.balance ? k_inv_panel<256, true> : k_inv_panel<256, false>);
-      const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, views, orders, c0, sh.width, pn.rows);
-      n += 1;
-      if (e != cudaSuccess) {
-        *err = e;
-        return n;
-      }
-      update(c0, sh.width, outer > sh.width ? o0 : 0, outer > sh.width ? o0 + outer : max_order);
+  for (int c0 = 0; c0 < max_order; c0 += sh.set.width) {
+    const InvPanel& pn = sh.panels[c0 / sh.set.width];
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(items * pn.cluster));
+    cfg.blockDim = dim3((unsigned)pn.threads);
+    cfg.dynamicSmemBytes = (size_t)pn.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)pn.cluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    auto* fn = pn.threads == 512 ? (sh.dev.balance ? k_inv_panel<512, true> : k_inv_panel<512, false>)
+                                 : (sh.dev.balance ? k_inv_panel<256, true> : k_inv_panel<256, false>);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, views, orders, c0, sh.set.width, pn.rows);
+    n += 1;
+    if (e != cudaSuccess) {
+      *err = e;
+      return n;
     }
-    if (outer == sh.width) continue;
-    if (max_order <= outer) continue;   // no columns outside the panel
-    if (sh.chunks == 4) {
-      k_inv_cols<<<grid(items * ((max_order + 15) / 16), 8 * sms), 256, 0, st>>>(views, orders, items, o0);
+    const int o0 = c0 / 128 * 128, next = c0 + sh.set.width;
+    update(c0, false, sh.one_level ? max_order : max_order - o0 < 128 ? max_order - o0 : 128);
+    // the rank-128 product, unless no column lies outside the panel
+    if (sh.set.two_level && max_order > 128 && (next % 128 == 0 || next >= max_order)) {
+      k_inv_cols<<<grid(items * ((max_order + 15) / 16), 8 * sms), 256, 0, st>>>(views, orders, items, sh.set, o0);
       n += 1;
+      update(o0, true, max_order);
     }
-    update(o0, outer, 0, max_order);
   }
   *err = cudaGetLastError();
   return n;

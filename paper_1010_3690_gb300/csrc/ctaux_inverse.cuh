@@ -14,6 +14,7 @@ struct InvView {
   double* X;            // the matrix, column-major, leading dimension ld
   int ld;
   int chunks;           // images per row block: 1, or 4 (panels of 128 columns in two levels)
+  int width;            // panel width
   unsigned char* As;    // slice images of the panel's columns: ceil(ld / 128) x chunks x oz::kImageA
   unsigned char* Bs;    // slice images of the pivot rows: ceil(ld / 64) x chunks x oz::kImageB
   int* ea;              // row exponents of the images
@@ -28,14 +29,17 @@ struct InvView {
   int* status;          // DS_SINGULAR and DS_TIMEOUT bits
 };
 
-// Panels of 128 columns in two levels (see ctaux_inverse.cu) where the largest
-// leading dimension of a launch is at least this: the five extra launches per
-// 128 columns against three of four passes over the matrix.  One level against
-// two, ms per recomputation of one chain: 2.29 / 2.49 at order 700, 3.19 / 3.29
-// at 900, 4.44 / 4.46 at 1100, 6.51 / 6.23 at 1500, 10.9 / 9.6 at 2000 (leading
-// dimensions a quarter above the order).
-constexpr int kInvTwoLevel = 1408;
-inline int inv_chunks(int max_ld) { return max_ld >= kInvTwoLevel ? 4 : 1; }
+// Panels of 128 columns in two levels (see ctaux_inverse.cu) for matrices whose
+// leading dimension is at least this, whatever else is in the launch (a chain gives
+// the same bits alone or in a batch): the five extra launches per 128 columns against
+// three of four passes over the matrix.  One level against two, ms per recomputation
+// of one chain: 2.29 / 2.49 at order 700, 3.19 / 3.29 at 900, 4.44 / 4.46 at 1100, 6.51
+// / 6.23 at 1500, 10.9 / 9.6 at 2000 (leading dimensions a quarter above the order).
+// In a batch the passes cost more and the launches less: 96 chains up to order 1084,
+// 8 blocks with one recomputation, 32.9 ms with the line at 1408, 31.7 at 1024, 31.6
+// at 512, where one chain of order 431 takes a tenth longer.
+constexpr int kInvTwoLevel = 1024;
+inline int inv_chunks(int ld) { return ld >= kInvTwoLevel ? 4 : 1; }
 
 // Doubles of As, Bs, ea, eb and piv for a leading dimension (the matrix itself
 // comes first and takes ld^2 doubles).
@@ -65,6 +69,17 @@ __host__ __device__ inline int inv_column(int status, int singular, const int* p
   return (status & ~singular) ? j : perm[j];
 }
 
+// What the launches need to know of the device; sets the kernels up.  balance: for
+// matrices whose rows may differ in scale (one level only); their views then have
+// room for it.
+struct InvDevice {
+  int sm_count;
+  int largest;     // CTAs of the largest cluster
+  bool balance;
+};
+cudaError_t inv_device(int sm_count, bool balance, InvDevice* out);
+int inv_width(int ld, const InvDevice& dev);   // 32; less where a panel would not fit
+
 // Launch parameters of the inversion of a set of matrices.
 struct InvPanel {
   int cluster;     // CTAs of a matrix's cluster (2 to 16)
@@ -72,16 +87,21 @@ struct InvPanel {
   int rows;        // panel rows per CTA at the largest leading dimension
   int smem;        // dynamic shared memory
 };
+// What the matrices of a launch have in common: the panel width, and whether they go in
+// one level or two (mixed: each matrix says so itself).
+struct InvSet {
+  int width;
+  bool two_level, mixed;
+};
 struct InvShape {
-  int width;                     // panel width (32; 16 or 8 where a panel would not fit)
-  int chunks;                    // 4: two levels
-  int sm_count;
-  bool balance;
+  InvDevice dev;
+  InvSet set;
+  bool one_level;                // some matrix has one level
   std::vector<InvPanel> panels;  // of each panel: fewer matrices reach the later ones
 };
-// lds: the leading dimension of every matrix.  balance: for matrices whose rows may
-// differ in scale (one level only); their views then have room for it.
-cudaError_t inv_configure(const std::vector<int>& lds, int sm_count, bool balance, InvShape* out);
+// lds: the leading dimension of every matrix.  One shape for each panel width among them,
+// nearly always one in all.
+std::vector<InvShape> inv_shapes(const std::vector<int>& lds, const InvDevice& dev);
 
 // Inverts the matrices views[0..items) of orders orders[0..items) (device; 0 =
 // leave out), none above max_order: afterwards inv[c][perm[j]] = X[perm[c]][j].

@@ -129,8 +129,11 @@ struct LaunchShape {
   int meas_cb_blocks;
   int meas_acc_blocks;   // one warp per (class, bin) output
   const InvView* inv_views;   // [chain][spin] matrices of the from-scratch recomputation (device)
-  int* inv_orders;            // [chain][spin] their orders, written by each recomputation
-  InvShape inv_all, inv_one;  // its launch shapes: every chain, one chain
+  int* inv_orders;            // [chain][spin] their orders, written by each recomputation; then,
+                              // for each of several shapes, the orders of its matrices
+  std::vector<InvShape> inv_all;  // its launch shapes for every chain
+  std::vector<InvShape> inv_one;  // and for one chain alone, by leading dimension
+  std::vector<int> inv_one_of;    // [chain] place in inv_one
   int use_tc;            // mixed form: flush on the tensor cores
   int tc_ctas;           // persistent grid of the tensor-core flush (one CTA per SM)
   int split_x_blocks;

@@ -136,7 +136,6 @@ struct DeviceSetup {
   std::once_flag once;
   cudaError_t err = cudaSuccess;
   unsigned char* scratch = nullptr;  // device address of g_noalloc_scratch
-  int sms = 0;
   InvShape shape;
 };
 constexpr int kMaxDevices = 64;
@@ -156,12 +155,16 @@ extern "C" ctaux_status ctaux_invert_noalloc(const double* d_a, int lda, double*
   // array is only a stand-in, so resolve its device address here
   std::call_once(s.once, [&s, dev]() {
     s.err = cudaGetSymbolAddress(reinterpret_cast<void**>(&s.scratch), g_noalloc_scratch);
-    if (s.err == cudaSuccess) s.err = cudaDeviceGetAttribute(&s.sms, cudaDevAttrMultiProcessorCount, dev);
-    if (s.err == cudaSuccess) s.err = inv_configure({kM}, s.sms, true, &s.shape);
+    int sms = 0;
+    InvDevice d{};
+    if (s.err == cudaSuccess) s.err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (s.err == cudaSuccess) s.err = inv_device(sms, true, &d);
+    if (s.err == cudaSuccess) s.shape = inv_shapes({kM}, d)[0];
   });
   if (s.err != cudaSuccess || !s.scratch) return CTAUX_ECUDA;
   InvView v{};
   inv_layout(reinterpret_cast<double*>(s.scratch), kM, 1, v);
+  v.width = inv_width(kM, s.shape.dev);
   v.perm = reinterpret_cast<int*>(s.scratch + kPerm);
   v.pcol = reinterpret_cast<int*>(s.scratch + kPcol);
   v.used = reinterpret_cast<int8_t*>(s.scratch + kUsed);

@@ -11,15 +11,22 @@ namespace ctaux {
 
 namespace {
 
-// Orders of the matrices (chain, spin) that take part: all chains, or one.
+// Orders of the matrices (chain, spin) that take part: all chains, or one.  With
+// several panel widths, those of each as well.
+struct InvWidths {
+  int count, w[4];
+};
 template <typename T>
-__global__ void k_refresh_orders(const Chain<T>* chains, int n_chains, int only_chain, int* orders) {
+__global__ void k_refresh_orders(const Chain<T>* chains, int n_chains, int only_chain, int* orders,
+                                 const InvView* views, InvWidths widths) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 2 * n_chains) return;
   const int ci = i >> 1;
   const Dyn& d = *chains[ci].dyn;
   const bool take = (only_chain < 0 || only_chain == ci) && !(d.status & ~DS_SINGULAR);
   orders[i] = take ? d.n : 0;
+  for (int s = 0; s < widths.count; ++s)
+    orders[(size_t)(1 + s) * 2 * n_chains + i] = take && views[i].width == widths.w[s] ? d.n : 0;
 }
 
 // N^{-1} into X: kBuildCols columns by kBuildRows rows per CTA and unit, so that
@@ -138,7 +145,10 @@ cudaError_t launch_refresh(Chain<T>* dchains, const LaunchShape& ls, int only_ch
                            cudaStream_t st, PhaseTimer* pt) {
   pt->begin(6, st);
   const int items = 2 * ls.n_chains, nch = ls.n_chains;
-  k_refresh_orders<T><<<(items + 127) / 128, 128, 0, st>>>(dchains, nch, only_chain, ls.inv_orders);
+  InvWidths widths{};
+  if (only_chain < 0 && ls.inv_all.size() > 1)
+    for (const InvShape& sh : ls.inv_all) widths.w[widths.count++] = sh.set.width;
+  k_refresh_orders<T><<<(items + 127) / 128, 128, 0, st>>>(dchains, nch, only_chain, ls.inv_orders, ls.inv_views, widths);
   // one chain: only its two matrices
   const int first = only_chain >= 0 ? 2 * only_chain : 0, count = only_chain >= 0 ? 2 : items;
   const InvView* views = ls.inv_views + first;
@@ -146,7 +156,13 @@ cudaError_t launch_refresh(Chain<T>* dchains, const LaunchShape& ls, int only_ch
   const Chain<T>* chains = dchains + first / 2;
   k_refresh_build<T><<<ls.persist_ctas, 256, 0, st>>>(chains, views, orders, count);
   cudaError_t e = cudaSuccess;
-  const int n = launch_inverse(views, orders, count, max_order, only_chain >= 0 ? ls.inv_one : ls.inv_all, st, &e);
+  int n = 0;
+  if (only_chain >= 0) {
+    n = launch_inverse(views, orders, count, max_order, ls.inv_one[ls.inv_one_of[only_chain]], st, &e);
+  } else {
+    for (size_t s = 0; s < ls.inv_all.size() && e == cudaSuccess; ++s)
+      n += launch_inverse(views, widths.count ? orders + (1 + s) * items : orders, count, max_order, ls.inv_all[s], st, &e);
+  }
   if (e == cudaSuccess) {
     k_refresh_store<T><<<ls.persist_ctas, 256, 0, st>>>(chains, views, orders, count);
     k_refresh_finish<T><<<only_chain >= 0 ? 1 : nch, 256, 0, st>>>(dchains, ls.inv_views, ls.inv_orders, only_chain);
