@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -34,6 +35,23 @@ struct ctaux_ctx {
   int blocks_since_refresh = 0;
   std::string err;
   int max_ld = 0;
+  // What the host knows of the orders, without waiting: a recomputation is launched
+  // panel by panel, up to a bound on the largest order (order_bound).  An order grows
+  // by at most k_max per block, so it is bounded by one seen earlier and the blocks
+  // launched since: the one last read or set here, or the one that the device wrote
+  // when the last recomputation that it reached began (`seen`, mapped host memory:
+  // number of the recomputation << 32 | order).
+  struct KnownOrder {
+    int n = 0;
+    long long blocks = 0;      // launched when the order was n
+    uint32_t refresh = 0;      // recomputations launched by then: older entries of `seen` do not hold
+  };
+  std::vector<KnownOrder> known;
+  long long blocks = 0;        // launched
+  uint32_t refreshes = 0;      // launched, of every chain
+  std::vector<long long> blocks_at = std::vector<long long>(1024, 0);   // blocks before a recomputation
+  unsigned long long* seen = nullptr;
+  bool captured = false;       // a caller's graph may replay blocks: nothing is known
   std::vector<SlicedStrip> strips;   // of ls.sliced
   // arrival counters of a chain's split products (device address, bytes)
   std::vector<std::vector<std::pair<void*, size_t>>> tickets;
@@ -546,14 +564,50 @@ ctaux_status build_chains(ctaux_ctx* ctx) {
   return CTAUX_OK;
 }
 
+// The host has read or set a chain's order, with no block in flight.
+void note_order(ctaux_ctx* ctx, int chain, int n) {
+  ctx->known[chain] = ctaux_ctx::KnownOrder{n, ctx->blocks, ctx->refreshes};
+}
+
+// No chain's order is above this when a recomputation launched now begins.
+int order_bound(ctaux_ctx* ctx) {
+  if (ctx->captured) return ctx->max_ld;
+  long long most = 0;
+  for (size_t ci = 0; ci < ctx->chains.size(); ++ci) {
+    const ctaux_chain_params& cp = ctx->chains[ci];
+    const ctaux_ctx::KnownOrder& kn = ctx->known[ci];
+    long long b = kn.n + cp.k_max * (ctx->blocks - kn.blocks);
+    if (ctx->seen) {
+      const unsigned long long w = *(volatile unsigned long long*)(ctx->seen + ci);
+      const uint32_t r = (uint32_t)(w >> 32);
+      if (r > kn.refresh && ctx->refreshes - r < ctx->blocks_at.size())
+        b = std::min(b, (long long)(uint32_t)w + cp.k_max * (ctx->blocks - ctx->blocks_at[r % ctx->blocks_at.size()]));
+    }
+    most = std::max(most, std::min(b, (long long)cp.capacity + cp.k_max));
+  }
+  return (int)most;
+}
+
+// A caller that captures the stream replays what is launched now as often as it likes.
+void note_capture(ctaux_ctx* ctx, cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    cs = cudaStreamCaptureStatusActive;
+  }
+  if (cs != cudaStreamCaptureStatusNone) ctx->captured = true;
+}
+
 ctaux_status check_device_status(ctaux_ctx* ctx) {
   const bool mixed = is_mixed(ctx);
   int drift_chain = -1;
   double drift_rel = 0.0;
   for (size_t ci = 0; ci < ctx->chains.size(); ++ci) {
     Dyn* dp = mixed ? ctx->hc32[ci].dyn : ctx->hc64[ci].dyn;
-    int st = 0;
-    CUDA_TRY(ctx, cudaMemcpy(&st, &dp->status, sizeof(int), cudaMemcpyDeviceToHost));
+    int head[offsetof(Dyn, status) / sizeof(int) + 1];   // n to status
+    CUDA_TRY(ctx, cudaMemcpy(head, dp, sizeof(head), cudaMemcpyDeviceToHost));
+    const int st = head[offsetof(Dyn, status) / sizeof(int)];
+    note_order(ctx, (int)ci, head[offsetof(Dyn, n) / sizeof(int)]);
     if (st & DS_CAPACITY)
       return set_err(ctx, CTAUX_ECAPACITY, "chain %zu: expansion order + k_max exceeded the capacity", ci);
     if (st & DS_SINGULAR)
@@ -586,13 +640,25 @@ Dyn* dyn_of(ctaux_ctx* ctx, int chain) {
 ctaux_status read_dyn(ctaux_ctx* ctx, int chain, Dyn* out) {
   CUDA_TRY(ctx, cudaStreamSynchronize(ctx->last_stream));
   CUDA_TRY(ctx, cudaMemcpy(out, dyn_of(ctx, chain), sizeof(Dyn), cudaMemcpyDeviceToHost));
+  note_order(ctx, chain, out->n);
   return CTAUX_OK;
 }
 
+// Of every chain (only_chain < 0), or of one whose order the host has just set.
 template <typename T>
-ctaux_status do_refresh(ctaux_ctx* ctx, int only_chain, int max_order, cudaStream_t st) {
+ctaux_status do_refresh(ctaux_ctx* ctx, int only_chain, cudaStream_t st) {
+  note_capture(ctx, st);
+  RefreshOrders ro{order_bound(ctx), 0, nullptr};
+  if (only_chain >= 0) {
+    ro.bound = ctx->known[only_chain].n;
+  } else if (ctx->seen) {
+    ctx->refreshes += 1;
+    ctx->blocks_at[ctx->refreshes % ctx->blocks_at.size()] = ctx->blocks;
+    ro.number = ctx->refreshes;
+    ro.seen = ctx->seen;
+  }
   cudaError_t e = launch_refresh<T>(reinterpret_cast<Chain<T>*>(ctx->chains_dev), ctx->ls, only_chain,
-                                    max_order, st, ctx->timer);
+                                    ro, st, ctx->timer);
   if (e != cudaSuccess) return set_err(ctx, CTAUX_ECUDA, "refresh launch: %s", cudaGetErrorString(e));
   return CTAUX_OK;
 }
@@ -674,6 +740,7 @@ ctaux_status do_sweeps(ctaux_ctx* ctx, int n_sweeps, int measure, cudaStream_t s
   // runs beside block s + 1, also across calls; it is left pending after the
   // last block, and launched alone (n_sweeps = 0) before any other entry point
   // reads or changes the state
+  note_capture(ctx, st);
   const bool can_fold = graphs && ctx->side_stream != nullptr;
   bool pend = ctx->meas_pending;
   ctx->meas_pending = false;
@@ -686,9 +753,10 @@ ctaux_status do_sweeps(ctaux_ctx* ctx, int n_sweeps, int measure, cudaStream_t s
     cudaError_t e = pend ? run(2, block_meas) : run(0, block);
     pend = false;
     if (e != cudaSuccess) return set_err(ctx, CTAUX_ECUDA, "block launch: %s", cudaGetErrorString(e));
+    ctx->blocks += 1;
     ctx->blocks_since_refresh += 1;
     if (ctx->params.refresh_every > 0 && ctx->blocks_since_refresh >= ctx->params.refresh_every) {
-      ctaux_status r = do_refresh<T>(ctx, -1, ctx->max_ld, st);
+      ctaux_status r = do_refresh<T>(ctx, -1, st);
       if (r != CTAUX_OK) return r;
       ctx->blocks_since_refresh = 0;
     }
@@ -755,6 +823,7 @@ ctaux_status ctaux_init(const ctaux_params* params, ctaux_ctx** out) {
   ctx->params = *params;
   ctx->chains.assign(params->chains, params->chains + params->n_chains);
   ctx->params.chains = nullptr;
+  ctx->known.resize(ctx->chains.size());
   ctx->device = params->device;
   cudaError_t e = cudaSetDevice(ctx->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, ctx->device);
@@ -767,6 +836,12 @@ ctaux_status ctaux_init(const ctaux_params* params, ctaux_ctx** out) {
   if (st != CTAUX_OK) {
     ctaux_destroy(ctx);
     return st;
+  }
+  if (cudaHostAlloc((void**)&ctx->seen, ctx->chains.size() * sizeof(*ctx->seen), cudaHostAllocMapped) == cudaSuccess) {
+    std::fill(ctx->seen, ctx->seen + ctx->chains.size(), 0ull);
+  } else {   // the bounds then rest on what the host reads
+    cudaGetLastError();
+    ctx->seen = nullptr;
   }
   ctx->timer = new PhaseTimer();
   for (int i = 0; i < PhaseTimer::kPool; ++i) cudaEventCreate(&ctx->timer->ev[i]);
@@ -906,8 +981,8 @@ ctaux_status ctaux_reset_measurements(ctaux_ctx* ctx) {
 ctaux_status ctaux_recompute(ctaux_ctx* ctx, double* drift_max_out) {
   if (!ctx) return CTAUX_EINVAL;
   FLUSH_PENDING(ctx);
-  ctaux_status r = is_mixed(ctx) ? do_refresh<float>(ctx, -1, ctx->max_ld, ctx->last_stream)
-                                 : do_refresh<double>(ctx, -1, ctx->max_ld, ctx->last_stream);
+  ctaux_status r = is_mixed(ctx) ? do_refresh<float>(ctx, -1, ctx->last_stream)
+                                 : do_refresh<double>(ctx, -1, ctx->last_stream);
   if (r != CTAUX_OK) return r;
   ctx->blocks_since_refresh = 0;
   r = ctaux_synchronize(ctx);
@@ -1057,8 +1132,9 @@ ctaux_status ctaux_set_config(ctaux_ctx* ctx, int chain, const double* tau, cons
   int sg = 1;
   d.sign = sg;
   CUDA_TRY(ctx, cudaMemcpy(dyn_of(ctx, chain), &d, sizeof(Dyn), cudaMemcpyHostToDevice));
-  ctaux_status r = is_mixed(ctx) ? do_refresh<float>(ctx, chain, n, ctx->last_stream)
-                                 : do_refresh<double>(ctx, chain, n, ctx->last_stream);
+  note_order(ctx, chain, n);
+  ctaux_status r = is_mixed(ctx) ? do_refresh<float>(ctx, chain, ctx->last_stream)
+                                 : do_refresh<double>(ctx, chain, ctx->last_stream);
   if (r != CTAUX_OK) return r;
   // the drift of this refresh compares N of the previous configuration with the
   // new one: it is not a drift of the chain
@@ -1438,6 +1514,7 @@ void ctaux_destroy(ctaux_ctx* ctx) {
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
   for (void* p : ctx->allocations) cudaFree(p);
+  if (ctx->seen) cudaFreeHost(ctx->seen);
   if (ctx->timer) {
     if (ctx->timer->created)
       for (int i = 0; i < PhaseTimer::kPool; ++i) cudaEventDestroy(ctx->timer->ev[i]);

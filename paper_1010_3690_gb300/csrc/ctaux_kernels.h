@@ -235,9 +235,17 @@ template <typename T>
 int launch_measure_head(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st);
 template <typename T>
 int launch_measure_tail(Chain<T>* dchains, const LaunchShape& ls, cudaStream_t st);
+// What a recomputation is launched for: no chain's order is above `bound` (a chain for
+// which that does not hold stops with DS_NUMERIC); `number` and each chain's order go to
+// `seen` (mapped host memory) when it begins, unless null.
+struct RefreshOrders {
+  int bound;
+  uint32_t number;
+  unsigned long long* seen;
+};
 template <typename T>
-cudaError_t launch_refresh(Chain<T>* dchains, const LaunchShape& ls, int only_chain, int max_order,
-                           cudaStream_t st, PhaseTimer* pt);   // max_order: no chain's order is above it
+cudaError_t launch_refresh(Chain<T>* dchains, const LaunchShape& ls, int only_chain, const RefreshOrders& ro,
+                           cudaStream_t st, PhaseTimer* pt);
 // scratch: each chain's refresh work area (both spins)
 cudaError_t launch_tie_refine(Chain<float>* dchains, const LaunchShape& ls, cudaStream_t st);
 template <typename T>

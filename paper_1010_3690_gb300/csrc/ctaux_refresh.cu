@@ -18,12 +18,17 @@ struct InvWidths {
 };
 template <typename T>
 __global__ void k_refresh_orders(const Chain<T>* chains, int n_chains, int only_chain, int* orders,
-                                 const InvView* views, InvWidths widths) {
+                                 const InvView* views, InvWidths widths, RefreshOrders ro) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 2 * n_chains) return;
   const int ci = i >> 1;
-  const Dyn& d = *chains[ci].dyn;
-  const bool take = (only_chain < 0 || only_chain == ci) && !(d.status & ~DS_SINGULAR);
+  Dyn& d = *chains[ci].dyn;
+  bool take = (only_chain < 0 || only_chain == ci) && !(d.status & ~DS_SINGULAR);
+  if (take && d.n > ro.bound) {
+    atomicOr(&d.status, DS_NUMERIC);
+    take = false;
+  }
+  if (ro.seen && !(i & 1)) ro.seen[ci] = ((unsigned long long)ro.number << 32) | (unsigned)d.n;
   orders[i] = take ? d.n : 0;
   for (int s = 0; s < widths.count; ++s)
     orders[(size_t)(1 + s) * 2 * n_chains + i] = take && views[i].width == widths.w[s] ? d.n : 0;
@@ -141,14 +146,16 @@ __global__ void __launch_bounds__(256) k_refresh_finish(const Chain<T>* chains, 
 }  // namespace
 
 template <typename T>
-cudaError_t launch_refresh(Chain<T>* dchains, const LaunchShape& ls, int only_chain, int max_order,
+cudaError_t launch_refresh(Chain<T>* dchains, const LaunchShape& ls, int only_chain, const RefreshOrders& ro,
                            cudaStream_t st, PhaseTimer* pt) {
   pt->begin(6, st);
+  const int max_order = ro.bound;
   const int items = 2 * ls.n_chains, nch = ls.n_chains;
   InvWidths widths{};
   if (only_chain < 0 && ls.inv_all.size() > 1)
     for (const InvShape& sh : ls.inv_all) widths.w[widths.count++] = sh.set.width;
-  k_refresh_orders<T><<<(items + 127) / 128, 128, 0, st>>>(dchains, nch, only_chain, ls.inv_orders, ls.inv_views, widths);
+  k_refresh_orders<T><<<(items + 127) / 128, 128, 0, st>>>(dchains, nch, only_chain, ls.inv_orders, ls.inv_views, widths,
+                                                        ro);
   // one chain: only its two matrices
   const int first = only_chain >= 0 ? 2 * only_chain : 0, count = only_chain >= 0 ? 2 : items;
   const InvView* views = ls.inv_views + first;
@@ -172,10 +179,10 @@ cudaError_t launch_refresh(Chain<T>* dchains, const LaunchShape& ls, int only_ch
   return e;
 }
 
-template cudaError_t launch_refresh<double>(Chain<double>*, const LaunchShape&, int, int, cudaStream_t,
-                                            PhaseTimer*);
-template cudaError_t launch_refresh<float>(Chain<float>*, const LaunchShape&, int, int, cudaStream_t,
-                                           PhaseTimer*);
+template cudaError_t launch_refresh<double>(Chain<double>*, const LaunchShape&, int, const RefreshOrders&,
+                                            cudaStream_t, PhaseTimer*);
+template cudaError_t launch_refresh<float>(Chain<float>*, const LaunchShape&, int, const RefreshOrders&,
+                                           cudaStream_t, PhaseTimer*);
 size_t refresh_work_doubles(int ld) { return 2 * refresh_work_per_spin(ld); }
 size_t refresh_work_one(int ld) { return refresh_work_per_spin(ld); }
 
