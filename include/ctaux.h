@@ -21,7 +21,11 @@
  *     arrays are copied before the call returns; the caller keeps ownership.
  *     Output arrays are caller-owned and written synchronously.
  *   - The library allocates all device memory it needs in ctaux_init
- *     (cudaMalloc) and frees it in ctaux_destroy.
+ *     (cudaMalloc) and frees it in ctaux_destroy.  The FP64 products on the
+ *     tensor cores (capacity + k_max of 256 and more) use up to 8 GB for
+ *     images of N, less where little is free: the results are the same.  Only
+ *     where not one image fits do they run on the float64 pipe, with other
+ *     roundings; ctaux_last_error() then says so after ctaux_init.
  *   - Errors are returned as ctaux_status; nothing aborts or traps.  A device
  *     side fault flag (capacity exceeded, non-finite ratio) is reported by the
  *     next synchronous call; ctaux_last_error() gives a text for the last

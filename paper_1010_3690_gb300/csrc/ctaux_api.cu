@@ -122,9 +122,11 @@ template <>
 std::vector<Chain<float>>& host_chains<float>(ctaux_ctx* ctx) { return ctx->hc32; }
 
 // Buffers and work list of the sliced prep and flush products (float64 form)
-// for the chains whose capacity calls for them, in one allocation made last.
-// They are an option: where they would take more than a quarter of the memory
-// that is left, the products stay on the float64 pipe.
+// for the chains whose capacity calls for them, in one allocation made last.  The
+// images of N, most of it, are made in strips of several products: fewer where they
+// would not fit in kSlicedPool or the whole in a quarter of the memory that is left,
+// down to one at a time.  That costs launches, not bits.  Only where not even that
+// leaves kSlicedReserve free do the products stay on the float64 pipe.
 ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
   LaunchShape& ls = ctx->ls;
   const int nch = (int)hc.size();
@@ -137,7 +139,6 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
   std::vector<SlicedView> views(2 * nch);
   std::vector<SlicedJob> jobs;
   std::vector<std::vector<size_t>> offs(2 * nch);
-  size_t img = 0, exps = 0, pool = 0, pool_exp = 0;
   for (int ci = 0; ci < nch; ++ci) {
     const Chain<double>& c = hc[ci];
     if (c.cap_m < kSlicedMinOrder) continue;
@@ -165,31 +166,37 @@ ctaux_status build_sliced(ctaux_ctx* ctx, std::vector<Chain<double>>& hc) {
       }
       views[2 * ci + spin].pl = (int)pl;
       views[2 * ci + spin].yc = (int)yc;
-      for (int pr = 0; pr < 2; ++pr) {
-        const size_t ib = pl * pl * 4 * kSlicedImageA;
-        if (ctx->strips.empty() || img + ib > kSlicedPool) {   // a new strip
-          ctx->strips.push_back(SlicedStrip{(int)jobs.size(), 0});
-          img = exps = 0;
-        }
-        jobs.push_back(SlicedJob{ci, spin, pr, 0, img, exps});
-        ctx->strips.back().count += 1;
-        img += ib;
-        exps += rows * pl;
-        pool = std::max(pool, img);
-        pool_exp = std::max(pool_exp, exps);
-      }
+      for (int pr = 0; pr < 2; ++pr) jobs.push_back(SlicedJob{ci, spin, pr, 0, 0, 0});
     }
   }
   ls.any_sliced = ls.any_sliced_y = ls.any_sliced_new = 0;
   ls.any_plain = ls.any_plain_y = ls.any_plain_new = 1;
   if (jobs.empty()) return CTAUX_OK;
-  const size_t o_views = take(views.size() * sizeof(SlicedView)), o_jobs = take(jobs.size() * sizeof(SlicedJob)),
-               o_exp = take(pool_exp * sizeof(int)), o_pool = take(pool);
+  const size_t o_views = take(views.size() * sizeof(SlicedView)), o_jobs = take(jobs.size() * sizeof(SlicedJob));
   size_t free_b = 0, total_b = 0;
   CUDA_TRY(ctx, cudaMemGetInfo(&free_b, &total_b));
+  const size_t room = free_b / 4 > at ? std::min(kSlicedPool, free_b / 4 - at) : 0;
+  size_t img = 0, exps = 0, pool = 0, pool_exp = 0;
+  for (size_t i = 0; i < jobs.size(); ++i) {
+    const size_t pl = views[2 * jobs[i].ci].pl, ib = pl * pl * 4 * kSlicedImageA;
+    if (i == 0 || img + ib > room) {   // a new strip
+      ctx->strips.push_back(SlicedStrip{(int)i, 0});
+      img = exps = 0;
+    }
+    jobs[i].img = img;
+    jobs[i].exps = exps;
+    ctx->strips.back().count += 1;
+    img += ib;
+    exps += pl * 128 * pl;
+    pool = std::max(pool, img);
+    pool_exp = std::max(pool_exp, exps);
+  }
+  const size_t o_exp = take(pool_exp * sizeof(int)), o_pool = take(pool);
   void* mem = nullptr;
-  if (at > free_b / 4 || cudaMalloc(&mem, at) != cudaSuccess) {
+  if (at + kSlicedReserve > free_b || cudaMalloc(&mem, at) != cudaSuccess) {
     cudaGetLastError();
+    set_err(ctx, CTAUX_OK, "note: %zu MB for the sliced products do not fit in %zu MB; they stay on the float64 pipe",
+            at >> 20, free_b >> 20);
     return CTAUX_OK;
   }
   ctx->allocations.push_back(mem);

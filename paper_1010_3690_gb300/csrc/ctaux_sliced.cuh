@@ -89,7 +89,8 @@ constexpr int kSlicedNewMinK = 128;
 // Split of G_{new,new} = C G_{old,new} over its inner dimension: a part or two per
 // slice, since it has few tiles (at most eight per spin).
 __host__ __device__ inline int sliced_new_slices(int n) { return ((n + 127) / 128 + 1) / 2; }
-// Bytes of the strip pool, unless one job needs more.
-constexpr size_t kSlicedPool = (size_t)8 << 30;
+// Bytes of the strip pool, unless one job needs more; and what its allocation leaves
+// for the stacks of kernels, which are allocated when they are first launched.
+constexpr size_t kSlicedPool = (size_t)8 << 30, kSlicedReserve = (size_t)256 << 20;
 
 }  // namespace ctaux
