@@ -14,9 +14,11 @@
 // products); what is dropped is below 2^(ea + eb - 61) per element.  The eight
 // group sums are combined as one 64-bit integer S with
 //   <a, b> = S 2^(ea + eb - 56)
-// rounded once in its last place, so the result is closer to the exact product
-// than a chain of 32 float64 multiply-adds, whose roundings are relative to
-// the running sum.
+// rounded once in its last place.  That is below the rounding of a chain of 32 float64
+// multiply-adds, which is relative to the running sum, where the elements of a row (and
+// of a column of the other operand) are of one scale: an element 2^t below its row's
+// largest keeps 55 - t bits.  Where they are not, the caller balances the inner index by
+// powers of two first (ctaux_sliced.cu, ctaux_inverse.cu).
 //
 // Slice images: an operand block of R rows (128 for A, 64 for B) and 32 inner
 // elements is stored as 7 consecutive [R][32] float16 tiles (64-byte rows,

@@ -55,13 +55,11 @@ __host__ __device__ inline size_t refresh_work_per_spin(int ld) {
 
 // Whether a chain waits for the fallback (its N is then kept in float64 too),
 // and its order.
-template <typename T>
 __device__ __forceinline__ bool refresh_pending(const Dyn& d) {
   return !(d.status & ~DS_SINGULAR) && d.tie_pending == 1;
 }
-template <typename T>
-__device__ __forceinline__ int refresh_order(const Chain<T>& c) {
-  return refresh_pending<T>(*c.dyn) ? c.dyn->n : 0;
+__device__ __forceinline__ int refresh_order(const Chain<float>& c) {
+  return refresh_pending(*c.dyn) ? c.dyn->n : 0;
 }
 
 // Work of every stage is spread over the grid across all chains: "row units"
@@ -149,8 +147,7 @@ __device__ __forceinline__ void refresh_store_column(const Chain<T>& c, int spin
   }
 }
 
-template <typename T>
-__device__ void refresh_body(Chain<T>* chains, int n_chains) {
+__device__ __forceinline__ void refresh_body(Chain<float>* chains, int n_chains) {
   cg::grid_group grid = cg::this_grid();
   const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
   const int gthreads = gridDim.x * blockDim.x;
@@ -181,7 +178,7 @@ __device__ void refresh_body(Chain<T>* chains, int n_chains) {
   // CTA and unit); pivot key of column 0
   for (int u = blockIdx.x; u < tot_r; u += gridDim.x) {
     const RowUnit ru = row_unit(offr, n_chains, u);
-    const Chain<T>& c = chains[ru.ci];
+    const Chain<float>& c = chains[ru.ci];
     const int m = ru.m, spin = ru.spin, j = ru.i, buf = c.dyn->buf, ld = c.ld;
     double* X = (c.work + (size_t)spin * refresh_work_per_spin(ld));
     unsigned long long* keys = c.pkeys + (size_t)spin * ld;
@@ -205,7 +202,7 @@ __device__ void refresh_body(Chain<T>* chains, int n_chains) {
       const int k = u / tot_r;
       const RowUnit ru = row_unit(offr, n_chains, u - k * tot_r);
       if (c0 + k >= ru.m) continue;
-      const Chain<T>& c = chains[ru.ci];
+      const Chain<float>& c = chains[ru.ci];
       const int ld = c.ld;
       double* X = (c.work + (size_t)ru.spin * refresh_work_per_spin(ld));
       double* Pa = X + (size_t)ld * ld;
@@ -230,7 +227,7 @@ __device__ void refresh_body(Chain<T>* chains, int n_chains) {
           const int grp = u / tot_r;
           const RowUnit ru = row_unit(offr, n_chains, u - grp * tot_r);
           if (c0 + k < ru.m) {
-            const Chain<T>& c = chains[ru.ci];
+            const Chain<float>& c = chains[ru.ci];
             const int ld = c.ld, col = c0 + k, i = ru.i, spin = ru.spin;
             const int nkk = min(kPB, ru.m - c0);
             double* X = (c.work + (size_t)spin * refresh_work_per_spin(ld));
@@ -307,7 +304,7 @@ __device__ void refresh_body(Chain<T>* chains, int n_chains) {
       const int k = u % kPB;
       const RowUnit ru = row_unit(offr, n_chains, u / kPB);
       if (c0 >= ru.m) continue;
-      const Chain<T>& c = chains[ru.ci];
+      const Chain<float>& c = chains[ru.ci];
       const int ld = c.ld, j = ru.i;
       double* X = (c.work + (size_t)ru.spin * refresh_work_per_spin(ld));
       double* Rr = X + (size_t)ld * ld + (size_t)2 * kPB * ld;
@@ -321,7 +318,7 @@ __device__ void refresh_body(Chain<T>* chains, int n_chains) {
       const int ci = find_chain(offt, n_chains, u);
       const int m = (offr[ci + 1] - offr[ci]) >> 1;
       if (c0 >= m) continue;  // uniform over the CTA
-      const Chain<T>& c = chains[ci];
+      const Chain<float>& c = chains[ci];
       const int tb = (m + TB - 1) / TB, l = u - offt[ci];
       const int spin = l / (tb * tb), tile = l - spin * tb * tb;
       const int ld = c.ld, bw = min(kPB, m - c0), cn = c0 + bw;
@@ -379,14 +376,14 @@ __device__ void refresh_body(Chain<T>* chains, int n_chains) {
   // and column), replace it; clear the pivot keys and flags for the next refresh
   for (int u = blockIdx.x; u < tot_r; u += gridDim.x) {
     const RowUnit ru = row_unit(offr, n_chains, u);
-    const Chain<T>& c = chains[ru.ci];
+    const Chain<float>& c = chains[ru.ci];
     const double* X = c.work + (size_t)ru.spin * refresh_work_per_spin(c.ld);
     refresh_store_column(c, ru.spin, ru.i, ru.m, X, c.N64[ru.spin], red);
   }
   grid.sync();  // every column has read perm before the flags are cleared
   for (int u = gtid; u < tot_r; u += gthreads) {
     const RowUnit ru = row_unit(offr, n_chains, u);
-    const Chain<T>& c = chains[ru.ci];
+    const Chain<float>& c = chains[ru.ci];
     const int ld = c.ld;
     c.pkeys[(size_t)ru.spin * ld + ru.i] = 0ull;
     c.used[ru.spin * ld + ru.i] = 0;

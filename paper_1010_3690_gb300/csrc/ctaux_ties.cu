@@ -421,10 +421,10 @@ __global__ void __launch_bounds__(256) k_tie_refine(Chain<float>* chains, int n_
   if (!fail_s) return;
   // fallback for the chains still pending: from-scratch FP64 refresh keeping
   // the FP64 N (N64), its stats, then the decision from N64
-  refresh_body<float>(chains, n_chains);
+  refresh_body(chains, n_chains);
   grid.sync();
   for (int ci = gtid; ci < n_chains; ci += gthreads)
-    if (refresh_pending<float>(*chains[ci].dyn)) refresh_finish_one(chains[ci]);
+    if (refresh_pending(*chains[ci].dyn)) refresh_finish_one(chains[ci]);
   grid.sync();
   for (int ci = blockIdx.x; ci < n_chains; ci += gridDim.x) tie_eval_chain(chains[ci]);
 }
