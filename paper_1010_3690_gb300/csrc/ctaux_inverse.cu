@@ -32,7 +32,7 @@
 // (order 310: 773 -> 794 us).
 // N^{-1} = [e^V / (e^V - 1) - G0] (e^V - 1) has rows of one scale and goes without;
 // scaled columns cancel by themselves.
-// From leading dimension 1024 on (kInvTwoLevel), two levels: the rank-32 products of four panels stay
+// From order kInvTwoLevel on, two levels: the rank-32 products of four panels stay
 // inside 128 columns, the rest of the matrix follows with one rank-128 product
 // (k_inv_cols slices the 128 columns).  That reads and writes X, and runs the
 // float64 epilogue, once per 128 columns instead of four times.
@@ -381,30 +381,28 @@ k_inv_panel(const InvView* views, const int* orders, int c0, int width, int rows
 struct InvRange {
   int c0, width, j0, j1;
 };
-// The columns of matrix i, of order m, in the product of rank 32 with the panel from c0
+// The columns of a matrix of order m in the product of rank 32 with the panel from c0
 // on: all, or the panel's own 128 in two levels.
-__device__ __forceinline__ InvRange inv_range(const InvView* views, const InvSet& set, int i, int m, int c0) {
-  const bool two = set.mixed ? views[i].chunks > 1 : set.two_level;
+__device__ __forceinline__ InvRange inv_range(int m, int c0, int width) {
+  const bool two = m >= kInvTwoLevel;
   const int j0 = two ? c0 & ~127 : 0;
-  return InvRange{c0, set.width, j0, two ? min(m, j0 + 128) : m};
+  return InvRange{c0, width, j0, two ? min(m, j0 + 128) : m};
 }
-// Whether it takes part in the product of rank 128: not where no column lies outside.
-__device__ __forceinline__ bool inv_wide(const InvView* views, const InvSet& set, int i, int m, int c0) {
-  return m > c0 && m > 128 && (!set.mixed || views[i].chunks > 1);
-}
+// Whether it takes part in the product of rank 128.
+__device__ __forceinline__ bool inv_wide(int m, int c0) { return m > c0 && m >= kInvTwoLevel; }
 
 // The pivot rows of the panel, in the columns of the range, as slice images: a
 // warp per column, a lane per pivot row.  Rank 32: y_k, the column at pivot row k
 // just before step k, y_k = X[R_k][j] + sum_{l<k} L[k][l] y_l; the panel's own
 // column c0 + k starts from the unit vector e_k.
 template <bool BALANCE>
-__global__ void __launch_bounds__(256) k_inv_rows(const InvView* views, const int* orders, int items, InvSet set,
+__global__ void __launch_bounds__(256) k_inv_rows(const InvView* views, const int* orders, int items, int width,
                                                   int c0, bool wide) {
   __shared__ int off[2 * kMaxChains + 1];
   for (int i = threadIdx.x; i < items; i += blockDim.x) {
     const int m = orders[i];
-    const InvRange g = inv_range(views, set, i, m, c0);
-    off[i] = wide ? (inv_wide(views, set, i, m, c0) ? (m + 7) / 8 : 0) : m > c0 ? (g.j1 - g.j0 + 7) / 8 : 0;
+    const InvRange g = inv_range(m, c0, width);
+    off[i] = wide ? (inv_wide(m, c0) ? (m + 7) / 8 : 0) : m > c0 ? (g.j1 - g.j0 + 7) / 8 : 0;
   }
   __syncthreads();
   block_exclusive_scan(off, items);
@@ -413,7 +411,7 @@ __global__ void __launch_bounds__(256) k_inv_rows(const InvView* views, const in
     const int it = find_chain(off, items, u);
     const InvView& v = views[it];
     const int m = orders[it];
-    const InvRange g = wide ? InvRange{c0, 128, 0, m} : inv_range(views, set, it, m, c0);
+    const InvRange g = wide ? InvRange{c0, 128, 0, m} : inv_range(m, c0, width);
     const int bw = min(g.width, m - g.c0);
     const int j = g.j0 + (u - off[it]) * 8 + (threadIdx.x >> 5);
     const bool own = j >= g.c0 && j < g.c0 + bw;
@@ -467,13 +465,12 @@ __global__ void __launch_bounds__(256) k_inv_rows(const InvView* views, const in
 // The columns [c0, c0 + 128) of X as slice images, one exponent per row: a CTA
 // stages 16 rows in shared memory, a thread then writes a 16-byte chunk of
 // every slice of a row.
-__global__ void __launch_bounds__(256) k_inv_cols(const InvView* views, const int* orders, int items,
-                                                  InvSet set, int c0) {
+__global__ void __launch_bounds__(256) k_inv_cols(const InvView* views, const int* orders, int items, int c0) {
   __shared__ int off[2 * kMaxChains + 1];
   __shared__ double xs[128][17];
   __shared__ int mxs[16];
   for (int i = threadIdx.x; i < items; i += blockDim.x)
-    off[i] = inv_wide(views, set, i, orders[i], c0) ? (orders[i] + 15) / 16 : 0;
+    off[i] = inv_wide(orders[i], c0) ? (orders[i] + 15) / 16 : 0;
   __syncthreads();
   block_exclusive_scan(off, items);
   const int total = off[items], r = threadIdx.x & 15, ch = threadIdx.x >> 4;
@@ -529,27 +526,26 @@ struct UpdTile {
   int it, m, i0, j0;
 };
 template <bool WIDE>
-__device__ __forceinline__ UpdTile upd_tile(const int* off, const InvView* views, const int* orders, int items,
-                                            const InvSet& set, int w, int c0) {
+__device__ __forceinline__ UpdTile upd_tile(const int* off, const int* orders, int items, int w, int c0) {
   UpdTile t;
   t.it = find_chain(off, items, w);
   t.m = orders[t.it];
   const int tm = (t.m + 127) / 128, l = w - off[t.it];
   t.i0 = (l % tm) * 128;
-  t.j0 = (WIDE ? 0 : inv_range(views, set, t.it, t.m, c0).j0) + (l / tm) * 64;
+  t.j0 = (WIDE ? 0 : inv_range(t.m, c0, 0).j0) + (l / tm) * 64;
   return t;
 }
 
 // WIDE: rank 128 (up to four image pairs per tile), else rank 32.
 template <bool WIDE>
 __global__ void __launch_bounds__(kUpdThreads, 1)
-k_inv_update(const InvView* views, const int* orders, int items, InvSet set, int c0) {
+k_inv_update(const InvView* views, const int* orders, int items, int width, int c0) {
   using namespace tc;
   __shared__ int off[2 * kMaxChains + 1];
   for (int i = threadIdx.x; i < items; i += blockDim.x) {
     const int m = orders[i], tm = (m + 127) / 128;
-    const InvRange g = inv_range(views, set, i, m, c0);
-    off[i] = WIDE ? (inv_wide(views, set, i, m, c0) ? tm * ((m + 63) / 64) : 0)
+    const InvRange g = inv_range(m, c0, width);
+    off[i] = WIDE ? (inv_wide(m, c0) ? tm * ((m + 63) / 64) : 0)
                   : m > c0 ? tm * ((g.j1 - g.j0 + 63) / 64) : 0;
   }
   __syncthreads();
@@ -594,7 +590,7 @@ k_inv_update(const InvView* views, const int* orders, int items, InvSet set, int
 
   if (warp == 0 && lane == 0) {
     for (int w = blockIdx.x; w < total && !err_s; w += gridDim.x) {
-      const UpdTile t = upd_tile<WIDE>(off, views, orders, items, set, w, c0);
+      const UpdTile t = upd_tile<WIDE>(off, orders, items, w, c0);
       const InvView& v = views[t.it];
       const int nc = WIDE ? (min(128, t.m - c0) + oz::kK - 1) / oz::kK : 1;
       const unsigned char* sa = v.As + (size_t)(t.i0 >> 7) * v.chunks * oz::kImageA;
@@ -622,7 +618,7 @@ k_inv_update(const InvView* views, const int* orders, int items, InvSet set, int
     uint32_t q = 0, taken = 0;
     for (int w = blockIdx.x; w < total; w += gridDim.x, ++q) {
       if (__any_sync(0xffffffffu, err_s != 0)) break;
-      const UpdTile t = upd_tile<WIDE>(off, views, orders, items, set, w, c0);
+      const UpdTile t = upd_tile<WIDE>(off, orders, items, w, c0);
       const int nc = WIDE ? (min(128, t.m - c0) + oz::kK - 1) / oz::kK : 1;
       bool ok = __all_sync(0xffffffffu, q == 0 || mbar_wait(smem_u32(&accempty), (q - 1) & 1));
       for (int c = 0; c < nc && ok; ++c, ++taken) {
@@ -652,9 +648,9 @@ k_inv_update(const InvView* views, const int* orders, int items, InvSet set, int
     const int quarter = warp & 3, group = (warp - 2) >> 2;
     uint32_t q = 0;
     for (int w = blockIdx.x; w < total; w += gridDim.x, ++q) {
-      const UpdTile t = upd_tile<WIDE>(off, views, orders, items, set, w, c0);
+      const UpdTile t = upd_tile<WIDE>(off, orders, items, w, c0);
       const InvView& v = views[t.it];
-      const InvRange g = WIDE ? InvRange{c0, 128, 0, t.m} : inv_range(views, set, t.it, t.m, c0);
+      const InvRange g = WIDE ? InvRange{c0, 128, 0, t.m} : inv_range(t.m, c0, width);
       const int ld = v.ld, i = t.i0 + quarter * 32 + lane, jb = t.j0 + group * kUpdCols;
       const int cn = min(g.c0 + g.width, t.m), je = g.j1;
       const bool row_ok = i < t.m;
@@ -768,15 +764,11 @@ int inv_width(int ld, const InvDevice& dev) {
 std::vector<InvShape> inv_shapes(const std::vector<int>& lds, const InvDevice& dev) {
   std::vector<InvShape> out;
   for (int width = kMaxWidth; width >= 4; width /= 2) {
-    InvShape s{dev, InvSet{width, false, false}, false, {}};
+    InvShape s{dev, width, {}};
     int max_ld = 0;
     for (int ld : lds)
-      if (inv_width(ld, dev) == width) {
-        max_ld = ld > max_ld ? ld : max_ld;
-        (inv_chunks(ld) > 1 ? s.set.two_level : s.one_level) = true;
-      }
+      if (inv_width(ld, dev) == width && ld > max_ld) max_ld = ld;
     if (max_ld == 0) continue;
-    s.set.mixed = s.set.two_level && s.one_level;
     auto smem_of = [&](int cluster) { return panel_smem_bytes(width, (max_ld + cluster - 1) / cluster, dev.balance); };
     for (int c0 = 0; c0 < max_ld; c0 += width) {
       int active = 0;
@@ -793,21 +785,21 @@ std::vector<InvShape> inv_shapes(const std::vector<int>& lds, const InvDevice& d
 int launch_inverse(const InvView* views, const int* orders, int items, int max_order,
                    const InvShape& sh, cudaStream_t st, cudaError_t* err) {
   int n = 0;
-  const int reach = (int)sh.panels.size() * sh.set.width;   // no order of this set is above it
+  const int reach = (int)sh.panels.size() * sh.width;   // no order of this set is above it
   max_order = max_order < reach ? max_order : reach;
   auto grid = [&](long units, long most) { return (int)(units < most ? units : most); };
   const long rb = (max_order + 127) / 128, sms = sh.dev.sm_count;
   // the product of the panel from c0 on with up to `cols` columns of a matrix
   auto update = [&](int c0, bool wide, long cols) {
     auto* rows = sh.dev.balance ? k_inv_rows<true> : k_inv_rows<false>;
-    rows<<<grid(items * ((cols + 7) / 8), 8 * sms), 256, 0, st>>>(views, orders, items, sh.set, c0, wide);
+    rows<<<grid(items * ((cols + 7) / 8), 8 * sms), 256, 0, st>>>(views, orders, items, sh.width, c0, wide);
     const int ug = grid(items * rb * ((cols + 63) / 64), sms);
-    if (wide) k_inv_update<true><<<ug, kUpdThreads, upd_smem(), st>>>(views, orders, items, sh.set, c0);
-    else k_inv_update<false><<<ug, kUpdThreads, upd_smem(), st>>>(views, orders, items, sh.set, c0);
+    if (wide) k_inv_update<true><<<ug, kUpdThreads, upd_smem(), st>>>(views, orders, items, sh.width, c0);
+    else k_inv_update<false><<<ug, kUpdThreads, upd_smem(), st>>>(views, orders, items, sh.width, c0);
     n += 2;
   };
-  for (int c0 = 0; c0 < max_order; c0 += sh.set.width) {
-    const InvPanel& pn = sh.panels[c0 / sh.set.width];
+  for (int c0 = 0; c0 < max_order; c0 += sh.width) {
+    const InvPanel& pn = sh.panels[c0 / sh.width];
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(items * pn.cluster));
     cfg.blockDim = dim3((unsigned)pn.threads);
@@ -821,17 +813,17 @@ int launch_inverse(const InvView* views, const int* orders, int items, int max_o
     cfg.numAttrs = 1;
     auto* fn = pn.threads == 512 ? (sh.dev.balance ? k_inv_panel<512, true> : k_inv_panel<512, false>)
                                  : (sh.dev.balance ? k_inv_panel<256, true> : k_inv_panel<256, false>);
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, views, orders, c0, sh.set.width, pn.rows);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, views, orders, c0, sh.width, pn.rows);
     n += 1;
     if (e != cudaSuccess) {
       *err = e;
       return n;
     }
-    const int o0 = c0 / 128 * 128, next = c0 + sh.set.width;
-    update(c0, false, sh.one_level ? max_order : max_order - o0 < 128 ? max_order - o0 : 128);
-    // the rank-128 product, unless no column lies outside the panel
-    if (sh.set.two_level && max_order > 128 && (next % 128 == 0 || next >= max_order)) {
-      k_inv_cols<<<grid(items * ((max_order + 15) / 16), 8 * sms), 256, 0, st>>>(views, orders, items, sh.set, o0);
+    const int o0 = c0 / 128 * 128, next = c0 + sh.width;
+    // (some order may be below the line also where the largest is above it)
+    update(c0, false, max_order < kInvTwoLevel ? max_order : kInvTwoLevel);
+    if (max_order >= kInvTwoLevel && (next % 128 == 0 || next >= max_order)) {
+      k_inv_cols<<<grid(items * ((max_order + 15) / 16), 8 * sms), 256, 0, st>>>(views, orders, items, o0);
       n += 1;
       update(o0, true, max_order);
     }

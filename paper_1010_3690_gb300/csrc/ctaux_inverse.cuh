@@ -13,7 +13,7 @@ namespace ctaux {
 struct InvView {
   double* X;            // the matrix, column-major, leading dimension ld
   int ld;
-  int chunks;           // images per row block: 1, or 4 (panels of 128 columns in two levels)
+  int chunks;           // images per row block that there is room for: 1, or 4 (two levels)
   int width;            // panel width
   unsigned char* As;    // slice images of the panel's columns: ceil(ld / 128) x chunks x oz::kImageA
   unsigned char* Bs;    // slice images of the pivot rows: ceil(ld / 64) x chunks x oz::kImageB
@@ -29,17 +29,17 @@ struct InvView {
   int* status;          // DS_SINGULAR and DS_TIMEOUT bits
 };
 
-// Panels of 128 columns in two levels (see ctaux_inverse.cu) for matrices whose
-// leading dimension is at least this, whatever else is in the launch (a chain gives
-// the same bits alone or in a batch): the five extra launches per 128 columns against
-// three of four passes over the matrix.  One level against two, ms per recomputation
-// of one chain: 2.29 / 2.49 at order 700, 3.19 / 3.29 at 900, 4.44 / 4.46 at 1100, 6.51
-// / 6.23 at 1500, 10.9 / 9.6 at 2000 (leading dimensions a quarter above the order).
-// In a batch the passes cost more and the launches less: 96 chains up to order 1084,
-// 8 blocks with one recomputation, 32.9 ms with the line at 1408, 31.7 at 1024, 31.6
-// at 512, where one chain of order 431 takes a tenth longer.
-constexpr int kInvTwoLevel = 1024;
-inline int inv_chunks(int ld) { return ld >= kInvTwoLevel ? 4 : 1; }
+// Panels of 128 columns in two levels (see ctaux_inverse.cu) for matrices of this order
+// on, whatever else is in the launch (a chain gives the same bits alone or in a batch):
+// the five extra launches per 128 columns against three of four passes over the matrix.
+// One level against two, ms per recomputation of one chain: 2.29 / 2.49 at order 700,
+// 3.19 / 3.29 at 900, 4.44 / 4.46 at 1100, 6.51 / 6.23 at 1500, 10.9 / 9.6 at 2000.  In a
+// batch the passes cost more and the launches less: 96 chains of order 58 to 1084, 8
+// blocks with one recomputation, 33.7 ms with the line at 1060, 32.2 at 768, 32.7 at 512
+// (31.1 with all of them in two levels, where one chain of order 431 alone takes a tenth
+// longer).
+constexpr int kInvTwoLevel = 768;
+inline int inv_chunks(int ld) { return ld >= kInvTwoLevel ? 4 : 1; }   // images, at the largest order
 
 // Doubles of As, Bs, ea, eb and piv for a leading dimension (the matrix itself
 // comes first and takes ld^2 doubles).
@@ -87,16 +87,9 @@ struct InvPanel {
   int rows;        // panel rows per CTA at the largest leading dimension
   int smem;        // dynamic shared memory
 };
-// What the matrices of a launch have in common: the panel width, and whether they go in
-// one level or two (mixed: each matrix says so itself).
-struct InvSet {
-  int width;
-  bool two_level, mixed;
-};
 struct InvShape {
   InvDevice dev;
-  InvSet set;
-  bool one_level;                // some matrix has one level
+  int width;                     // panel width
   std::vector<InvPanel> panels;  // of each panel: fewer matrices reach the later ones
 };
 // lds: the leading dimension of every matrix.  One shape for each panel width among them,

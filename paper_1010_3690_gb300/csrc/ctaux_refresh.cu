@@ -153,7 +153,7 @@ cudaError_t launch_refresh(Chain<T>* dchains, const LaunchShape& ls, int only_ch
   const int items = 2 * ls.n_chains, nch = ls.n_chains;
   InvWidths widths{};
   if (only_chain < 0 && ls.inv_all.size() > 1)
-    for (const InvShape& sh : ls.inv_all) widths.w[widths.count++] = sh.set.width;
+    for (const InvShape& sh : ls.inv_all) widths.w[widths.count++] = sh.width;
   k_refresh_orders<T><<<(items + 127) / 128, 128, 0, st>>>(dchains, nch, only_chain, ls.inv_orders, ls.inv_views, widths,
                                                         ro);
   // one chain: only its two matrices

@@ -11,11 +11,11 @@ pytestmark = pytest.mark.gpu
 pk = pytest.importorskip("paper_1010_3690_gb300")
 
 
-@pytest.mark.parametrize("sizes", [((300, 400), (900, 1500)), ((500, 960), (500, 961), (40, 64)),
+@pytest.mark.parametrize("sizes", [((300, 400), (900, 1500)), ((767, 1000), (768, 1000), (40, 64)),
                                    ((60, 200), (150, 13000))])
 def test_recomputation_in_a_mixed_set_gives_the_bits_of_the_chain_alone(sizes):
-    """(order, capacity) on both sides of the line between panels in one and two levels,
-    and of the one between panels of 32 and 16 columns."""
+    """(order, capacity) on both sides of the line between panels in one and two levels
+    (order 768), and of the one between panels of 32 and 16 columns."""
     chains = [configs.cube8(K=256.0, k_max=32, capacity=cap) for _, cap in sizes]
     chains = [dataclasses.replace(c, chain_id=i) for i, c in enumerate(chains)]
     cfgs = [configs.synthetic_configuration(c, n, seed=9 + i) for i, (c, (n, _)) in enumerate(zip(chains, sizes))]
