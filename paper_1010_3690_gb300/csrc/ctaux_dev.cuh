@@ -317,6 +317,12 @@ __device__ __forceinline__ A g_int(const Chain<T>& c, const T* Nb, const T* Gc, 
   return (A)Gc[(long)(j - n_old) * c.ld + i];
 }
 
+// A wait gave up: the CTA may leave items of any chain of its launch undone.
+template <typename T>
+__device__ __noinline__ void stop_chains(Chain<T>* chains, int n_chains) {
+  for (int i = 0; i < n_chains; ++i) atomicOr(&chains[i].dyn->status, DS_TIMEOUT);
+}
+
 // ------------------------------------------------------------ work lists
 // Batched kernels loop over (chain, item) pairs: every CTA computes each
 // chain's item count from its device-side sizes, an exclusive prefix sum in

@@ -29,8 +29,9 @@
 //     epilogue of one tile overlaps the loads and MMAs of the next.
 // Every mbarrier wait is bounded: the pipeline roles poll at most `wl` times
 // (a launch argument, 2^24 unless the context sets a smaller limit), the
-// final drains always 2^24 times.  On timeout the chain's status gets
-// DS_TIMEOUT (CTAUX_ETIMEOUT) and every role stops; before the CTA exits, the
+// final drains always 2^24 times.  On timeout the status of every chain gets
+// DS_TIMEOUT (CTAUX_ETIMEOUT; the CTA may leave tiles of any of them undone) and
+// every role stops; before the CTA exits, the
 // copies issued are waited for, the MMA thread waits for its MMAs, and the
 // TMEM is freed.  With `stall` set (a test of this path) the MMA issuer first
 // waits on a barrier that nothing completes, so every launch times out.
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_flush_tc(Chain<float>* chains
         const uint32_t stage = issued % kTcStages, use = issued / kTcStages;
         if (use > 0 && !mbar_wait(smem_u32(empty + stage), (use - 1) & 1, wl)) {
           *err_s = 1;
-          atomicOr(&chains[t.ci].dyn->status, DS_TIMEOUT);
+          stop_chains(chains, n_chains);
           break;
         }
         const uint32_t fb = smem_u32(full + stage);
@@ -201,7 +202,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_flush_tc(Chain<float>* chains
     if (stall && !mbar_wait(smem_u32(never), 0, wl)) {
       // test of the bounded waits: a barrier that nothing completes
       *err_s = 1;
-      atomicOr(&chains[find_chain(off, n_chains, blockIdx.x)].dyn->status, DS_TIMEOUT);
+      stop_chains(chains, n_chains);
     }
     for (int w = blockIdx.x; w < total && !*err_s; w += gridDim.x) {
       const TcItem t = tc_item(chains, off, n_chains, w);
@@ -232,7 +233,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_flush_tc(Chain<float>* chains
       }
       if (!ok) {
         *err_s = 1;
-        atomicOr(&chains[t.ci].dyn->status, DS_TIMEOUT);
+        stop_chains(chains, n_chains);
         break;
       }
       mma_commit(smem_u32(accfull + b));
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_flush_tc(Chain<float>* chains
       if (nq > 0 && !__all_sync(0xffffffffu, mbar_wait(smem_u32(nsempty), (nq - 1) & 1, wl))) {
         if (lane == 0) {
           *err_s = 1;
-          atomicOr(&c.dyn->status, DS_TIMEOUT);
+          stop_chains(chains, n_chains);
         }
         break;
       }
@@ -309,7 +310,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_flush_tc(Chain<float>* chains
       if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(nsfull), nq & 1, wl))) {
         if (lane == 0) {
           *err_s = 1;
-          atomicOr(&c.dyn->status, DS_TIMEOUT);
+          stop_chains(chains, n_chains);
         }
         break;
       }
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_flush_tc(Chain<float>* chains
       if (!ok) {
         if (lane == 0) {
           *err_s = 1;
-          atomicOr(&c.dyn->status, DS_TIMEOUT);
+          stop_chains(chains, n_chains);
         }
         break;
       }

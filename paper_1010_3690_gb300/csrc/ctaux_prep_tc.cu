@@ -29,7 +29,7 @@
 //   warps 8-11: epilogue, TMEM lane quarter w % 4, all 128 columns: adds each
 //     segment's partial tile to the float32 tile accumulator in shared memory
 //     and writes the tile after the last segment.
-// Every mbarrier wait is bounded; on timeout the chain's status gets
+// Every mbarrier wait is bounded; on timeout the status of every chain gets
 // DS_TIMEOUT and every role stops, the copies issued are drained, the MMA
 // thread waits for its MMAs and the TMEM is freed.
 #include <cuda.h>
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) k_prep_tc(Chain<float>* chain
       }
       if (!ok) {
         *err_s = 1;
-        atomicOr(&chains[t.ci].dyn->status, DS_TIMEOUT);
+        stop_chains(chains, n_chains);
         break;
       }
     }
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) k_prep_tc(Chain<float>* chain
       if (!ok) {
         if (lane == 0) {
           *err_s = 1;
-          atomicOr(&chains[t.ci].dyn->status, DS_TIMEOUT);
+          stop_chains(chains, n_chains);
         }
         break;
       }
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) k_prep_tc(Chain<float>* chain
         }
         if (!ok) {
           *err_s = 1;
-          atomicOr(&chains[t.ci].dyn->status, DS_TIMEOUT);
+          stop_chains(chains, n_chains);
           break;
         }
         mma_commit(smem_u32(accfull + b));
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) k_prep_tc(Chain<float>* chain
       if (!ok) {
         if (lane == 0) {
           *err_s = 1;
-          atomicOr(&c.dyn->status, DS_TIMEOUT);
+          stop_chains(chains, n_chains);
         }
         break;
       }

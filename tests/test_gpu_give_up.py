@@ -65,3 +65,12 @@ def test_chains_recover_from_a_product_that_gave_up(k, n_chains):
             assert len(tr) == len(clean[i])
             for name in tr.dtype.names:
                 np.testing.assert_array_equal(tr[name], clean[i][name])
+
+
+def test_every_chain_of_a_mixed_flush_that_gave_up_reports_it():
+    """The same for the tensor-core flush of the mixed form, whose test setting stalls
+    every CTA: chains that no CTA begins with stop as well."""
+    chains, cfgs = _chains(64, 24)
+    with pk.Context(chains, precision=pk.CTAUX_MIXED, refresh_every=0, tc_wait_limit=-2000) as ctx:
+        _give_up(ctx, cfgs)
+        assert all(ctx.stats(i)["status"] & 8 for i in range(24))
