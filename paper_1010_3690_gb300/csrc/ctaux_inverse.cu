@@ -719,12 +719,6 @@ int panel_smem_bytes(int width, int rows, bool balance) {
 
 }  // namespace
 
-// Cluster size per panel, from the matrices that can still reach it: 16 CTAs for
-// a few (a GPC holds one such cluster; order 431 alone: 1.23 ms, against 1.35 with
-// 8 and 1.48 with 4; order 2000: 8.3, 9.8, 13.2), 8 in batches (192 matrices of up
-// to order 1084: 13.0 ms, 14.3 with 4; larger clusters pay where a batch's last,
-// largest matrices are left), 4 beyond 256 matrices, whose rows fill the float64
-// pipes of all SMs anyway.
 cudaError_t inv_device(int sm_count, bool balance, InvDevice* out) {
   *out = InvDevice{sm_count, 16, balance};
   auto attrs = [&](auto* fn, int bytes) {
@@ -761,6 +755,12 @@ int inv_width(int ld, const InvDevice& dev) {
   return width;
 }
 
+// Cluster size per panel, from the matrices that can still reach it: 16 CTAs for
+// a few (a GPC holds one such cluster; order 431 alone: 1.23 ms, against 1.35 with
+// 8 and 1.48 with 4; order 2000: 8.3, 9.8, 13.2), 8 in batches (192 matrices of up
+// to order 1084: 13.0 ms, 14.3 with 4; larger clusters pay where a batch's last,
+// largest matrices are left), 4 beyond 256 matrices, whose rows fill the float64
+// pipes of all SMs anyway.
 std::vector<InvShape> inv_shapes(const std::vector<int>& lds, const InvDevice& dev) {
   std::vector<InvShape> out;
   for (int width = kMaxWidth; width >= 4; width /= 2) {

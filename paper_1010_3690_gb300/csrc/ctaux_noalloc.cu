@@ -25,6 +25,7 @@ constexpr size_t kPerm = kWork, kPcol = kPerm + kM * sizeof(int), kUsed = kPcol 
                  kColExp = kView + (sizeof(InvView) + 15) / 16 * 16, kRowExp = kColExp + kM * sizeof(int),
                  kEnd = kRowExp + kM * sizeof(int);
 static_assert(kEnd <= CTAUX_NOALLOC_SCRATCH_BYTES, "scratch size in the header");
+static_assert(kM < kInvTwoLevel, "one level: one image per row block, and the balance");
 
 // Shared by every call on a device; held by each device that loads the library.
 static __device__ __align__(1024) unsigned char g_noalloc_scratch[CTAUX_NOALLOC_SCRATCH_BYTES];
